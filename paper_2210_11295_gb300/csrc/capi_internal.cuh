@@ -19,6 +19,11 @@ bsrht_opts opts_or_default(const bsrht_opts* o);
 // that precision on 16-bit data, EINVAL for an unknown precision.
 int plan_dtype(const bsrht_opts& o, int* dt);
 
+// Scratch of bsrht_rsvd / bsrht_nystrom: the size that gives every product
+// its fastest form, or (lean) the smallest the call accepts.
+int rsvd_scratch(const bsrht_opts& o, int64_t n, int64_t m, int k, int64_t l, int p, bool lean, size_t* bytes);
+int nystrom_scratch(const bsrht_opts& o, int64_t n, int k, int64_t l, int p, bool lean, size_t* bytes);
+
 // BSRHT_OK for calls without an FP64-arithmetic form on FP32 storage when
 // opts asks for none (precision AUTO, or F64 on FP64 data).
 int precision_auto_only(const bsrht_opts& o);

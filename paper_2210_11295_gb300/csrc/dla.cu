@@ -141,6 +141,14 @@ int gemm(const Dla& d, Arena& ar, DT ta, DT tb, DT tc, bool acc64, int64_t M, in
   if (M <= 0 || N <= 0) return BSRHT_OK;
   if ((gram) && beta != 0.0) return BSRHT_EINVAL;
   if (acc64) {
+    if (ta == DT::F64 && tb == DT::F64 && tc == DT::F64 && alpha == 1.0 && beta == 0.0 &&
+        !(ar.measure && ar.lean) && (ar.measure || d.status) && gemm_int8x7_wants(M, N, K)) {
+      const size_t mk = ar.mark();
+      const int st = gemm_int8x7(d, ar, M, N, K, static_cast<const double*>(A), lda, a_trans,
+                                 static_cast<const double*>(B), ldb, static_cast<double*>(C), ldc, tri_b, gram);
+      if (!ar.measure && st != BSRHT_EUNSUP) return st;
+      ar.release(mk);  // size (or run) the CUDA-core form as well
+    }
     if (ta == DT::F64 && tb == DT::F64 && tc == DT::F64)
       return gemm_launch<double, double, double, double, 4>(d, ar, M, N, K, A, lda, a_trans, B, ldb, C, ldc,
                                                             alpha, beta, tri_b, gram);

@@ -21,6 +21,7 @@ struct Arena {
   char* base = nullptr;
   size_t cap = 0, used = 0, high = 0;
   bool measure = false;  // only count bytes (no pointers handed out)
+  bool lean = false;     // measuring: without the scratch of forms that a call can do without
   void* take(size_t bytes) {
     used = (used + 255) / 256 * 256;
     void* p = measure ? nullptr : base + used;
@@ -108,6 +109,27 @@ int gemm_tc(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const floa
             const void* B, int64_t ldb, bool b_kmajor, DT tc_out, void* C, int64_t ldc, bool gram,
             bool b_upper = false, float* Ct = nullptr);
 bool gemm_tc_eligible(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda);
+
+// Forms that need more scratch than the CUDA-core GEMM and leave it to that
+// one (BSRHT_EUNSUP, nothing enqueued) when the arena does not hold it
+// (gemm_slices.cuh).
+//
+// FP64 products on the 16-bit tensor cores in exact integer arithmetic:
+// C (M x N, ldc) = op(A) B as in gemm(), all FP64.  An entry of a row of
+// op(A) or of a column of B is taken to 2^-55 of the largest one there; sums
+// are exact and each split of K is rounded once, so an entry of C is off by
+// at most about K 2^-54 times the row's and the column's largest entries, a
+// normwise bound like that of the factorizations that use it.
+// gemm_int8x7_wants: large enough to gain.
+bool gemm_int8x7_wants(int64_t M, int64_t N, int64_t K);
+int gemm_int8x7(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const double* A, int64_t lda, bool a_trans,
+                const double* B, int64_t ldb, double* C, int64_t ldc, bool b_upper, bool gram);
+// FP32-accurate products of 16-bit data: C (M x N, FP32, ldc) = A (M x K,
+// BF16 or F16, 16-byte aligned rows) * B (K x N, FP32 or FP64, ldb); Ct as
+// in gemm_tc.
+bool gemm_a16_eligible(DT ta, int64_t M, int64_t N, int64_t K, const void* A, int64_t lda);
+int gemm_a16(const Dla& d, Arena& ar, DT ta, int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, DT tb,
+             const void* B, int64_t ldb, float* C, int64_t ldc, float* Ct);
 // Bt (N x ldk, FP32) = B^T for B K x N (FP32 or FP64, ldb); Bt[:, K:ldk] = 0.
 int transpose_to_f32(const Dla& d, DT tb, const void* B, int64_t K, int64_t N, int64_t ldb, float* Bt, int64_t ldk,
                      float* Blo = nullptr);

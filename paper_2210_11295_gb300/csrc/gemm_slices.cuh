@@ -1,0 +1,511 @@
+// Tensor-core products on operands held as 16-bit slices (tcgen05 kind::f16).
+//
+// Two kernels share the layout: K-major slices [slice][row][k] in global
+// memory, TMA into swizzled shared memory, one thread issuing the MMAs, FP32
+// accumulators in tensor memory, eight warps folding them.
+//
+// k_gemm_int8x7: FP64 products in exact integer arithmetic.  The FP64 units
+// of this GPU give about two FMAs per SM and clock (1.2 TFLOP/s on the whole
+// chip), the 16-bit tensor cores 4096.  Every row of A and every column of B
+// gets one power-of-two scale, under which an entry is an integer of 55 bits
+// and a sign, written as seven balanced base-256 digits d_0 .. d_6 (|d| <=
+// 128, exact in FP16).  A product of two digits is at most 2^14, so the FP32
+// accumulators add up to 7 x 128 of them (2^23.8) without rounding.  The
+// digit products of equal weight, i + j = c, share one accumulator; classes
+// c = 0 .. 6 are formed (28 of 49 products), the rest lies below 2^-55 of
+// the row's and the column's largest entries.  After every 128 columns of K the
+// seven accumulators are folded into two 64-bit integers per entry, and the
+// sum is rounded to FP64 once, at the end.
+//
+// k_gemm_a16: FP32-accurate products of 16-bit data.  A (BF16 or FP16) is
+// exact as it is stored and comes in by TMA straight into the MMA operand;
+// B (FP32 values) is split once into three slices of A's type (24 bits in
+// BF16, 33 in FP16), scaled per column to FP16's range.  Three 16-bit MMAs
+// per product; each K block of 64 starts a fresh accumulator, smallest slice
+// first, which the fold adds to FP32 registers, rounding to nearest (the
+// tensor core's own accumulation truncates).
+#pragma once
+
+#include <cuda.h>
+#include <stdint.h>
+
+#include "common.cuh"
+#include "tma.cuh"
+#include "tmem.cuh"
+
+namespace bsrht {
+namespace sl {
+
+constexpr int kDig = 7;               // digits of an FP64 operand
+constexpr int BM = 128;
+constexpr uint32_t kWaitSl = 1u << 24;  // bounded mbarrier waits
+constexpr int kErrSl = 8;             // status bit of a failed wait (kStatusTcWait)
+constexpr int kThreads = 64 + 256;    // warps 0: TMA, 1: MMA, 2..9: fold
+constexpr int kNonFiniteExp = 0x7FF;  // biased exponent of Inf / NaN
+
+// 3-D tiled TMA load of box {x, y, z} (x innermost).
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int32_t x, int32_t y,
+                                            int32_t z) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], "
+      "[%2];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z)
+      : "memory");
+}
+
+// K-major operand descriptors: rows of 128 bytes (128-byte swizzle, 8-row
+// atoms 1024 bytes apart) or 64 bytes (64-byte swizzle, 512 bytes apart).
+template <int ROW_BYTES>
+__device__ __forceinline__ uint64_t desc_k(uint32_t saddr) {
+  static_assert(ROW_BYTES == 128 || ROW_BYTES == 64, "swizzle span");
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)((8u * ROW_BYTES) >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)(ROW_BYTES == 128 ? 2 : 4) << 61;
+  return d;
+}
+
+// Instruction descriptor: D FP32, A and B FP16 (bf16: BF16), both K-major.
+__device__ __forceinline__ uint32_t idesc_f16(bool bf16, int n) {
+  const uint32_t t = bf16 ? 1u : 0u;
+  return (1u << 4) | (t << 7) | (t << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+}
+
+__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                        uint32_t accum) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
+          d_tmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
+      : "memory");
+}
+__device__ __forceinline__ void mma_commit(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+               : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// ------------------------------------------------------------ digit split
+// The 55-bit fixed-point value of the FP64 bits `raw` under the scale
+// exponent E (>= the biased exponent of every entry that shares it, E >= 1):
+// t = round(x 2^(55 - (E - 1022))), |t| < 2^55.  With u = t +
+// 0x0080808080808080 (0 <= u < 2^57) the balanced base-256 digits of t are
+// the bytes 0 .. 5 of u and its bits 48 .. 56, each less 128.
+__device__ __forceinline__ int64_t fixed55(uint64_t raw, int E) {
+  const uint32_t hi = (uint32_t)(raw >> 32);
+  const int e = (int)((hi >> 20) & 0x7FFu);
+  const uint64_t mant = (raw & 0x000FFFFFFFFFFFFFull) | ((uint64_t)(e != 0) << 52);
+  const int sh = (e ? e : 1) - E + 2;  // <= 2
+  uint64_t q;
+  if (sh >= 0) {
+    q = mant << sh;
+  } else {
+    const int r = min(-sh, 63);
+    q = (mant + (1ull << (r - 1))) >> r;  // half up: r <= 63, mant < 2^53
+  }
+  return (int64_t)raw < 0 ? -(int64_t)q : (int64_t)q;
+}
+__device__ __forceinline__ uint64_t digit_bytes(int64_t t) { return (uint64_t)t + 0x0080808080808080ull; }
+
+// Digit s (0 the highest) of the two values u0, u1 as an FP16 pair: a value b
+// <= 256 in the low mantissa bits under the exponent of 1024 is 1024 + b
+// exactly, and 1152 off it is the digit.
+__device__ __forceinline__ uint32_t digit_pair(uint64_t u0, uint64_t u1, int s) {
+  const uint32_t mask = s == 0 ? 0x1FFu : 0xFFu;
+  const uint32_t x0 = (uint32_t)(u0 >> (8 * (6 - s))) & mask, x1 = (uint32_t)(u1 >> (8 * (6 - s))) & mask;
+  const uint32_t v = x0 | (x1 << 16) | 0x64006400u;
+  const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&v), __floats2half2_rn(1152.f, 1152.f));
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// FP64 nearest to (h 2^32 + l) 2^x.
+__device__ __forceinline__ double scale_int(int64_t h, int64_t l, int x) {
+  uint64_t lo = ((uint64_t)h << 32) + (uint64_t)l;
+  int64_t hi = (h >> 32) + (l >> 63) + (lo < (uint64_t)l ? 1 : 0);
+  const bool neg = hi < 0;
+  uint64_t uh = (uint64_t)hi, ul = lo;
+  if (neg) {
+    ul = 0ull - ul;
+    uh = ~uh + (ul == 0 ? 1 : 0);
+  }
+  if ((uh | ul) == 0) return 0.0;
+  const int lz = uh ? __clzll((long long)uh) : 64 + __clzll((long long)ul);
+  uint64_t top;
+  bool sticky;
+  if (lz >= 64) {
+    top = ul << (lz - 64);
+    sticky = false;
+  } else {
+    top = lz ? (uh << lz) | (ul >> (64 - lz)) : uh;
+    sticky = lz < 64 && (ul << lz) != 0;
+  }
+  uint64_t m = top >> 11;
+  const uint32_t rem = (uint32_t)top & 0x7FFu;
+  m += (rem > 0x400u || (rem == 0x400u && (sticky || (m & 1)))) ? 1 : 0;
+  int e = x + (127 - lz) + 1023;  // biased exponent of the leading bit
+  if (m >> 53) {
+    m >>= 1;
+    ++e;
+  }
+  double v;
+  if (e >= 1 && e <= 2046)
+    v = __longlong_as_double((long long)((m & 0x000FFFFFFFFFFFFFull) | ((uint64_t)e << 52)));
+  else
+    v = ldexp((double)m, e - 1023 - 52);
+  return neg ? -v : v;
+}
+
+// ------------------------------------------------------- FP64 (7 digits)
+struct Int8x7 {
+  static constexpr int BN = 64, BK = 32, STAGES = 2;
+  static constexpr int KG = 4;  // stages (128 columns of K) between folds
+  static constexpr uint32_t A_SLICE = BM * BK * 2, B_SLICE = BN * BK * 2;
+  static constexpr uint32_t A_BYTES = kDig * A_SLICE, B_BYTES = kDig * B_SLICE;
+  static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
+  static constexpr size_t smem_bytes() { return 1024 + (size_t)STAGES * STAGE_BYTES + 256; }
+  static constexpr uint32_t TMEM_COLS = 512;  // 7 x 64 used
+  // Exact sums: 2^14 per product, at most 7 products a class, KG BK columns.
+  static_assert(kDig * KG * BK * (1 << 14) <= (1 << 24), "exact FP32 accumulation");
+  static_assert(A_SLICE % 1024 == 0 && B_SLICE % 1024 == 0, "swizzle atoms");
+};
+
+struct Int8x7Args {
+  int64_t M, N, K;
+  double* C;       // output, or partials [z][M][N] when `part`
+  int64_t ldc;
+  const int* ea;   // scale exponents of the rows of A and the columns of B
+  const int* eb;
+  int part, gram, b_upper;
+  int* err;
+};
+
+__host__ __device__ __forceinline__ bool int8x7_skipped(int64_t bm, int64_t bn) {
+  return bm * BM >= (bn + 1) * Int8x7::BN;
+}
+
+__global__ void __launch_bounds__(kThreads, 1)
+    k_gemm_int8x7(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, Int8x7Args g) {
+  using S = Int8x7;
+  constexpr int BN = S::BN, BK = S::BK, STAGES = S::STAGES, KG = S::KG;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* base = smem_raw + ((1024 - (reinterpret_cast<uintptr_t>(smem_raw) & 1023)) & 1023);
+  uint64_t* full = reinterpret_cast<uint64_t*>(base + STAGES * S::STAGE_BYTES);
+  uint64_t* empty = full + STAGES;
+  uint64_t* accf = empty + STAGES;     // [7] class finished
+  uint64_t* accfree = accf + kDig;     // [7] class folded
+  uint64_t* drain = accfree + kDig;    // every MMA issued has finished
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t tn = (g.N + BN - 1) / BN;
+  const int64_t bm = (int64_t)blockIdx.x / tn, bn = (int64_t)blockIdx.x - bm * tn;
+  const int64_t m0 = bm * BM, n0 = bn * BN;
+  if (g.gram && int8x7_skipped(bm, bn)) return;  // uniform: before any barrier
+  const int64_t kmax = g.b_upper ? (g.K < n0 + BN ? g.K : n0 + BN) : g.K;
+  // Split K in groups of KG stages, so that every fold but the last is full.
+  const int64_t ngr = (kmax + KG * BK - 1) / (KG * BK);
+  const int64_t g0 = ngr * blockIdx.z / gridDim.z, g1 = ngr * (blockIdx.z + 1) / gridDim.z;
+  const int64_t kb0 = g0 * KG;
+  const int64_t kb_end = (kmax + BK - 1) / BK < g1 * KG ? (kmax + BK - 1) / BK : g1 * KG;
+  const int nst = (int)(kb_end > kb0 ? kb_end - kb0 : 0);
+  const int ngroups = (nst + KG - 1) / KG;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int c = 0; c < kDig; ++c) {
+      mbar_init(&accf[c], 1);
+      mbar_init(&accfree[c], 8);
+    }
+    mbar_init(drain, 1);
+    fence_mbar_init();
+  }
+  if (warp == 0) tc::tmem_alloc(tmem_slot, S::TMEM_COLS);
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  bool failed = false;
+
+  if (warp == 0) {
+    if (lane == 0) {  // TMA producer
+      int issued = 0;
+      for (int st = 0; st < nst; ++st) {
+        const int s = st % STAGES, u = st / STAGES;
+        if (u > 0 && !mbar_wait_bounded(&empty[s], (uint32_t)((u - 1) & 1), kWaitSl)) {
+          failed = true;
+          break;
+        }
+        unsigned char* p = base + (size_t)s * S::STAGE_BYTES;
+        mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
+        const int32_t kx = (int32_t)((kb0 + st) * BK);
+        tma_load_3d(p, &mapA, &full[s], kx, (int32_t)m0, 0);
+        tma_load_3d(p + S::A_BYTES, &mapB, &full[s], kx, (int32_t)n0, 0);
+        issued = st + 1;
+      }
+      if (failed)  // shared memory must not be released under copies still landing
+        for (int st = (issued > STAGES ? issued - STAGES : 0); st < issued; ++st)
+          if (!mbar_wait_bounded(&full[st % STAGES], (uint32_t)((st / STAGES) & 1), kWaitSl)) atomicOr(g.err, kErrSl);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {  // MMA issuer
+      const uint32_t idesc = idesc_f16(false, BN);
+      for (int st = 0; st < nst && !failed; ++st) {
+        const int s = st % STAGES, u = st / STAGES, grp = st / KG;
+        const bool first = st % KG == 0, last = st % KG == KG - 1 || st == nst - 1;
+        if (!mbar_wait_bounded(&full[s], (uint32_t)(u & 1), kWaitSl)) {
+          failed = true;
+          break;
+        }
+        tc::tc_fence_after();
+        const uint32_t a0 = smem_u32(base + (size_t)s * S::STAGE_BYTES), b0 = a0 + S::A_BYTES;
+#pragma unroll 1
+        for (int c = 0; c < kDig; ++c) {
+          if (first && grp > 0) {
+            if (!mbar_wait_bounded(&accfree[c], (uint32_t)((grp - 1) & 1), kWaitSl)) {
+              failed = true;
+              break;
+            }
+            tc::tc_fence_after();
+          }
+          const uint32_t d = tmem + (uint32_t)(c * BN);
+          for (int i = 0; i <= c; ++i) {
+            const uint32_t sa = a0 + i * S::A_SLICE, sb = b0 + (c - i) * S::B_SLICE;
+#pragma unroll
+            for (int kk = 0; kk < BK / 16; ++kk)
+              mma_f16(d, desc_k<64>(sa + 32 * kk), desc_k<64>(sb + 32 * kk), idesc,
+                      (first && i == 0 && kk == 0) ? 0u : 1u);
+          }
+          if (last) mma_commit(&accf[c]);
+        }
+        if (failed) break;
+        mma_commit(&empty[s]);
+      }
+      // Never free TMEM under MMAs that may still run.
+      mma_commit(drain);
+      if (!mbar_wait_bounded(drain, 0, kWaitSl)) atomicOr(g.err, kErrSl);
+    }
+  } else {
+    const int wq = warp & 3;              // TMEM lane quarter of this warp
+    const int ch = (warp - 2) >> 2;       // column half: 32 columns
+    const uint32_t lane_base = tmem + ((uint32_t)(32 * wq) << 16) + (uint32_t)(32 * ch);
+    int64_t H[32], L[32];
+#pragma unroll
+    for (int q = 0; q < 32; ++q) H[q] = L[q] = 0;
+    auto fold = [&](int c, int grp, int64_t(&T)[32], int w) -> bool {
+      const bool ok = mbar_wait_bounded(&accf[c], (uint32_t)(grp & 1), kWaitSl);
+      if (!__all_sync(0xffffffffu, ok)) return false;
+      tc::tc_fence_after();
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float v[16];
+        tc::tmem_ld16(lane_base + (uint32_t)(c * BN + 16 * h), v);
+#pragma unroll
+        for (int q = 0; q < 16; ++q) T[16 * h + q] += (int64_t)__float2int_rn(v[q]) * w;
+      }
+      tc::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&accfree[c]);
+      return true;
+    };
+    for (int grp = 0; grp < ngroups && !failed; ++grp) {
+      failed = !(fold(0, grp, H, 1 << 16) && fold(1, grp, H, 1 << 8) && fold(2, grp, H, 1) &&
+                 fold(3, grp, L, 1 << 24) && fold(4, grp, L, 1 << 16) && fold(5, grp, L, 1 << 8) &&
+                 fold(6, grp, L, 1));
+    }
+    const int64_t row = m0 + 32 * wq + lane;
+    const int64_t c0 = n0 + 32 * ch;
+    if (row < g.M && c0 < g.N) {
+      const int ea = g.ea[row];
+      double* dst = g.part ? g.C + ((int64_t)blockIdx.z * g.M + row) * g.N + c0 : g.C + row * g.ldc + c0;
+#pragma unroll
+      for (int q = 0; q < 32; ++q) {
+        if (c0 + q >= g.N) break;
+        const int eb = g.eb[c0 + q];
+        // Entry scales 2^(E - 1022 - 55) each; weights 2^48 and up.
+        double v = scale_int(H[q], L[q], 48 + (ea - 1077) + (eb - 1077));
+        if (failed || ea >= kNonFiniteExp || eb >= kNonFiniteExp) v = __longlong_as_double(0x7ff8000000000000ll);
+        dst[q] = v;
+      }
+    }
+  }
+  if (failed) atomicOr(g.err, kErrSl);
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  if (warp == 0) tc::tmem_dealloc(tmem, S::TMEM_COLS);
+}
+
+// --------------------------------------------- 16-bit A, B in three slices
+struct A16 {
+  static constexpr int BNMAX = 256, BK = 64, STAGES = 2, NB = 3;
+  static constexpr uint32_t A_BYTES = BM * BK * 2;
+  static constexpr uint32_t B_SLICE_MAX = BNMAX * BK * 2;
+  static constexpr uint32_t STAGE_BYTES = A_BYTES + NB * B_SLICE_MAX;
+  static constexpr size_t smem_bytes() { return 1024 + (size_t)STAGES * STAGE_BYTES + 256; }
+  static constexpr uint32_t TMEM_COLS = 2 * BNMAX;
+  static_assert(STAGES * STAGE_BYTES + 1280 <= 227 * 1024, "shared memory");
+};
+
+struct A16Args {
+  int64_t M, N, K;
+  float* C;
+  int64_t ldc;
+  const float* bscale;  // undoes the column scale of B's slices
+  float* Ct;            // optional FP32 copy of C transposed (N x M)
+  int64_t ldct;
+  int bn;               // tile width: a multiple of 16, at most 256
+  int bf16;
+  int* err;
+};
+
+__global__ void __launch_bounds__(kThreads, 1)
+    k_gemm_a16(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, A16Args g) {
+  using S = A16;
+  constexpr int BK = S::BK, STAGES = S::STAGES;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* base = smem_raw + ((1024 - (reinterpret_cast<uintptr_t>(smem_raw) & 1023)) & 1023);
+  uint64_t* full = reinterpret_cast<uint64_t*>(base + STAGES * S::STAGE_BYTES);
+  uint64_t* empty = full + STAGES;
+  uint64_t* accf = empty + STAGES;  // [2]
+  uint64_t* accfree = accf + 2;     // [2]
+  uint64_t* drain = accfree + 2;    // every MMA issued has finished
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int bnw = g.bn;
+  const int64_t tn = (g.N + bnw - 1) / bnw;
+  const int64_t bm = (int64_t)blockIdx.x / tn, bn = (int64_t)blockIdx.x - bm * tn;
+  const int64_t m0 = bm * BM, n0 = bn * bnw;
+  const int nkb = (int)((g.K + BK - 1) / BK);
+  const uint32_t bslice = (uint32_t)bnw * BK * 2;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&accf[b], 1);
+      mbar_init(&accfree[b], 8);
+    }
+    mbar_init(drain, 1);
+    fence_mbar_init();
+  }
+  if (warp == 0) tc::tmem_alloc(tmem_slot, S::TMEM_COLS);
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  bool failed = false;
+
+  if (warp == 0) {
+    if (lane == 0) {  // TMA producer
+      int issued = 0;
+      for (int kb = 0; kb < nkb; ++kb) {
+        const int s = kb % STAGES, u = kb / STAGES;
+        if (u > 0 && !mbar_wait_bounded(&empty[s], (uint32_t)((u - 1) & 1), kWaitSl)) {
+          failed = true;
+          break;
+        }
+        unsigned char* p = base + (size_t)s * S::STAGE_BYTES;
+        mbar_arrive_expect_tx(&full[s], S::A_BYTES + S::NB * bslice);
+        tma_load_2d(p, &mapA, &full[s], kb * BK, (int32_t)m0);
+        tma_load_3d(p + S::A_BYTES, &mapB, &full[s], kb * BK, (int32_t)n0, 0);
+        issued = kb + 1;
+      }
+      if (failed)
+        for (int kb = (issued > STAGES ? issued - STAGES : 0); kb < issued; ++kb)
+          if (!mbar_wait_bounded(&full[kb % STAGES], (uint32_t)((kb / STAGES) & 1), kWaitSl)) atomicOr(g.err, kErrSl);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {  // MMA issuer
+      const uint32_t idesc = idesc_f16(g.bf16 != 0, bnw);
+      for (int kb = 0; kb < nkb; ++kb) {
+        const int s = kb % STAGES, u = kb / STAGES, b = kb & 1;
+        if (!mbar_wait_bounded(&full[s], (uint32_t)(u & 1), kWaitSl) ||
+            (kb >= 2 && !mbar_wait_bounded(&accfree[b], (uint32_t)(((kb >> 1) - 1) & 1), kWaitSl))) {
+          failed = true;
+          break;
+        }
+        tc::tc_fence_after();
+        const uint32_t a0 = smem_u32(base + (size_t)s * S::STAGE_BYTES), b0 = a0 + S::A_BYTES;
+        const uint32_t d = tmem + (uint32_t)(b * S::BNMAX);
+        // Smallest slice first: the truncating additions then happen while
+        // the accumulator is small.
+#pragma unroll
+        for (int q = S::NB - 1; q >= 0; --q) {
+#pragma unroll
+          for (int kk = 0; kk < BK / 16; ++kk)
+            mma_f16(d, desc_k<128>(a0 + 32 * kk), desc_k<128>(b0 + q * bslice + 32 * kk), idesc,
+                    (q == S::NB - 1 && kk == 0) ? 0u : 1u);
+        }
+        mma_commit(&empty[s]);
+        mma_commit(&accf[b]);
+      }
+      // Never free TMEM under MMAs that may still run.
+      mma_commit(drain);
+      if (!mbar_wait_bounded(drain, 0, kWaitSl)) atomicOr(g.err, kErrSl);
+    }
+  } else {
+    const int wq = warp & 3;
+    const int ch = (warp - 2) >> 2;  // column half: 128 columns of the tile
+    const uint32_t lane_base = tmem + ((uint32_t)(32 * wq) << 16) + (uint32_t)(128 * ch);
+    const int nc = min(128, max(0, bnw - 128 * ch));  // columns of this warp (uniform)
+    float run[128];
+#pragma unroll
+    for (int i = 0; i < 128; ++i) run[i] = 0.f;
+    for (int kb = 0; kb < nkb; ++kb) {
+      const bool ok = mbar_wait_bounded(&accf[kb & 1], (uint32_t)((kb >> 1) & 1), kWaitSl);
+      if (!__all_sync(0xffffffffu, ok)) {
+        failed = true;
+        break;
+      }
+      tc::tc_fence_after();
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        if (16 * c < nc) {
+          float v[16];
+          tc::tmem_ld16(lane_base + (uint32_t)((kb & 1) * S::BNMAX + 16 * c), v);
+#pragma unroll
+          for (int q = 0; q < 16; ++q) run[16 * c + q] += v[q];
+        }
+      }
+      tc::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&accfree[kb & 1]);
+    }
+    const int64_t row = m0 + 32 * wq + lane;
+    const int64_t c0 = n0 + 128 * ch;
+    const int64_t left = g.N - c0;
+    const int ncol = (int)(left < nc ? left : nc);
+    if (row < g.M && ncol > 0) {
+      float* dst = g.C + row * g.ldc + c0;
+      float* ct = g.Ct ? g.Ct + c0 * g.ldct + row : nullptr;
+#pragma unroll
+      for (int q = 0; q < 128; ++q) {
+        if (q < ncol) {
+          const float x = failed ? __int_as_float(0x7fc00000) : run[q] * __ldg(g.bscale + c0 + q);
+          dst[q] = x;
+          // Column q is row c0 + q of C^T; lane = row of C: 128 contiguous
+          // bytes per warp store.
+          if (ct) ct[(int64_t)q * g.ldct] = x;
+        }
+      }
+    }
+  }
+  if (failed) atomicOr(g.err, kErrSl);
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  if (warp == 0) tc::tmem_dealloc(tmem, S::TMEM_COLS);
+}
+
+}  // namespace sl
+}  // namespace bsrht

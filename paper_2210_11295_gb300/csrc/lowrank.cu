@@ -82,10 +82,22 @@ int tall_gemm(const Dla& d, Arena& ar, DT ta, DT tc, DT tout, int64_t M, int64_t
         if (st != BSRHT_OK && st != BSRHT_EUNSUP) return st;
       }
     }
+    if (!ar.lean && tc == DT::F32 && tout == DT::F32 && gemm_a16_eligible(ta, M, N, K, nullptr, lda)) {
+      const int st = gemm_a16(d, ar, ta, M, N, K, nullptr, lda, DT::F64, nullptr, ldb, nullptr, ldc, Ct);
+      ar.release(mk);
+      if (st != BSRHT_OK) return st;
+    }
     const int st = gemm_c(d, ar, ta, tc, tout, M, N, K, A, lda, false, tc == DT::F64 ? (const void*)B64 : B32, ldb,
                           C, ldc, tri_b, false);
     ar.release(mk);
     return st;
+  }
+  if (tc == DT::F32 && tout == DT::F32 && B64 != nullptr && gemm_a16_eligible(ta, M, N, K, A, lda)) {
+    const size_t mk = ar.mark();
+    const int st = gemm_a16(d, ar, ta, M, N, K, A, lda, DT::F64, B64, ldb, static_cast<float*>(C), ldc, Ct);
+    ar.release(mk);
+    if (st == BSRHT_OK && ct_done) *ct_done = Ct != nullptr;
+    if (st != BSRHT_EUNSUP) return st;
   }
   if (ta == DT::F32 && use_tc(tc, M, N, K, A, lda) && B64 != nullptr) {
     if (tout != DT::F32) Ct = nullptr;
@@ -1254,18 +1266,62 @@ int validate_nystrom_rbf(const bsrht_opts& o, const float* X, int64_t n, int64_t
 
 using namespace bsrht;
 
+namespace bsrht {
+
+// Scratch of one call: run(ar) in a dry arena, with (full) and without (lean)
+// the forms of its products that need more scratch than the others and are
+// left out when the workspace does not hold them.
+template <typename F>
+static int scratch_bytes(F&& run, bool lean, size_t* bytes) {
+  Arena ar;
+  ar.measure = true;
+  ar.lean = lean;
+  TRY(run(ar));
+  *bytes = ar.high + 256;
+  return BSRHT_OK;
+}
+
+// Workspace of a call for run(ar): the caller's (at least the lean size, used
+// up to the full one) or the library pool (the full size, or the lean one
+// when the device cannot give that).
+template <typename F>
+static int take_workspace(const bsrht_opts& o, F&& run, Arena* ar) {
+  size_t need = 0;
+  TRY(scratch_bytes(run, false, &need));
+  void* ws = nullptr;
+  int st = o.workspace && o.workspace_bytes < need ? BSRHT_ENOMEM : workspace_for(&o, need, &ws);
+  if (st == BSRHT_ENOMEM) {
+    TRY(scratch_bytes(run, true, &need));
+    st = workspace_for(&o, need, &ws);
+    if (o.workspace) need = std::max(need, o.workspace_bytes);
+  }
+  if (st != BSRHT_OK) return st;
+  ar->base = static_cast<char*>(ws);
+  ar->cap = need;
+  return BSRHT_OK;
+}
+
+int rsvd_scratch(const bsrht_opts& o, int64_t n, int64_t m, int k, int64_t l, int p, bool lean, size_t* bytes) {
+  TRY(validate_rsvd(o, n, m, k, l, p));
+  return scratch_bytes(
+      [&](Arena& ar) { return rsvd_impl(o, nullptr, n, m, k, l, p, 0, nullptr, nullptr, nullptr, ar, true); }, lean,
+      bytes);
+}
+
+int nystrom_scratch(const bsrht_opts& o, int64_t n, int k, int64_t l, int p, bool lean, size_t* bytes) {
+  TRY(validate_nystrom(o, n, k, l, p));
+  return scratch_bytes([&](Arena& ar) { return nystrom_impl(o, nullptr, n, k, l, p, 0, nullptr, nullptr, ar, true); },
+                       lean, bytes);
+}
+
+}  // namespace bsrht
+
 extern "C" {
 
 int bsrht_rsvd_workspace(int64_t n, int64_t m, int32_t k, int64_t l, int32_t p, const bsrht_opts* opts,
                          size_t* bytes) {
   if (!bytes) return BSRHT_EINVAL;
-  const bsrht_opts o = opts_or_default(opts);
-  TRY(validate_rsvd(o, n, m, k, l, p));
-  Arena ar;
-  ar.measure = true;
-  TRY(rsvd_impl(o, nullptr, n, m, k, l, p, 0, nullptr, nullptr, nullptr, ar, true));
-  *bytes = ar.high + 256;
-  return BSRHT_OK;
+  return rsvd_scratch(opts_or_default(opts), n, m, k, l, p, false, bytes);
 }
 
 int bsrht_rsvd(const void* A, int64_t n, int64_t m, int32_t k, int64_t l, int32_t p, uint64_t seed, double* U,
@@ -1273,13 +1329,9 @@ int bsrht_rsvd(const void* A, int64_t n, int64_t m, int32_t k, int64_t l, int32_
   const bsrht_opts o = opts_or_default(opts);
   TRY(validate_rsvd(o, n, m, k, l, p));
   if (!A || !U || !S || !V) return BSRHT_EINVAL;
-  size_t need = 0;
-  TRY(bsrht_rsvd_workspace(n, m, k, l, p, &o, &need));
-  void* ws = nullptr;
-  TRY(workspace_for(&o, need, &ws));
   Arena ar;
-  ar.base = static_cast<char*>(ws);
-  ar.cap = need;
+  TRY(take_workspace(
+      o, [&](Arena& a) { return rsvd_impl(o, nullptr, n, m, k, l, p, 0, nullptr, nullptr, nullptr, a, true); }, &ar));
   return rsvd_impl(o, A, n, m, k, l, p, seed, U, S, V, ar, false);
 }
 
@@ -1288,11 +1340,9 @@ int bsrht_srsvd_workspace(int64_t n, int64_t m, int32_t k, int64_t l, int64_t s,
   if (!bytes) return BSRHT_EINVAL;
   const bsrht_opts o = opts_or_default(opts);
   TRY(validate_srsvd(o, n, m, k, l, s, p));
-  Arena ar;
-  ar.measure = true;
-  TRY(srsvd_impl(o, nullptr, n, m, k, l, s, p, 0, nullptr, nullptr, nullptr, ar, true));
-  *bytes = ar.high + 256;
-  return BSRHT_OK;
+  return scratch_bytes(
+      [&](Arena& ar) { return srsvd_impl(o, nullptr, n, m, k, l, s, p, 0, nullptr, nullptr, nullptr, ar, true); },
+      false, bytes);
 }
 
 int bsrht_srsvd(const void* A, int64_t n, int64_t m, int32_t k, int64_t l, int64_t s, int32_t p, uint64_t seed,
@@ -1300,25 +1350,16 @@ int bsrht_srsvd(const void* A, int64_t n, int64_t m, int32_t k, int64_t l, int64
   const bsrht_opts o = opts_or_default(opts);
   TRY(validate_srsvd(o, n, m, k, l, s, p));
   if (!A || !U || !S || !V) return BSRHT_EINVAL;
-  size_t need = 0;
-  TRY(bsrht_srsvd_workspace(n, m, k, l, s, p, &o, &need));
-  void* ws = nullptr;
-  TRY(workspace_for(&o, need, &ws));
   Arena ar;
-  ar.base = static_cast<char*>(ws);
-  ar.cap = need;
+  TRY(take_workspace(
+      o, [&](Arena& a) { return srsvd_impl(o, nullptr, n, m, k, l, s, p, 0, nullptr, nullptr, nullptr, a, true); },
+      &ar));
   return srsvd_impl(o, A, n, m, k, l, s, p, seed, U, S, V, ar, false);
 }
 
 int bsrht_nystrom_workspace(int64_t n, int32_t k, int64_t l, int32_t p, const bsrht_opts* opts, size_t* bytes) {
   if (!bytes) return BSRHT_EINVAL;
-  const bsrht_opts o = opts_or_default(opts);
-  TRY(validate_nystrom(o, n, k, l, p));
-  Arena ar;
-  ar.measure = true;
-  TRY(nystrom_impl(o, nullptr, n, k, l, p, 0, nullptr, nullptr, ar, true));
-  *bytes = ar.high + 256;
-  return BSRHT_OK;
+  return nystrom_scratch(opts_or_default(opts), n, k, l, p, false, bytes);
 }
 
 
@@ -1333,11 +1374,9 @@ int bsrht_nystrom_rbf_workspace(int64_t n, int64_t dim, int32_t k, int64_t l, in
   src.ldx = o.lda ? o.lda : dim;
   src.h = 1.0;
   o.lda = 0;
-  Arena ar;
-  ar.measure = true;
-  TRY(nystrom_impl(o, nullptr, n, k, l, p, 0, nullptr, nullptr, ar, true, src));
-  *bytes = ar.high + 256;
-  return BSRHT_OK;
+  return scratch_bytes(
+      [&](Arena& ar) { return nystrom_impl(o, nullptr, n, k, l, p, 0, nullptr, nullptr, ar, true, src); }, false,
+      bytes);
 }
 
 int bsrht_nystrom_rbf(const float* X, int64_t n, int64_t dim, double h, int32_t k, int64_t l, int32_t p,
@@ -1345,10 +1384,6 @@ int bsrht_nystrom_rbf(const float* X, int64_t n, int64_t dim, double h, int32_t 
   bsrht_opts o = opts_or_default(opts);
   if (!X || !U || !Lambda) return BSRHT_EINVAL;
   TRY(validate_nystrom_rbf(o, X, n, dim, h, k, l, p));
-  size_t need = 0;
-  TRY(bsrht_nystrom_rbf_workspace(n, dim, k, l, p, &o, &need));
-  void* ws = nullptr;
-  TRY(workspace_for(&o, need, &ws));
   RbfSource src;
   src.X = X;
   src.dim = dim;
@@ -1356,8 +1391,8 @@ int bsrht_nystrom_rbf(const float* X, int64_t n, int64_t dim, double h, int32_t 
   src.h = h;
   o.lda = 0;
   Arena ar;
-  ar.base = static_cast<char*>(ws);
-  ar.cap = need;
+  TRY(take_workspace(
+      o, [&](Arena& a) { return nystrom_impl(o, nullptr, n, k, l, p, 0, nullptr, nullptr, a, true, src); }, &ar));
   return nystrom_impl(o, nullptr, n, k, l, p, seed, U, Lambda, ar, false, src);
 }
 
@@ -1366,13 +1401,9 @@ int bsrht_nystrom(const void* A, int64_t n, int32_t k, int64_t l, int32_t p, uin
   const bsrht_opts o = opts_or_default(opts);
   TRY(validate_nystrom(o, n, k, l, p));
   if (!A || !U || !Lambda) return BSRHT_EINVAL;
-  size_t need = 0;
-  TRY(bsrht_nystrom_workspace(n, k, l, p, &o, &need));
-  void* ws = nullptr;
-  TRY(workspace_for(&o, need, &ws));
   Arena ar;
-  ar.base = static_cast<char*>(ws);
-  ar.cap = need;
+  TRY(take_workspace(o, [&](Arena& a) { return nystrom_impl(o, nullptr, n, k, l, p, 0, nullptr, nullptr, a, true); },
+                     &ar));
   return nystrom_impl(o, A, n, k, l, p, seed, U, Lambda, ar, false);
 }
 

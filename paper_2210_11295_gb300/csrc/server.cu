@@ -471,11 +471,15 @@ int validate_and_size(bsrht_server* sv, const bsrht_request& r, Req& q) {
     }
   } else if (r.kind == BSRHT_REQ_RSVD) {
     if (!r.U || !r.S || !r.V) return BSRHT_EINVAL;
-    const int st = bsrht_rsvd_workspace(r.n, r.m, r.k, r.l, r.p, &o, &bytes);
+    int st = rsvd_scratch(o, r.n, r.m, r.k, r.l, r.p, false, &bytes);
+    if (st == BSRHT_OK && FirstFit::round(bytes) > sv->alloc.cap())
+      st = rsvd_scratch(o, r.n, r.m, r.k, r.l, r.p, true, &bytes);
     if (st != BSRHT_OK) return st;
   } else {
     if (!r.U || !r.S) return BSRHT_EINVAL;
-    const int st = bsrht_nystrom_workspace(r.n, r.k, r.l, r.p, &o, &bytes);
+    int st = nystrom_scratch(o, r.n, r.k, r.l, r.p, false, &bytes);
+    if (st == BSRHT_OK && FirstFit::round(bytes) > sv->alloc.cap())
+      st = nystrom_scratch(o, r.n, r.k, r.l, r.p, true, &bytes);
     if (st != BSRHT_OK) return st;
   }
   q.bytes = FirstFit::round(bytes);

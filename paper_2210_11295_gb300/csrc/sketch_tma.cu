@@ -825,6 +825,19 @@ bool make_tensor_map_2d(CUtensorMap* map, const void* base, CUtensorMapDataType 
             swizzle, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool make_tensor_map_3d(CUtensorMap* map, const void* base, CUtensorMapDataType dtype, size_t elem_bytes,
+                        uint64_t cols, uint64_t rows, uint64_t planes, uint64_t ld, uint64_t plane_ld,
+                        uint32_t box_cols, uint32_t box_rows, uint32_t box_planes, CUtensorMapSwizzle swizzle) {
+  EncodeFn fn = encode_fn();
+  if (!fn) return false;
+  const cuuint64_t dims[3] = {cols, rows, planes};
+  const cuuint64_t strides[2] = {ld * elem_bytes, plane_ld * elem_bytes};
+  const cuuint32_t box[3] = {box_cols, box_rows, box_planes};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return fn(map, dtype, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            swizzle, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 
 int sketch_occupancy_tma(const SketchPlan& plan) {
   switch (plan.dtype) {

@@ -65,5 +65,10 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, u
 bool make_tensor_map_2d(CUtensorMap* map, const void* base, CUtensorMapDataType dtype, size_t elem_bytes,
                         uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_cols, uint32_t box_rows,
                         CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_NONE);
+// The same for `planes` matrices of equal shape, plane_ld elements apart
+// (box box_cols x box_rows x box_planes).
+bool make_tensor_map_3d(CUtensorMap* map, const void* base, CUtensorMapDataType dtype, size_t elem_bytes,
+                        uint64_t cols, uint64_t rows, uint64_t planes, uint64_t ld, uint64_t plane_ld,
+                        uint32_t box_cols, uint32_t box_rows, uint32_t box_planes, CUtensorMapSwizzle swizzle);
 
 }  // namespace bsrht
