@@ -13,6 +13,7 @@
 #include "gemm.cuh"
 #include "sketch.cuh"
 #include "f32x2.cuh"
+#include "jacobi_cluster.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -882,6 +883,170 @@ __global__ void k_ns_coeff(double* __restrict__ G, int64_t l) {
   if (idx < l * l) G[idx] = (idx / l == idx % l ? 1.5 : 0.0) - 0.5 * G[idx];
 }
 
+// out[c][r] = in[r][c] 2^-e in FP32, 2^e <= *fnorm < 2^(e+1): the columns of
+// M^T (row-major in = M by columns) at Frobenius norm 1 to 2, so that squared
+// norms and products of them stay in FP32's range.
+__global__ void __launch_bounds__(256) k_transpose_scaled32(const double* __restrict__ in, int64_t l,
+                                                            const double* __restrict__ fnorm,
+                                                            float* __restrict__ out) {
+  __shared__ float t[32][33];
+  const double f = *fnorm;
+  const double sc = f > 0.0 && f < INFINITY ? scalbn(1.0, -ilogb(f)) : 1.0;
+  const int64_t bx = (int64_t)blockIdx.x * 32, by = (int64_t)blockIdx.y * 32;
+  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  for (int r = ty; r < 32; r += 8) {
+    const int64_t i = by + r, j = bx + tx;
+    t[r][tx] = (i < l && j < l) ? (float)(in[i * l + j] * sc) : 0.f;
+  }
+  __syncthreads();
+  for (int r = ty; r < 32; r += 8) {
+    const int64_t i = bx + r, j = by + tx;
+    if (i < l && j < l) out[i * l + j] = t[tx][r];
+  }
+}
+
+// V[i][r] = column perm[r] of X over its norm, entry i (row-major l x s).
+__global__ void k_gather_directions(const float* __restrict__ X, const double* __restrict__ nrm,
+                                    const int* __restrict__ perm, int64_t l, int64_t s, double* __restrict__ V) {
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= l * s) return;
+  const int64_t i = idx / s, r = idx - i * s;
+  const int64_t c = perm[r];
+  const double n = nrm[c];
+  V[idx] = n > 0.0 ? (double)X[c * l + i] / n : 0.0;
+}
+
+__global__ void k_scale_cols(double* X, int64_t rows, int64_t cols, int64_t ld, const double* sc, int inv);
+
+// Flags of the FP64 refinement.
+constexpr int kRefPair = 1;     // some pair's cosine exceeds the stopping threshold
+constexpr int kRefCluster = 2;  // such a pair is too close for the first-order rotation
+constexpr int kRefCoarse = 4;   // such a pair turns by more than kRefFine
+constexpr int kRefOrth = 8;     // V was not yet orthogonal to rounding
+// Below this angle I + X + X^2 / 2 is a rotation to rounding (error X^4 / 4).
+constexpr double kRefFine = 0x1.0p-26;
+
+// Coefficients of one orthonormalisation step V <- V G of nearly orthonormal
+// columns from their Gram G, in place.  tri: Gram-Schmidt to first order
+// (each column less its components along the ones before it, which are the
+// larger singular directions and not touched for the later ones' sake);
+// otherwise Newton-Schulz, 1.5 I - 0.5 G.  Deviations of G from I above
+// `loose` set `bit` in *flags.
+__global__ void k_orth_coeff(double* __restrict__ G, int64_t n, int tri, double loose, int bit,
+                             int* __restrict__ flags) {
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= n * n) return;
+  const int64_t i = idx / n, j = idx - i * n;
+  const double g = G[idx];
+  if (!(fabs(g - (i == j ? 1.0 : 0.0)) <= loose)) atomicOr(flags, bit);
+  if (tri)
+    G[idx] = i == j ? 1.5 - 0.5 * g : i < j ? -g : 0.0;
+  else
+    G[idx] = (i == j ? 1.5 : 0.0) - 0.5 * g;
+}
+
+// U[i][j] = Y[i][j] / sig[j], sig[j] = sqrt(G[j][j]) the norm of column j of Y
+// (row-major l x n).
+__global__ void k_normalize_cols(const double* __restrict__ Y, const double* __restrict__ G, int64_t l, int64_t n,
+                                 double* __restrict__ U, double* __restrict__ sig) {
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= l * n) return;
+  const int64_t j = idx % n;
+  const double s = sqrt(G[j * n + j]);
+  if (idx < n) sig[j] = s;
+  U[idx] = s > 0.0 ? Y[idx] / s : 0.0;
+}
+
+// sig[j] *= sqrt(C[j][j]): the norms of U diag(sig) from C = U^T U.
+__global__ void k_scale_norms(const double* __restrict__ C, int64_t n, double* __restrict__ sig) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j < n) sig[j] *= sqrt(C[j * n + j]);
+}
+
+// Generators of the rotation that makes the columns of Y = U diag(sig)
+// orthogonal to first order, from C = U^T U (norms of U's columns near 1,
+// sig without them): V (I + X) and U (I + Z), X_ij = c s_i s_j / (s_j^2 - s_i^2),
+// Z = D X D^-1 (D = diag(s)), c the cosine of the pair and s_i = sig_i |u_i|.
+// Z (for U's columns once normalised) stays as small as the cosines (over the relative gaps) however far apart
+// the norms are, so small columns are made orthogonal to their own accuracy.
+// Pairs with |X_ij| > 0.03 (clustered singular values) are left alone.
+// Flags: see above; a pair exceeds by the test of a Jacobi sweep (k_jacobi).
+__global__ void k_refine_generator(const double* __restrict__ C, const double* __restrict__ sig, int64_t n,
+                                   const double* __restrict__ fnorm, double tiny_rel, double tol,
+                                   double* __restrict__ X, double* __restrict__ Z, int* __restrict__ flags) {
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= n * n) return;
+  const int64_t i = idx / n, j = idx - i * n;
+  double x = 0.0, z = 0.0;
+  if (i != j) {
+    const double tiny = tiny_rel * fnorm[0];
+    // The entry of the upper triangle for both, so that X is antisymmetric.
+    const double g = i < j ? C[idx] : C[j * n + i];
+    const double ni = C[i * n + i], nj = C[j * n + j];
+    const double si = sig[i] * sqrt(ni), sj = sig[j] * sqrt(nj);
+    if (!(si <= tiny && sj <= tiny) && g != 0.0) {
+      const bool exceeds = !(g * g <= tol * tol * ni * nj);
+      // Ratio of the smaller norm to the larger one: no overflow, no
+      // difference of squares.
+      const bool up = sj >= si;
+      const double q = up ? si / sj : sj / si;
+      const double den = (1.0 - q) * (1.0 + q);       // |s_j^2 - s_i^2| / max^2
+      const double c = g / sqrt(ni * nj);
+      const bool ok = fabs(c) * q <= 0.03 * den;
+      if (ok) {
+        x = (up ? c : -c) * q / den;
+        z = up ? c * (q * q) / den : -c / den;        // s_i^2 over s_j^2 - s_i^2
+      }
+      if (exceeds) {
+        int f = kRefPair;
+        if (!ok) f |= kRefCluster;
+        if (fabs(x) > kRefFine) f |= kRefCoarse;
+        atomicOr(flags, f);
+      }
+    }
+  }
+  X[idx] = x;
+  Z[idx] = z;
+}
+
+// T = I + X + P / 2 (P = X X, in place in P).
+__global__ void k_refine_rotation(const double* __restrict__ X, double* __restrict__ P, int64_t n) {
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx < n * n) P[idx] = (idx / n == idx % n ? 1.0 : 0.0) + X[idx] + 0.5 * P[idx];
+}
+
+// Outputs of an SVD whose s leading columns were refined: entry i of column c
+// of U (Y = U diag(sigS) when `over`: then U = Y / sigS) and of V at
+// [i si + c sc], norms sigS, ranks permS.  Ranks >= s
+// (not used by a caller with s < l): the FP32 phase's directions and norms
+// (X, nrm, perm; scaled back by *fnorm's power of two), U zero.
+__global__ void k_svd_finish_lead(const double* __restrict__ Y, const double* __restrict__ V, int over, int64_t si,
+                                  int64_t sc,
+                                  const double* __restrict__ sigS, const int* __restrict__ permS, int64_t s,
+                                  const float* __restrict__ X, const double* __restrict__ nrm,
+                                  const int* __restrict__ perm, const double* __restrict__ fnorm, int64_t l,
+                                  double* __restrict__ U, double* __restrict__ Vout, double* __restrict__ sig_out) {
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= l * l) return;
+  const int64_t i = idx / l, r = idx - i * l;
+  double u = 0.0, v, sv;
+  if (r < s) {
+    const int64_t c = permS[r];
+    sv = sigS[c];
+    if (sv > 0.0) u = over ? Y[i * si + c * sc] / sv : Y[i * si + c * sc];
+    v = V[i * si + c * sc];
+  } else {
+    const int64_t c = perm[r];
+    const double f = *fnorm;
+    const double n = nrm[c];
+    sv = f > 0.0 && f < INFINITY ? scalbn(n, ilogb(f)) : n;
+    v = n > 0.0 ? (double)X[c * l + i] / n : 0.0;
+  }
+  U[idx] = u;
+  Vout[idx] = v;
+  if (i == 0) sig_out[r] = sv;
+}
+
 namespace {
 
 // WP warps per column pair (measured on GB300 at l = 128 .. 1024): two for
@@ -1238,6 +1403,65 @@ int launch_jacobi_blk(const Dla& d, float* M, float* V, int64_t l, double tol, d
   return launch_jacobi_blk_jr<8>(d, M, V, l, tol, tol_stop, fnorm, tiny_rel, max_sweeps, rot);
 }
 
+// The FP32 phase in one cluster (jacobi_cluster.cuh) for 64 < l <= 768: the
+// columns X (l columns of l entries) are rotated until every pair that counts
+// is orthogonal.  BSRHT_EUNSUP when the device cannot hold the cluster.
+// Blocks of at most 16 columns (24 above l = 512): smaller clusters for
+// smaller l, since an exchange costs more than a round.
+template <int JQ, int MAXT>
+int launch_jacobi_cluster_jq(const Dla& d, jc::Args a, int nc) {
+  auto kern = jc::k_jacobi_cluster<JQ, MAXT>;
+  const size_t smem = jc::smem_bytes(a.B, a.ld);
+  // Host threads launch one instance at several sizes at once: the attribute
+  // always holds the instance's largest need.
+  const size_t smem_max = jc::smem_bytes(MAXT / 32, 128 * JQ);
+  BSRHT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
+  BSRHT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)nc);
+  cfg.blockDim = dim3(32u * (unsigned)a.B);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = d.s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)nc;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return BSRHT_EUNSUP;
+  }
+  if (clusters < 1) return BSRHT_EUNSUP;
+  BSRHT_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, a));
+  note_launches(1);
+  return BSRHT_OK;
+}
+
+int launch_jacobi_cluster(const Dla& d, float* X, int64_t l, double tol, double tol_stop, double tiny, int64_t lead,
+                          int max_sweeps, int* rot, float* nrm) {
+  if (l < 2 || l > jc::kMaxRows) return BSRHT_EUNSUP;
+  const int nc = l <= 64 ? 2 : l <= 128 ? 4 : l <= 256 ? 8 : 16;
+  jc::Args a;
+  a.X = X;
+  a.l = a.rows = (int)l;
+  a.ld = (int)((l + 3) / 4 * 4);
+  a.B = 2 * (int)((l + 4 * nc - 1) / (4 * nc));
+  a.tol2 = (float)(tol * tol);
+  a.tstop2 = (float)(tol_stop * tol_stop);
+  a.tiny2 = (float)(tiny * tiny);
+  a.lead = (int)lead;
+  a.max_sweeps = max_sweeps;
+  a.rot_counts = rot;
+  a.nrm = nrm;
+  if (l <= 128) return launch_jacobi_cluster_jq<1, 512>(d, a, nc);
+  if (l <= 256) return launch_jacobi_cluster_jq<2, 512>(d, a, nc);
+  if (l <= 512) return launch_jacobi_cluster_jq<4, 512>(d, a, nc);
+  return launch_jacobi_cluster_jq<6, 32 * jc::kMaxB>(d, a, nc);
+}
+
 }  // namespace
 
 int jacobi_svd(const Dla& d, Arena& ar, double* colsM, int64_t l, double* U, double* sigma, double* Vout,
@@ -1272,7 +1496,7 @@ int jacobi_svd(const Dla& d, Arena& ar, double* colsM, int64_t l, double* U, dou
   double* sigS = static_cast<double*>(ar.take(sizeof(double) * l));
   int* permS = static_cast<int*>(ar.take(sizeof(int) * l));
   float *M32 = nullptr, *V32 = nullptr;
-  double *S2 = nullptr, *G = nullptr, *Y = nullptr;
+  double *S2 = nullptr, *G = nullptr, *Y = nullptr, *Ux = nullptr, *Zs = nullptr;
   if (mixed) {
     M32 = static_cast<float*>(ar.take(sizeof(float) * l * l));
     V32 = static_cast<float*>(ar.take(sizeof(float) * l * l));
@@ -1305,7 +1529,8 @@ int jacobi_svd(const Dla& d, Arena& ar, double* colsM, int64_t l, double* U, dou
       TRY_DLA(gemm64(nullptr, true, nullptr, nullptr, true));
       TRY_DLA(gemm64(nullptr, false, nullptr, nullptr, false));
     }
-    if (part) {
+    if (mixed) {
+      TRY_DLA(gemm_f64(s, s, s, nullptr, s, false, nullptr, s, nullptr, s, false));
       TRY_DLA(gemm_f64(l, s, s, nullptr, s, false, nullptr, s, nullptr, s, false));
       TRY_DLA(gemm_f64(l, s, l, nullptr, l, true, nullptr, s, nullptr, s, false));
     }
@@ -1356,7 +1581,184 @@ int jacobi_svd(const Dla& d, Arena& ar, double* colsM, int64_t l, double* U, dou
     return BSRHT_OK;
   };
 
+  // The mixed SVD without accumulated rotations, for l <= 768.
+  // (a) The columns of M^T (scaled, FP32) are rotated in one cluster until
+  //     orthogonal; their directions are M's right singular vectors to FP32
+  //     accuracy.  The factors R of this library's QRs have rows graded like
+  //     the singular values (their columns are random mixes), so the columns
+  //     of R^T need far fewer sweeps than those of R (l = 512 of the
+  //     benchmark's kind: 7 against 13), and no V moves along.  With s < l
+  //     only pairs that hold one of the s largest columns count for the stop.
+  // (b) The s leading directions, largest first, are made orthonormal in
+  //     FP64: one first-order Gram-Schmidt step (a small column carries
+  //     components along larger ones, not the other way round), then
+  //     Newton-Schulz.  Y = M V.
+  // (c) Refinement by products: U = Y over its column norms, C = U^T U; while
+  //     a pair's cosine exceeds the threshold, all pairs are rotated at once
+  //     to first order, V <- V (I + X + X^2 / 2) and U likewise
+  //     (k_refine_generator), which squares the cosines.  While angles are
+  //     large, V is then made orthonormal again and Y = M V formed anew; a
+  //     new Y carries rounding of ||M||, so the last steps, whose angles are
+  //     too small to disturb V, update U itself and leave each column
+  //     orthogonal to its own accuracy.  Pairs too close for first order
+  //     (clustered singular values) are left to FP64 Jacobi sweeps, which
+  //     the result passes through only then.
+  // *done stays false (and colsM as it was) when the FP32 phase's directions
+  // are not near orthonormal (M numerically singular in FP32): the caller
+  // goes on with accumulated rotations.
+  auto lead_svd = [&](bool* done) -> int {
+    Ux = U;     // the outputs serve as scratch until they are written
+    Zs = Vout;
+    float* X = M32;
+    float* nrm = V32;  // 2 NC B squared norms: below l^2 floats
+    const unsigned t32 = (unsigned)((l + 31) / 32);
+    k_transpose_scaled32<<<dim3(t32, t32), 256, 0, d.s>>>(colsM, l, fnorm, X);
+    DLA_LAUNCH_CHECK();
+    // Rotate down to a few FP32 units, stop below 16 sqrt(l) of them: the
+    // last sweep then leaves cosines of rounding size.
+    const double tstop32 = 16.0 * std::sqrt((double)l) * 0x1.0p-24;
+    const int64_t lead = part && ktop > 0 ? s : 0;
+    const int st = launch_jacobi_cluster(d, X, l, 0x1.0p-21, tstop32, (double)l * 0x1.0p-24, lead, 20,
+                                         rot + max_sweeps, nrm);
+    if (st == BSRHT_EUNSUP) return BSRHT_OK;
+    if (st != BSRHT_OK) return st;
+    trace_mark(d.s, "svd_jacobi_fp32");
+    k_col_norms_t<float><<<blocks_for(l, 8), 256, 0, d.s>>>(X, sig, l, l);
+    DLA_LAUNCH_CHECK();
+    k_rank_desc<<<blocks_for(l, 256), 256, 0, d.s>>>(sig, perm, l);
+    DLA_LAUNCH_CHECK();
+    if (part && ktop <= 0) {
+      std::vector<double> sh((size_t)l);
+      BSRHT_CUDA_TRY(cudaMemcpyAsync(sh.data(), sig, sizeof(double) * l, cudaMemcpyDeviceToHost, d.s));
+      BSRHT_CUDA_TRY(cudaStreamSynchronize(d.s));
+      const double smax = *std::max_element(sh.begin(), sh.end());
+      int64_t c = 0;
+      for (double v : sh) c += v > keep_rel * smax;
+      s = with_margin(std::max<int64_t>(c, 1));
+    }
+    double *V = S2, *Vn = Vc, *Xg = Yt, *P = Gc, *Zg = Zs, *sig1 = nrm64;
+    k_gather_directions<<<blocks_for(l * s, 256), 256, 0, d.s>>>(X, sig, perm, l, s, V);
+    DLA_LAUNCH_CHECK();
+    note_launches(4);
+    const unsigned sb = blocks_for(s * s, 256);
+    int flags = 0;
+    auto read_flags = [&]() -> int {
+      BSRHT_CUDA_TRY(cudaMemcpyAsync(&flags, cflag, sizeof(int), cudaMemcpyDeviceToHost, d.s));
+      BSRHT_CUDA_TRY(cudaStreamSynchronize(d.s));
+      return BSRHT_OK;
+    };
+    // One orthonormalisation step of V (l x s), see k_orth_coeff.
+    auto orth_step = [&](bool tri, double loose, int bit) -> int {
+      TRY_DLA(gemm_f64(s, s, l, V, s, true, V, s, G, s, true));
+      k_orth_coeff<<<sb, 256, 0, d.s>>>(G, s, tri ? 1 : 0, loose, bit, cflag);
+      DLA_LAUNCH_CHECK();
+      note_launches(1);
+      TRY_DLA(gemm_f64(l, s, s, V, s, false, G, s, Vn, s, false));
+      std::swap(V, Vn);
+      return BSRHT_OK;
+    };
+    auto form_y = [&]() -> int {  // colsM row-major is M^T
+      return gemm_f64(l, s, l, colsM, l, true, V, s, Y, s, false);
+    };
+    BSRHT_CUDA_TRY(cudaMemsetAsync(cflag, 0, sizeof(int), d.s));
+    TRY_DLA(orth_step(true, 1e-3, kRefCluster));
+    TRY_DLA(read_flags());
+    if (flags) {  // not near orthonormal
+      s = part && ktop > 0 ? s : l;
+      BSRHT_CUDA_TRY(cudaMemsetAsync(rot, 0, sizeof(int) * 2 * max_sweeps, d.s));
+      return BSRHT_OK;
+    }
+    constexpr double kLoose = 1e-10;  // one Newton-Schulz step then reaches rounding
+    TRY_DLA(orth_step(false, kLoose, kRefOrth));
+    TRY_DLA(form_y());
+    trace_mark(d.s, "svd_orthogonalize");
+    const double tiny_rel = std::max((double)l * 0x1.0p-53, zero_rel);
+    const unsigned lb = blocks_for(l * s, 256);
+    double* U1 = Y;    // normalised columns of Y
+    double* U2 = Ux;   // Y's other buffer
+    auto normalize_y = [&]() -> int {
+      TRY_DLA(gemm_f64(s, s, l, Y, s, true, Y, s, G, s, true));
+      k_normalize_cols<<<lb, 256, 0, d.s>>>(Y, G, l, s, U1 = Y, sigS);
+      DLA_LAUNCH_CHECK();
+      note_launches(1);
+      U2 = Ux;
+      return BSRHT_OK;
+    };
+    // T = I + X + X^2 / 2 in P, and W <- W T (W its partner buffer swapped).
+    auto rotate = [&](const double* gen, double*& W, double*& Wn) -> int {
+      TRY_DLA(gemm_f64(s, s, s, gen, s, false, gen, s, P, s, false));
+      k_refine_rotation<<<sb, 256, 0, d.s>>>(gen, P, s);
+      DLA_LAUNCH_CHECK();
+      note_launches(1);
+      TRY_DLA(gemm_f64(l, s, s, W, s, false, P, s, Wn, s, false));
+      std::swap(W, Wn);
+      return BSRHT_OK;
+    };
+    TRY_DLA(normalize_y());
+    bool converged = false;
+    for (int it = 0; it < 8; ++it) {
+      TRY_DLA(gemm_f64(s, s, l, U1, s, true, U1, s, G, s, true));
+      k_refine_generator<<<sb, 256, 0, d.s>>>(G, sigS, s, fnorm, tiny_rel, tol, Xg, Zg, cflag);
+      DLA_LAUNCH_CHECK();
+      note_launches(1);
+      TRY_DLA(read_flags());
+      converged = flags == 0;
+      if (converged || !(flags & (kRefCoarse | kRefOrth))) {
+        k_scale_norms<<<blocks_for(s, 256), 256, 0, d.s>>>(G, s, sigS);
+        k_normalize_cols<<<lb, 256, 0, d.s>>>(U1, G, l, s, U1, sig1);
+        DLA_LAUNCH_CHECK();
+        note_launches(2);
+      }
+      if (converged) break;
+      BSRHT_CUDA_TRY(cudaMemsetAsync(cflag, 0, sizeof(int), d.s));
+      if (flags & (kRefCoarse | kRefOrth)) {
+        if (flags & kRefPair) TRY_DLA(rotate(Xg, V, Vn));
+        TRY_DLA(orth_step(false, kLoose, kRefOrth));
+        TRY_DLA(form_y());
+        TRY_DLA(normalize_y());
+      } else {
+        TRY_DLA(rotate(Xg, V, Vn));
+        TRY_DLA(rotate(Zg, U1, U2));
+      }
+      if ((flags & kRefCluster) && !(flags & kRefOrth)) break;
+    }
+    const double *Yf = U1, *Vf = V;
+    int64_t si = s, sc = 1;
+    if (!converged) {
+      // FP64 Jacobi sweeps on the columns of U diag(sig) (the caller's M is
+      // spent).
+      k_scale_cols<<<lb, 256, 0, d.s>>>(U1, l, s, s, sigS, 0);
+      DLA_LAUNCH_CHECK();
+      TRY_DLA(transpose_cast(d, DT::F64, U1, l, s, s, DT::F64, colsM, l));
+      TRY_DLA(transpose_cast(d, DT::F64, V, l, s, s, DT::F64, G, l));
+      TRY_DLA(polish(colsM, G, s, l));
+      k_col_norms_t<double><<<blocks_for(s, 8), 256, 0, d.s>>>(colsM, sigS, s, l);
+      Yf = colsM;
+      Vf = G;
+      si = 1;
+      sc = l;
+    } else if (U1 == Ux) {  // the output buffer: move it out of the way
+      BSRHT_CUDA_TRY(cudaMemcpyAsync(Y, U1, sizeof(double) * l * s, cudaMemcpyDeviceToDevice, d.s));
+      Yf = Y;
+    }
+    DLA_LAUNCH_CHECK();
+    k_rank_desc<<<blocks_for(s, 256), 256, 0, d.s>>>(sigS, permS, s);
+    DLA_LAUNCH_CHECK();
+    k_svd_finish_lead<<<blocks_for(l * l, 256), 256, 0, d.s>>>(Yf, Vf, converged ? 0 : 1, si, sc, sigS, permS, s, X, sig,
+                                                                perm, fnorm, l, U, Vout, sigma);
+    DLA_LAUNCH_CHECK();
+    note_launches(3);
+    *done = true;
+    return BSRHT_OK;
+  };
+
   double* cols = colsM;
+  // FP32 phase in one cluster, refinement by FP64 products.
+  if (mixed && l <= jc::kMaxRows) {
+    bool done = false;
+    TRY_DLA(lead_svd(&done));
+    if (done) return BSRHT_OK;
+  }
   if (mixed) {
     // 1. FP32 one-sided Jacobi on a copy of M: V32 ~ the right singular
     //    vectors to FP32 accuracy, at 64x the FP64 rate of this GPU (block

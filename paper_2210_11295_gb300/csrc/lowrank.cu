@@ -581,20 +581,16 @@ int rsvd_impl(const bsrht_opts& o, const void* A, int64_t n, int64_t m, int k, i
   const double* Rinv2 = nullptr;
   TRY(orth_robust(d, ar, dry, tc, W1, W2, W3, n, lq, seed ^ 0x52ull, ob, R, true, false, &Pv, &Rinv2, w_t));
   if (!dry) trace_mark(d.s, "tall_qr");
-  // Step 5: SVD of R^T = U~ Sigma~ V~^T.  FP64 data: Jacobi on the columns
-  // of R^T (the rows of R) to FP64 tolerance.  FP32 data: Jacobi on the
-  // columns of R (R = V~ Sigma~ U~^T), so that the accumulated rotations,
-  // orthogonal to FP64 rounding, give U~ (multiplied by the FP64 Q below),
-  // and the polish stops at cosines of polish_tol_fp32(lq): the other factor
-  // V~ meets P, itself orthogonal only to FP32 accuracy.
+  // Step 5: SVD of R = V~ Sigma~ U~^T (R^T = U~ Sigma~ V~^T), Jacobi on the
+  // columns of R: its right factor, orthogonal to FP64 rounding, is U~, which
+  // Q multiplies below.  FP32 data: the polish stops at cosines of
+  // polish_tol_fp32(lq) and on the k leading triplets; the other factor V~
+  // meets P, itself orthogonal only to FP32 accuracy.
   {
     const size_t mk = ar.mark();
-    if (tc == DT::F32) {
-      if (!dry) TRY(transpose_lower_to_upper(d, R, RT, lq));
-      TRY(jacobi_svd(d, ar, RT, lq, Vs, sig, Us, polish_tol_fp32(lq), 0.0, k));
-    } else {
-      TRY(jacobi_svd(d, ar, R, lq, Us, sig, Vs));
-    }
+    if (!dry) TRY(transpose_lower_to_upper(d, R, RT, lq));
+    TRY(jacobi_svd(d, ar, RT, lq, Vs, sig, Us, tc == DT::F32 ? polish_tol_fp32(lq) : 0.0, 0.0,
+                   tc == DT::F32 ? k : 0));
     ar.release(mk);
   }
   if (!dry) trace_mark(d.s, "small_svd");
