@@ -585,6 +585,91 @@ int chol_inv(const Dla& d, double* g, double* LT, double* Rinv, double* T, doubl
   return BSRHT_OK;
 }
 
+// ------------------------------------- Cholesky of a matrix near the identity
+// A1 = Phi(G - I) (strict lower part and half the diagonal, so that A1 + A1^T
+// = G - I), row-major; *e2 += ||G - I||_F^2.
+__global__ void __launch_bounds__(256) k_near_identity(const double* __restrict__ G, int64_t l,
+                                                       double* __restrict__ A1, double* __restrict__ e2) {
+  __shared__ double red[256];
+  double s = 0.0;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < l * l;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = idx / l, j = idx - i * l;
+    const double e = G[idx] - (i == j ? 1.0 : 0.0);
+    A1[idx] = j < i ? e : (i == j ? 0.5 * e : 0.0);
+    s = fma(e, e, s);
+  }
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) atomicAdd(e2, red[0]);
+}
+
+// Second-order factors: with S = A1 A1^T and Q = A1 A1, L = I + A1 - Phi(S)
+// and L^-1 = I - A1 + Phi(S) + Q; LT = L^T, Rinv = L^-T (row-major, upper).
+__global__ void k_near_identity_factors(const double* __restrict__ A1, const double* __restrict__ S,
+                                        const double* __restrict__ Q, int64_t l, double* __restrict__ LT,
+                                        double* __restrict__ Rinv) {
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= l * l) return;
+  const int64_t j = idx / l, i = idx - j * l;  // element (j, i) of the outputs: (i, j) of L and L^-1
+  double lt = 0.0, ri = 0.0;
+  if (i >= j) {
+    const int64_t o = i * l + j;
+    const double id = i == j ? 1.0 : 0.0, phi = i == j ? 0.5 * S[o] : S[o];
+    lt = id + A1[o] - phi;
+    ri = id - A1[o] + phi + Q[o];
+  }
+  LT[idx] = lt;
+  Rinv[idx] = ri;
+}
+
+int chol_inv_near_identity(const Dla& d, Arena& ar, double* g, double* LT, double* Rinv, double* T, double* X,
+                           int64_t l, double bound, bool* done) {
+  *done = false;
+  const size_t mk = ar.mark();
+  double* e2 = static_cast<double*>(ar.take(sizeof(double)));
+  if (!ar.ok()) return BSRHT_ENOMEM;
+  auto product = [&](const double* A, bool a_trans, const double* B, double* C) -> int {
+    const size_t m2 = ar.mark();
+    const int st = gemm(d, ar, DT::F64, DT::F64, DT::F64, true, l, l, l, A, l, a_trans, B, l, C, l, 1.0, 0.0, false,
+                        false);
+    ar.release(m2);
+    return st;
+  };
+  if (ar.measure) {
+    int st = product(nullptr, false, nullptr, nullptr);
+    ar.release(mk);
+    return st;
+  }
+  BSRHT_CUDA_TRY(cudaMemsetAsync(e2, 0, sizeof(double), d.s));
+  k_near_identity<<<(unsigned)std::min<int64_t>((l * l + 255) / 256, 512), 256, 0, d.s>>>(g, l, T, e2);
+  DLA_LAUNCH_CHECK();
+  note_launches(1);
+  double h = 0.0;
+  int hs = 0;
+  BSRHT_CUDA_TRY(cudaMemcpyAsync(&h, e2, sizeof(double), cudaMemcpyDeviceToHost, d.s));
+  BSRHT_CUDA_TRY(cudaMemcpyAsync(&hs, d.status, sizeof(int), cudaMemcpyDeviceToHost, d.s));
+  BSRHT_CUDA_TRY(cudaStreamSynchronize(d.s));
+  if (hs & kStatusTcWait) return BSRHT_ETIMEDOUT;
+  ar.release(mk);
+  if (!(h <= bound * bound)) return BSRHT_OK;
+  // X = A1^T, S = A1 A1^T (over g), then X = A1 A1.
+  double* S = g;
+  int st = transpose_lower_to_upper(d, T, X, l);
+  if (st == BSRHT_OK) st = product(T, false, X, S);
+  if (st == BSRHT_OK) st = product(T, false, T, X);
+  if (st != BSRHT_OK) return st;
+  k_near_identity_factors<<<(unsigned)((l * l + 255) / 256), 256, 0, d.s>>>(T, S, X, l, LT, Rinv);
+  DLA_LAUNCH_CHECK();
+  note_launches(1);
+  *done = true;
+  return BSRHT_OK;
+}
+
 // ------------------------------------------------------- Jacobi SVD
 __device__ __forceinline__ int rr_player(int pos, int round, int lp) {
   if (pos == 0) return 0;
@@ -1411,15 +1496,15 @@ int launch_jacobi_blk(const Dla& d, float* M, float* V, int64_t l, double tol, d
 template <int JQ, int MAXT>
 int launch_jacobi_cluster_jq(const Dla& d, jc::Args a, int nc) {
   auto kern = jc::k_jacobi_cluster<JQ, MAXT>;
-  const size_t smem = jc::smem_bytes(a.B, a.ld);
+  const size_t smem = jc::smem_bytes(a.B, a.ld, nc);
   // Host threads launch one instance at several sizes at once: the attribute
   // always holds the instance's largest need.
-  const size_t smem_max = jc::smem_bytes(MAXT / 32, 128 * JQ);
+  const size_t smem_max = jc::smem_bytes(MAXT / 16, 128 * JQ, 16);
   BSRHT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
   BSRHT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)nc);
-  cfg.blockDim = dim3(32u * (unsigned)a.B);
+  cfg.blockDim = dim3(16u * (unsigned)a.B);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = d.s;
   cudaLaunchAttribute at[1];
@@ -1456,10 +1541,10 @@ int launch_jacobi_cluster(const Dla& d, float* X, int64_t l, double tol, double 
   a.max_sweeps = max_sweeps;
   a.rot_counts = rot;
   a.nrm = nrm;
-  if (l <= 128) return launch_jacobi_cluster_jq<1, 512>(d, a, nc);
-  if (l <= 256) return launch_jacobi_cluster_jq<2, 512>(d, a, nc);
-  if (l <= 512) return launch_jacobi_cluster_jq<4, 512>(d, a, nc);
-  return launch_jacobi_cluster_jq<6, 32 * jc::kMaxB>(d, a, nc);
+  if (l <= 128) return launch_jacobi_cluster_jq<1, 256>(d, a, nc);
+  if (l <= 256) return launch_jacobi_cluster_jq<2, 256>(d, a, nc);
+  if (l <= 512) return launch_jacobi_cluster_jq<4, 256>(d, a, nc);
+  return launch_jacobi_cluster_jq<6, 16 * jc::kMaxB>(d, a, nc);
 }
 
 }  // namespace
@@ -1936,6 +2021,32 @@ int cast_copy(const Dla& d, DT tin, const void* in, DT tout, void* out, int64_t 
   else if (tin == DT::F64 && tout == DT::F64)
     k_cast<double, double><<<blocks_for(count, 256), 256, 0, d.s>>>(static_cast<const double*>(in),
                                                                      static_cast<double*>(out), count);
+  else
+    return BSRHT_EUNSUP;
+  DLA_LAUNCH_CHECK();
+  note_launches(1);
+  return BSRHT_OK;
+}
+
+// out[i][c] = in[i][idx[c]] (row-major, leading dimensions l and lk).
+template <typename T>
+__global__ void k_gather_columns(const T* __restrict__ in, int64_t rows, int64_t l, const int* __restrict__ idx,
+                                 int64_t lk, T* __restrict__ out) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= rows * lk) return;
+  const int64_t i = e / lk, c = e - i * lk;
+  out[e] = in[i * l + idx[c]];
+}
+
+int gather_columns(const Dla& d, DT t, const void* in, int64_t rows, int64_t l, const int* idx, int64_t lk,
+                   void* out) {
+  if (rows * lk <= 0) return BSRHT_OK;
+  if (t == DT::F64)
+    k_gather_columns<double><<<blocks_for(rows * lk, 256), 256, 0, d.s>>>(static_cast<const double*>(in), rows, l, idx,
+                                                                          lk, static_cast<double*>(out));
+  else if (t == DT::F32)
+    k_gather_columns<float><<<blocks_for(rows * lk, 256), 256, 0, d.s>>>(static_cast<const float*>(in), rows, l, idx,
+                                                                         lk, static_cast<float*>(out));
   else
     return BSRHT_EUNSUP;
   DLA_LAUNCH_CHECK();

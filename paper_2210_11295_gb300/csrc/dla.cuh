@@ -72,6 +72,16 @@ int tri_inverse(const Dla& d, const double* L, double* LT, double* Rinv, int64_t
 // outputs are then meaningless).
 int chol_inv(const Dla& d, double* g, double* LT, double* Rinv, double* T, double* X, int64_t l);
 
+// The same factors for a G near the identity (the second Gram of CholeskyQR2),
+// by their series to second order: exact to about ||G - I||_F^3, taken when
+// ||G - I||_F <= bound; otherwise nothing is written and *done is false.
+// g is overwritten when the series is taken; T and X are l x l scratch.  Reads ||G - I||_F back on the stream (and
+// the status word: BSRHT_ETIMEDOUT when a product gave up a wait).  Two
+// products and two elementwise passes in place of the FP64 elimination
+// chains of chol_inv (l = 512: 0.8 ms).
+int chol_inv_near_identity(const Dla& d, Arena& ar, double* g, double* LT, double* Rinv, double* T, double* X,
+                           int64_t l, double bound, bool* done);
+
 // One-sided Jacobi SVD of the l x l FP64 matrix given by its COLUMNS:
 // colsM[c*l + i] = M[i][c].  The singular triplets, sorted by descending
 // sigma, go to U (l x l row-major, U[i][c]), sigma and Vout (row-major).
@@ -142,6 +152,9 @@ int householder_q(const Dla& d, Arena& ar, double* X, int64_t rows, int64_t l, d
 // Elementwise helpers.
 int transpose_cast(const Dla& d, DT tin, const void* in, int64_t rows, int64_t cols, int64_t ldin, DT tout,
                    void* out, int64_t ldout);  // out[c][r] = in[r][c]
+// out[i][c] = in[i][idx[c]], c < lk (F64 or F32; rows of l and lk elements).
+int gather_columns(const Dla& d, DT t, const void* in, int64_t rows, int64_t l, const int* idx, int64_t lk,
+                   void* out);
 int cast_copy(const Dla& d, DT tin, const void* in, DT tout, void* out, int64_t count);
 int transpose_lower_to_upper(const Dla& d, const double* Li, double* R, int64_t l);  // R = Li^T
 int scale_columns(const Dla& d, double* X, int64_t rows, int64_t cols, int64_t ld, const double* scale,

@@ -10,11 +10,13 @@
 // memory between steps (even -> odd to the left, odd -> even to the right).
 // The pairs inside the blocks are treated in the first step of a sweep.
 //
-// A step: one warp per pair.  Warp w keeps column w of the first block in
-// registers over the B rounds and meets column (w + r) mod B of the second
-// one in shared memory, so a round moves one column in and out instead of
-// two.  What bounds it: the latency of a round (dot product, warp sum,
-// rotation scalars, barrier) and, from l = 512 on, shared-memory bandwidth.
+// A step: warp w keeps columns 2w and 2w + 1 of the first block in registers
+// over B / 2 rounds and meets columns 2q and 2q + 1, q = (w + r) mod (B / 2),
+// of the second one: two times two independent pairs per round, so that one
+// pair's latency (dot product, warp sum, rotation scalars) hides the other's
+// and a column moves through shared memory once for two rotations.  What
+// bounds it: that latency chain and one barrier a round (measured at l = 512:
+// see launch_jacobi_cluster).
 //
 // No rotations are accumulated: the columns rotated are those of M^T, and
 // when they are orthogonal their directions are M's right singular vectors.
@@ -44,7 +46,9 @@ struct Args {
   float* nrm;        // [2 NC B]: squared column norms between sweeps
 };
 
-inline size_t smem_bytes(int B, int ld) { return sizeof(float) * (3 * (size_t)B * ld + 3 * (size_t)B) + 64; }
+inline size_t smem_bytes(int B, int ld, int nc) {
+  return sizeof(float) * (3 * (size_t)B * ld + 3 * (size_t)B + 2 * (size_t)nc * B) + 64;
+}
 
 __device__ __forceinline__ float wsum(float v) {
 #pragma unroll
@@ -59,14 +63,15 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 }
 
 // tan(theta) of the rotation that makes a pair with squared norms alpha,
-// beta and product gamma orthogonal (the smaller root).  Approximate division
-// and square root: the rotation is orthogonal for any t, and a relative
-// error of t leaves that fraction of the cosine.
+// beta and product gamma orthogonal (the smaller root), h / (|d| + sqrt(d^2 +
+// h^2)) with d = beta - alpha, h = 2 gamma: norms are at most 4 and one of
+// the two is above the zero threshold, so the squares stay in range.
+// Approximate root and division: the rotation is orthogonal for any t, and a
+// relative error of t leaves that fraction of the cosine.
 __device__ __forceinline__ float tangent(float alpha, float beta, float gamma) {
-  const float z = __fdividef(beta - alpha, 2.f * gamma);
-  const float az = fabsf(z);
-  const float t = az > 1e9f ? __fdividef(0.5f, az) : __fdividef(1.f, az + sqrt_approx(fmaf(az, az, 1.f)));
-  return copysignf(t, z);
+  const float d = beta - alpha, h = 2.f * gamma;
+  const float t = __fdividef(h, fabsf(d) + sqrt_approx(fmaf(d, d, h * h)));
+  return d >= 0.f ? t : -t;
 }
 
 // JQ: 16-byte chunks of a column per lane (rows <= 128 JQ).
@@ -77,7 +82,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_jacobi_cluster(Args a) {
   const int NC = (int)cluster.num_blocks(), c = (int)cluster.block_rank();
   const int B = a.B, ld = a.ld, bl = B * ld;
   float* nrm = js + 3 * (size_t)bl;                      // [3][B]
-  int* ids = reinterpret_cast<int*>(nrm + 3 * B);        // block held by each buffer
+  float* all_nrm = nrm + 3 * B;                          // [2 NC B]
+  int* ids = reinterpret_cast<int*>(all_nrm + 2 * NC * B);  // block held by each buffer
   float* s_th = reinterpret_cast<float*>(ids + 3);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, NT = blockDim.x;
   const int n4 = ld / 4;                                  // 16-byte chunks of a column
@@ -112,107 +118,129 @@ __global__ void __launch_bounds__(MAXT, 1) k_jacobi_cluster(Args a) {
     const float2 g = f2_to_float2(f2_add(g0, g1));
     return wsum(g.x + g.y);
   };
-  // Rotates x (registers) against the column yp (shared memory).
-  auto pair = [&](ulonglong2(&x)[JQ], float& alpha, ulonglong2* yp, float* ynrm) {
-    constexpr bool kKeep = JQ <= 4;  // y in registers between dot and rotation
-    ulonglong2 y[kKeep ? JQ : 1];
-    f2 g0 = 0ull, g1 = 0ull;
-#pragma unroll
-    for (int e = 0; e < JQ; ++e) {
-      const ulonglong2 v = chunk(e) < n4 ? yp[chunk(e)] : z2;
-      if constexpr (kKeep) y[e] = v;
-      g0 = f2_fma(x[e].x, v.x, g0);
-      g1 = f2_fma(x[e].y, v.y, g1);
-    }
-    const float beta = *ynrm;
-    const float2 g = f2_to_float2(f2_add(g0, g1));
-    const float gamma = wsum(g.x + g.y);
-    const float g2 = gamma * gamma, ab = alpha * beta;
-    if (!(g2 > a.tol2 * ab) || (alpha <= a.tiny2 && beta <= a.tiny2)) return;
-    const float t = tangent(alpha, beta, gamma);
-    const float cs = rsqrtf(fmaf(t, t, 1.f)), sn = cs * t;
-    const f2 C2 = f2_splat(cs), S2 = f2_splat(sn), N2 = f2_splat(-sn);
-#pragma unroll
-    for (int e = 0; e < JQ; ++e) {
-      if (chunk(e) < n4) {
-        ulonglong2 v;
-        if constexpr (kKeep)
-          v = y[e];
-        else
-          v = yp[chunk(e)];
-        ulonglong2 nx, ny;
-        nx.x = f2_fma(v.x, N2, f2_mul(x[e].x, C2));
-        nx.y = f2_fma(v.y, N2, f2_mul(x[e].y, C2));
-        ny.x = f2_fma(v.x, C2, f2_mul(x[e].x, S2));
-        ny.y = f2_fma(v.y, C2, f2_mul(x[e].y, S2));
-        x[e] = nx;
-        yp[chunk(e)] = ny;
-      }
-    }
-    if (g2 > a.tstop2 * ab && fmaxf(alpha, beta) >= th) ++mycount;
-    alpha = fmaf(-t, gamma, alpha);
-    __syncwarp();  // every lane has read *ynrm
-    if (lane == 0) *ynrm = fmaf(t, gamma, beta);
-  };
-  auto load_x = [&](ulonglong2(&x)[JQ], const ulonglong2* p) {
+  auto load = [&](ulonglong2(&x)[JQ], const ulonglong2* p) {
 #pragma unroll
     for (int e = 0; e < JQ; ++e) x[e] = chunk(e) < n4 ? p[chunk(e)] : z2;
   };
-  auto store_x = [&](const ulonglong2(&x)[JQ], ulonglong2* p) {
+  auto store = [&](const ulonglong2(&x)[JQ], ulonglong2* p) {
 #pragma unroll
     for (int e = 0; e < JQ; ++e)
       if (chunk(e) < n4) p[chunk(e)] = x[e];
   };
+  auto dot = [&](const ulonglong2(&x)[JQ], const ulonglong2(&y)[JQ]) {
+    f2 g0 = 0ull, g1 = 0ull;
+#pragma unroll
+    for (int e = 0; e < JQ; ++e) {
+      g0 = f2_fma(x[e].x, y[e].x, g0);
+      g1 = f2_fma(x[e].y, y[e].y, g1);
+    }
+    const float2 g = f2_to_float2(f2_add(g0, g1));
+    return g.x + g.y;
+  };
+  // Tangent of the pair's rotation, 0 for none; squared norms updated.
+  auto scalars = [&](float gamma, float& alpha, float& beta) {
+    const float g2 = gamma * gamma, ab = alpha * beta;
+    if (!(g2 > a.tol2 * ab) || (alpha <= a.tiny2 && beta <= a.tiny2)) return 0.f;
+    const float t = tangent(alpha, beta, gamma);
+    if (g2 > a.tstop2 * ab && fmaxf(alpha, beta) >= th) ++mycount;
+    alpha = fmaf(-t, gamma, alpha);
+    beta = fmaf(t, gamma, beta);
+    return t;
+  };
+  auto rotate = [&](ulonglong2(&x)[JQ], ulonglong2(&y)[JQ], float t) {
+    const float cs = rsqrtf(fmaf(t, t, 1.f)), sn = cs * t;
+    const f2 C2 = f2_splat(cs), S2 = f2_splat(sn), N2 = f2_splat(-sn);
+#pragma unroll
+    for (int e = 0; e < JQ; ++e) {
+      const ulonglong2 u = x[e], v = y[e];
+      x[e].x = f2_fma(v.x, N2, f2_mul(u.x, C2));
+      x[e].y = f2_fma(v.y, N2, f2_mul(u.y, C2));
+      y[e].x = f2_fma(v.x, C2, f2_mul(u.x, S2));
+      y[e].y = f2_fma(v.y, C2, f2_mul(u.y, S2));
+    }
+  };
+  // Two independent pairs (x1, y1) and (x2, y2), side by side.
+  auto pair2 = [&](ulonglong2(&x1)[JQ], float& a1, ulonglong2(&y1)[JQ], float& b1, ulonglong2(&x2)[JQ], float& a2,
+                   ulonglong2(&y2)[JQ], float& b2) {
+    float g1 = dot(x1, y1), g2 = dot(x2, y2);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      g1 += __shfl_xor_sync(0xffffffffu, g1, o);
+      g2 += __shfl_xor_sync(0xffffffffu, g2, o);
+    }
+    const float t1 = scalars(g1, a1, b1), t2 = scalars(g2, a2, b2);
+    if (t1 != 0.f || t2 != 0.f) {  // warp-uniform
+      rotate(x1, y1, t1);
+      rotate(x2, y2, t2);
+    }
+  };
   auto colp = [&](int buf, int j) { return reinterpret_cast<ulonglong2*>(js + (size_t)buf * bl + (size_t)j * ld); };
 
   // Cross pairs of the blocks in buffers P and Q.
+  const int H = B / 2;
   auto cross = [&](int P, int Q) {
-    ulonglong2 x[JQ];
-    load_x(x, colp(P, w));
-    float alpha = 0.f;
+    ulonglong2 x1[JQ], x2[JQ];
+    load(x1, colp(P, 2 * w));
+    load(x2, colp(P, 2 * w + 1));
+    float a1 = wsum(dot(x1, x1)), a2 = wsum(dot(x2, x2));
     {
-      f2 g0 = 0ull, g1 = 0ull;
-#pragma unroll
-      for (int e = 0; e < JQ; ++e) {
-        g0 = f2_fma(x[e].x, x[e].x, g0);
-        g1 = f2_fma(x[e].y, x[e].y, g1);
+      const float q1 = sq(colp(Q, 2 * w)), q2 = sq(colp(Q, 2 * w + 1));
+      if (lane == 0) {
+        nrm[Q * B + 2 * w] = q1;
+        nrm[Q * B + 2 * w + 1] = q2;
       }
-      const float2 g = f2_to_float2(f2_add(g0, g1));
-      alpha = wsum(g.x + g.y);
     }
-    const float qn = sq(colp(Q, w));
-    if (lane == 0) nrm[Q * B + w] = qn;
     __syncthreads();
     int q = w;
-    for (int r = 0; r < B; ++r) {
-      pair(x, alpha, colp(Q, q), &nrm[Q * B + q]);
-      if (++q == B) q = 0;
+    for (int r = 0; r < H; ++r) {
+      ulonglong2 y1[JQ], y2[JQ];
+      ulonglong2 *p1 = colp(Q, 2 * q), *p2 = colp(Q, 2 * q + 1);
+      load(y1, p1);
+      load(y2, p2);
+      float2* bn = reinterpret_cast<float2*>(&nrm[Q * B + 2 * q]);
+      float2 b = *bn;
+      pair2(x1, a1, y1, b.x, x2, a2, y2, b.y);
+      pair2(x1, a1, y2, b.y, x2, a2, y1, b.x);
+      store(y1, p1);
+      store(y2, p2);
+      if (lane == 0) *bn = b;
+      if (++q == H) q = 0;
       __syncthreads();
     }
-    store_x(x, colp(P, w));
-    if (lane == 0) nrm[P * B + w] = alpha;
+    store(x1, colp(P, 2 * w));
+    store(x2, colp(P, 2 * w + 1));
   };
-  // Pairs inside both blocks (round robin; warps 0 .. B/2-1 the first block).
+  // Pairs inside both blocks (round robin; each warp one pair of each).
   auto inside = [&](int P, int Q) {
-    {
-      const float pn = sq(colp(P, w)), qn = sq(colp(Q, w));
+    for (int h = 0; h < 2; ++h) {
+      const float pn = sq(colp(P, 2 * w + h)), qn = sq(colp(Q, 2 * w + h));
       if (lane == 0) {
-        nrm[P * B + w] = pn;
-        nrm[Q * B + w] = qn;
+        nrm[P * B + 2 * w + h] = pn;
+        nrm[Q * B + 2 * w + h] = qn;
       }
     }
     __syncthreads();
-    const int buf = w < B / 2 ? P : Q, k = w < B / 2 ? w : w - B / 2;
     for (int r = 0; r < B - 1; ++r) {
-      const int i = k == 0 ? 0 : 1 + (k - 1 + r) % (B - 1);
-      const int j = 1 + (B - 2 - k + r) % (B - 1);
-      ulonglong2 x[JQ];
-      load_x(x, colp(buf, i));
-      float alpha = nrm[buf * B + i];
-      pair(x, alpha, colp(buf, j), &nrm[buf * B + j]);
-      store_x(x, colp(buf, i));
+      const int i = w == 0 ? 0 : 1 + (w - 1 + r) % (B - 1);
+      const int j = 1 + (B - 2 - w + r) % (B - 1);
+      ulonglong2 x1[JQ], y1[JQ], x2[JQ], y2[JQ];
+      load(x1, colp(P, i));
+      load(y1, colp(P, j));
+      load(x2, colp(Q, i));
+      load(y2, colp(Q, j));
+      float a1 = nrm[P * B + i], b1 = nrm[P * B + j], a2 = nrm[Q * B + i], b2 = nrm[Q * B + j];
+      pair2(x1, a1, y1, b1, x2, a2, y2, b2);
+      store(x1, colp(P, i));
+      store(y1, colp(P, j));
+      store(x2, colp(Q, i));
+      store(y2, colp(Q, j));
       __syncwarp();
-      if (lane == 0) nrm[buf * B + i] = alpha;
+      if (lane == 0) {
+        nrm[P * B + i] = a1;
+        nrm[P * B + j] = b1;
+        nrm[Q * B + i] = a2;
+        nrm[Q * B + j] = b2;
+      }
       __syncthreads();
     }
   };
@@ -262,22 +290,26 @@ __global__ void __launch_bounds__(MAXT, 1) k_jacobi_cluster(Args a) {
     // counting rotation needs in the next sweep.
     {
       const int b0 = my(lo, Llo), b1 = my(hi, Lhi);
-      const float n0 = sq(colp(b0, w)), n1 = sq(colp(b1, w));
-      if (lane == 0) {
-        a.nrm[(2 * c) * B + w] = n0;
-        a.nrm[(2 * c + 1) * B + w] = n1;
-        if (mycount) atomicAdd(&a.rot_counts[sweep], mycount);
+      for (int h = 0; h < 2; ++h) {
+        const float n0 = sq(colp(b0, 2 * w + h)), n1 = sq(colp(b1, 2 * w + h));
+        if (lane == 0) {
+          a.nrm[(2 * c) * B + 2 * w + h] = n0;
+          a.nrm[(2 * c + 1) * B + 2 * w + h] = n1;
+        }
       }
+      if (lane == 0 && mycount) atomicAdd(&a.rot_counts[sweep], mycount);
       __threadfence();
       cluster.sync();
       if (__ldcg(&a.rot_counts[sweep]) == 0) break;
       if (a.lead > 0) {
         const int tot = 2 * NC * B;
+        for (int j = threadIdx.x; j < tot; j += NT) all_nrm[j] = __ldcg(&a.nrm[j]);
+        __syncthreads();
         for (int j = threadIdx.x; j < tot; j += NT) {
-          const float v = __ldcg(&a.nrm[j]);
+          const float v = all_nrm[j];
           int rank = 0;
           for (int e = 0; e < tot; ++e) {
-            const float u = __ldcg(&a.nrm[e]);
+            const float u = all_nrm[e];
             rank += (u > v) || (u == v && e < j);
           }
           if (rank == a.lead - 1) *s_th = 0.999f * v;

@@ -307,7 +307,13 @@ int orth_robust(const Dla& d, Arena& ar, bool dry, DT tc, void* X, void* Y, void
     TRY(tall_gemm(d, ar, tc, tc, tc, rows, l, l, X, l, b.Rinv, RinvB, l, Y, l, true,
                   tc == DT::F32 ? static_cast<float*>(Z) : nullptr, &y_t));
     TRY(tall_gram(d, ar, dry, tc, Y, rows, l, Z, b.G, y_t));
-    if (!dry) {
+    // FP64 data: the second Gram is the identity up to the first pass's
+    // rounding times the condition number squared, and the bound keeps the
+    // series' error, the cube of that distance, below FP64 rounding.  (FP32
+    // data are 1e-2 off after one pass at condition numbers of a few hundred.)
+    bool near = false;
+    if (tc == DT::F64) TRY(chol_inv_near_identity(d, ar, b.G, b.LT2, b.Rinv, b.Ug, b.Vg, l, 2e-6, &near));
+    if (!dry && !near) {
       TRY(chol_inv(d, b.G, b.LT2, b.Rinv, b.Ug, b.Vg, l));
       int hs = 0;
       TRY(read_status(d, &hs));
@@ -415,6 +421,62 @@ __global__ void k_upper_to_cols(const double* __restrict__ Z, int64_t l, double*
 // directions that vanish in exact arithmetic are dropped.
 double range_tol(int64_t l) { return (double)l * 0x1.0p-44; }
 
+// The block SRHT whose rows formed a sketch (n = 0: not one, or not known).
+struct OmegaOf {
+  uint64_t seed = 0;
+  int64_t n = 0;
+  int p = 1;
+};
+
+// Indices of one row of Omega out of each class of parallel rows, ascending.
+// Sampling with replacement (Sec. 2) repeats rows: rows j and k agree up to
+// one sign when s_j = s_k and the products of their Dt signs are the same in
+// every block.  About l^2 / 2r pairs share a sample and 2^(1-p) of those are
+// parallel, so the sign words are compared pair by pair.
+std::vector<int> distinct_rows(const OmegaOf& om, int64_t l) {
+  const int64_t rb = (om.n + om.p - 1) / om.p;
+  uint64_t r = 1;
+  while ((int64_t)r < rb) r <<= 1;
+  std::vector<std::pair<uint64_t, int>> at((size_t)l);
+  for (int64_t j = 0; j < l; ++j) at[(size_t)j] = {sample_word(om.seed, (uint64_t)j) & (r - 1), (int)j};
+  std::sort(at.begin(), at.end());
+  std::vector<char> drop((size_t)l, 0);
+  auto bit = [&](int64_t i, int j) {
+    return (int)((sign_word(om.seed, kStreamDt, (uint64_t)i, (uint64_t)(j >> 6)) >> (j & 63)) & 1);
+  };
+  auto parallel = [&](int j, int k) {
+    const int first = bit(0, j) ^ bit(0, k);
+    for (int64_t i = 1; i < om.p; ++i)
+      if ((bit(i, j) ^ bit(i, k)) != first) return false;
+    return true;
+  };
+  for (size_t a = 0; a < at.size(); ++a) {
+    if (drop[(size_t)at[a].second]) continue;
+    for (size_t c = a + 1; c < at.size() && at[c].first == at[a].first; ++c)
+      if (!drop[(size_t)at[c].second] && parallel(at[a].second, at[c].second)) drop[(size_t)at[c].second] = 1;
+  }
+  std::vector<int> keep;
+  for (int64_t j = 0; j < l; ++j)
+    if (!drop[(size_t)j]) keep.push_back((int)j);
+  return keep;
+}
+
+// The columns of the sketch matrix X (rows x *l, type t) that belong to
+// distinct rows of Omega, in place (through tmp); *l becomes their number.
+// The range of X does not change.  idx: l ints of device scratch.
+int drop_parallel_columns(const Dla& d, DT t, void* X, void* tmp, int64_t rows, int64_t* l, const OmegaOf& om,
+                          int* idx) {
+  const std::vector<int> keep = distinct_rows(om, *l);
+  const int64_t lk = (int64_t)keep.size();
+  if (lk == *l) return BSRHT_OK;
+  BSRHT_CUDA_TRY(cudaMemcpyAsync(idx, keep.data(), sizeof(int) * (size_t)lk, cudaMemcpyHostToDevice, d.s));
+  TRY(gather_columns(d, t, X, rows, *l, idx, lk, tmp));
+  BSRHT_CUDA_TRY(cudaMemcpyAsync(X, tmp, dt_size(t) * (size_t)rows * (size_t)lk, cudaMemcpyDeviceToDevice, d.s));
+  BSRHT_CUDA_TRY(cudaStreamSynchronize(d.s));  // `keep` is pageable host memory
+  *l = lk;
+  return BSRHT_OK;
+}
+
 // Orthonormal basis Q of the numerical range of the FP64 sketch matrix X
 // (rows x l), Algorithm 1 step 2: range(Q) = range(Y).  Sampling with
 // replacement (Sec. 2) lets Omega repeat a row up to sign in every block;
@@ -426,18 +488,31 @@ double range_tol(int64_t l) { return (double)l * 0x1.0p-44; }
 // cutoff (every direction kept, r' = l).  Otherwise: Householder QR
 // X = Qh R, one-sided Jacobi SVD R = Ur S Vr^T (FP64), and
 // Q = Qh Ur[:, :r'] with r' the count of sigma > tau sigma_1.
+// When the fast path declines a sketch whose Omega is known (om), its columns
+// of repeated rows of Omega are dropped first (they add nothing to the range)
+// and the fast path tried again: repeated rows are what singular sketches of
+// well-conditioned data come from.
 // Buffers: X (input, overwritten), Y and Z (rows x l scratch).  On return
 // *Qout (rows x r', leading dimension r') and *rank = r'; reads r' back on
 // the stream.  In dry mode both paths are measured and r' = l.
 int range_basis(const Dla& d, Arena& ar, bool dry, double* X, double* Y, double* Z, int64_t rows, int64_t l,
-                uint64_t seed, const OrthBufs& b, double** Qout, int64_t* rank) {
+                uint64_t seed, const OrthBufs& b, double** Qout, int64_t* rank, const OmegaOf& om = OmegaOf()) {
   *rank = l;
+  const double cut_rel = range_tol(l);
   void* Qv = nullptr;
   bool declined = false;
   TRY(orth_robust(d, ar, dry, DT::F64, X, Y, Z, rows, l, seed, b, nullptr, true, false, &Qv, nullptr, false,
                   &declined));
+  if (!dry && declined && om.n > 0) {
+    const int64_t l_all = l;
+    TRY(drop_parallel_columns(d, DT::F64, X, Z, rows, &l, om, reinterpret_cast<int*>(b.sc)));
+    if (l < l_all)
+      TRY(orth_robust(d, ar, dry, DT::F64, X, Y, Z, rows, l, seed, b, nullptr, true, false, &Qv, nullptr, false,
+                      &declined));
+  }
   if (!dry && !declined) {
     *Qout = static_cast<double*>(Qv);
+    *rank = l;
     return BSRHT_OK;
   }
   // Householder QR of a copy of X: Z holds R (upper triangle of its first
@@ -459,7 +534,7 @@ int range_basis(const Dla& d, Arena& ar, bool dry, double* X, double* Y, double*
     // the rank rule's tau (against ||R||_F) are numerically zero for the
     // Jacobi too: they hold the rounding of the sketch (about 2^-45 of its
     // scale for FP64 data) and would otherwise keep the sweeps going.
-    TRY(jacobi_svd(d, ar, b.G, l, b.Ug, b.lam, b.Vg, 0.0, range_tol(l)));
+    TRY(jacobi_svd(d, ar, b.G, l, b.Ug, b.lam, b.Vg, 0.0, cut_rel));
     ar.release(mk);
   }
   int64_t r = l;
@@ -470,7 +545,7 @@ int range_basis(const Dla& d, Arena& ar, bool dry, double* X, double* Y, double*
     TRY(read_status(d, &hs));
     if (hs) return status_to_code(hs) != BSRHT_OK ? status_to_code(hs) : BSRHT_ENOCONV;
     r = 0;
-    const double cut = range_tol(l) * sig[0];
+    const double cut = cut_rel * sig[0];
     for (int64_t c = 0; c < l; ++c)
       if (sig[0] > 0.0 && sig[c] > cut) ++r;
   }
@@ -528,6 +603,10 @@ int rsvd_impl(const bsrht_opts& o, const void* A, int64_t n, int64_t m, int k, i
   // kCholQrPivotMin32) and only V = Q U~_k is made orthonormal in FP64 at
   // the end (an m x k CholeskyQR2).  Otherwise, and for FP64 data: the
   // rank-revealing FP64 basis (range_basis).
+  // A sketch that CholeskyQR2 declines loses the columns of repeated rows of
+  // Omega first (drop_parallel_columns).
+  OmegaOf om;
+  if (o.variant != BSRHT_VARIANT_GAUSSIAN) om = OmegaOf{seed, n, p};
   double* Q = nullptr;
   int64_t lq = l;
   const void* Qa = nullptr;
@@ -539,8 +618,17 @@ int rsvd_impl(const bsrht_opts& o, const void* A, int64_t n, int64_t m, int k, i
     bool declined = false;
     TRY(orth_robust(d, ar, dry, DT::F32, Y32, X3, Qc, m, l, seed ^ 0x51ull, ob, nullptr, true, false, &Qv, nullptr,
                     false, &declined));
+    if (!dry && declined && om.n > 0) {
+      TRY(drop_parallel_columns(d, DT::F32, Y32, X3, m, &lq, om, reinterpret_cast<int*>(ob.sc)));
+      if (lq < l)
+        TRY(orth_robust(d, ar, dry, DT::F32, Y32, X3, Qc, m, lq, seed ^ 0x51ull, ob, nullptr, true, false, &Qv,
+                        nullptr, false, &declined));
+      // V below is made orthonormal in FP64 only when k columns are there.
+      declined = declined || lq < k;
+      if (declined) lq = l;
+    }
     if (!dry && !declined) {
-      TRY(cast_copy(d, DT::F32, Qv, DT::F64, X1, m * l));
+      TRY(cast_copy(d, DT::F32, Qv, DT::F64, X1, m * lq));
       Q = X1;
       Qa = Qv;
       q32 = true;
@@ -548,7 +636,7 @@ int rsvd_impl(const bsrht_opts& o, const void* A, int64_t n, int64_t m, int k, i
   }
   if (!q32) {
     if (!dry) TRY(transpose_cast(d, tc, B, l, m, m, DT::F64, X1, l));
-    TRY(range_basis(d, ar, dry, X1, X2, X3, m, l, seed ^ 0x51ull, ob, &Q, &lq));
+    TRY(range_basis(d, ar, dry, X1, X2, X3, m, l, seed ^ 0x51ull, ob, &Q, &lq, om));
   }
   if (!dry) trace_mark(d.s, "orth_sketch");
   // Below the numerical rank of Y the factors are zero (lq < k).
@@ -758,7 +846,7 @@ int srsvd_impl(const bsrht_opts& o, const void* A, int64_t n, int64_t m, int k, 
   // keep the rank-robust CholeskyQR2 basis of X (rp = l).
   double* Q = nullptr;
   int64_t rq = l, rp = l;
-  TRY(range_basis(d, ar, dry, Y1, Y2, Y3, m, l, seed ^ 0x61ull, ob, &Q, &rq));
+  TRY(range_basis(d, ar, dry, Y1, Y2, Y3, m, l, seed ^ 0x61ull, ob, &Q, &rq, OmegaOf{s_om, n, p}));
   void* Pv = nullptr;
   if (tc == DT::F64) {
     double* P64 = nullptr;
