@@ -1056,8 +1056,11 @@ __global__ void k_scale_norms(const double* __restrict__ C, int64_t n, double* _
 // the norms are, so small columns are made orthogonal to their own accuracy.
 // Pairs with |X_ij| > 0.03 (clustered singular values) are left alone.
 // Flags: see above; a pair exceeds by the test of a Jacobi sweep (k_jacobi).
+// Only pairs with one of the first `lead` columns (the caller's triplets, of
+// columns by descending norm) set flags: the others need not be orthogonal
+// among themselves.
 __global__ void k_refine_generator(const double* __restrict__ C, const double* __restrict__ sig, int64_t n,
-                                   const double* __restrict__ fnorm, double tiny_rel, double tol,
+                                   const double* __restrict__ fnorm, double tiny_rel, double tol, int64_t lead,
                                    double* __restrict__ X, double* __restrict__ Z, int* __restrict__ flags) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n * n) return;
@@ -1070,7 +1073,7 @@ __global__ void k_refine_generator(const double* __restrict__ C, const double* _
     const double ni = C[i * n + i], nj = C[j * n + j];
     const double si = sig[i] * sqrt(ni), sj = sig[j] * sqrt(nj);
     if (!(si <= tiny && sj <= tiny) && g != 0.0) {
-      const bool exceeds = !(g * g <= tol * tol * ni * nj);
+      const bool exceeds = (i < lead || j < lead) && !(g * g <= tol * tol * ni * nj);
       // Ratio of the smaller norm to the larger one: no overflow, no
       // difference of squares.
       const bool up = sj >= si;
@@ -1758,6 +1761,7 @@ int jacobi_svd(const Dla& d, Arena& ar, double* colsM, int64_t l, double* U, dou
     TRY_DLA(form_y());
     trace_mark(d.s, "svd_orthogonalize");
     const double tiny_rel = std::max((double)l * 0x1.0p-53, zero_rel);
+    const int64_t wanted = ktop > 0 ? std::min(s, with_margin(ktop)) : s;
     const unsigned lb = blocks_for(l * s, 256);
     double* U1 = Y;    // normalised columns of Y
     double* U2 = Ux;   // Y's other buffer
@@ -1783,7 +1787,7 @@ int jacobi_svd(const Dla& d, Arena& ar, double* colsM, int64_t l, double* U, dou
     bool converged = false;
     for (int it = 0; it < 8; ++it) {
       TRY_DLA(gemm_f64(s, s, l, U1, s, true, U1, s, G, s, true));
-      k_refine_generator<<<sb, 256, 0, d.s>>>(G, sigS, s, fnorm, tiny_rel, tol, Xg, Zg, cflag);
+      k_refine_generator<<<sb, 256, 0, d.s>>>(G, sigS, s, fnorm, tiny_rel, tol, wanted, Xg, Zg, cflag);
       DLA_LAUNCH_CHECK();
       note_launches(1);
       TRY_DLA(read_flags());

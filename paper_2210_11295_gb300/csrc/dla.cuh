@@ -98,7 +98,10 @@ int chol_inv_near_identity(const Dla& d, Arena& ar, double* g, double* LT, doubl
 // max(16, ktop / 4)) leading columns of the FP32 phase are polished in FP64
 // (the SVD of M restricted to their span, which differs from the leading
 // triplets of M in second order of the FP32 phase's residual cosines);
-// ranks s and beyond hold the FP32 phase's estimates.  keep_rel > 0 with
+// ranks s and beyond hold the FP32 phase's estimates (and U columns that may
+// be zero).  ktop > 0 without polish_tol: FP64 accuracy for the ktop leading
+// triplets; the columns of U beyond them need not be orthogonal to one
+// another.  keep_rel > 0 with
 // polish_tol > 0 and ktop = 0 (a caller that keeps the triplets with
 // sigma > keep_rel sigma_1): s = c + max(16, c / 4) with c the FP32 phase's
 // count above that threshold.  colsM is overwritten in every case.

@@ -671,14 +671,13 @@ int rsvd_impl(const bsrht_opts& o, const void* A, int64_t n, int64_t m, int k, i
   if (!dry) trace_mark(d.s, "tall_qr");
   // Step 5: SVD of R = V~ Sigma~ U~^T (R^T = U~ Sigma~ V~^T), Jacobi on the
   // columns of R: its right factor, orthogonal to FP64 rounding, is U~, which
-  // Q multiplies below.  FP32 data: the polish stops at cosines of
-  // polish_tol_fp32(lq) and on the k leading triplets; the other factor V~
+  // Q multiplies below.  Only the k leading triplets are used.  FP32 data:
+  // the polish stops at cosines of polish_tol_fp32(lq); the other factor V~
   // meets P, itself orthogonal only to FP32 accuracy.
   {
     const size_t mk = ar.mark();
     if (!dry) TRY(transpose_lower_to_upper(d, R, RT, lq));
-    TRY(jacobi_svd(d, ar, RT, lq, Vs, sig, Us, tc == DT::F32 ? polish_tol_fp32(lq) : 0.0, 0.0,
-                   tc == DT::F32 ? k : 0));
+    TRY(jacobi_svd(d, ar, RT, lq, Vs, sig, Us, tc == DT::F32 ? polish_tol_fp32(lq) : 0.0, 0.0, k));
     ar.release(mk);
   }
   if (!dry) trace_mark(d.s, "small_svd");
@@ -1105,7 +1104,7 @@ int nystrom_impl(const bsrht_opts& o, const void* A, int64_t n, int k, int64_t l
   // ||Y||, below the precision of the fixed-point FP64 sketch (an address
   // the TMA rules reject steers the plan to it, as for grouped sketches).
   TRY(sketch_make_plan(sp_y, BSRHT_F64, BSRHT_VARIANT_CUDACORE, n, l, l, p, l, !dry,
-                       reinterpret_cast<const void*>(uintptr_t(1))));
+                       kPlainSketchOnly));
   const int64_t rb = sp_a.rb, r = sp_a.r;
   Dla d{static_cast<cudaStream_t>(o.stream), nullptr};
   d.status = static_cast<int*>(ar.take(sizeof(int)));
@@ -1268,8 +1267,7 @@ int nystrom_impl(const bsrht_opts& o, const void* A, int64_t n, int k, int64_t l
   }
   {
     const size_t mk = ar.mark();
-    TRY(jacobi_svd(d, ar, RT, lr, Us, sig, Vs, tc == DT::F32 ? polish_tol_fp32(lr) : 0.0, 0.0,
-                   tc == DT::F32 ? k : 0));
+    TRY(jacobi_svd(d, ar, RT, lr, Us, sig, Vs, tc == DT::F32 ? polish_tol_fp32(lr) : 0.0, 0.0, k));
     ar.release(mk);
   }
   if (!dry) trace_mark(d.s, "small_svd");

@@ -26,6 +26,7 @@ struct SketchPlan {
   int64_t P = 0;      // column panels
   int64_t T = 0;      // tiles = P * C
   int G = 0;          // CTAs of the chunked kernel (persistent, one wave)
+  int rows = 0;       // path 2: rows off 16 bytes, copied row by row
   int paired = 0;     // TMA-fed paths: CTA pairs share panel pairs (16-bit inputs)
   int64_t jgroup = 0; // sketch rows handled per launch
   size_t smem = 0;    // dynamic shared memory per CTA
@@ -34,6 +35,9 @@ struct SketchPlan {
   size_t dttab_bytes = 0; // paths 2, 5: Dt^(i) sign table (one sketch-row group)
   size_t work_bytes = 0;  // total scratch
 };
+
+// Given for A, plans the chunked kernel (an address no matrix has).
+inline const void* const kPlainSketchOnly = reinterpret_cast<const void*>(uintptr_t(1));
 
 // Fills plan for the given sizes; returns a bsrht status. When
 // query_device is false, no CUDA call is made and G is an upper bound.
