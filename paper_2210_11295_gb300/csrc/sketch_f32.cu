@@ -1,6 +1,7 @@
 // K1 sketch instances with FP32 arithmetic: A in f32, bf16 or f16.
 #include <algorithm>
 
+#include "launch.cuh"
 #include "sketch.cuh"
 #include "sketch_kernels.cuh"
 
@@ -52,11 +53,13 @@ int occ_of() {
   using S = K1Shape<Tin, float, kW32, NT, R2, JM>;
   auto kern = k_sketch_chunked<Tin, float, kW32, NT, R2, JM>;
   const size_t smem = S::smem_bytes();
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return 0;
-  int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem) != cudaSuccess) return 0;
-  return occ;
+  static DeviceCache cache;
+  return std::max(0, cache.get([&] {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem) != cudaSuccess) return -1;
+    return occ;
+  }));
 }
 
 template <typename Tin>

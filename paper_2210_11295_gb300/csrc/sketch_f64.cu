@@ -1,6 +1,7 @@
 // K1 sketch instances with FP64 arithmetic (A in f64).
 #include <algorithm>
 
+#include "launch.cuh"
 #include "sketch.cuh"
 #include "sketch_kernels.cuh"
 
@@ -30,11 +31,13 @@ int occ_of() {
   using S = K1Shape<double, double, kW64, NT, R2, JM>;
   auto kern = k_sketch_chunked<double, double, kW64, NT, R2, JM>;
   const size_t smem = S::smem_bytes();
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return 0;
-  int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem) != cudaSuccess) return 0;
-  return occ;
+  static DeviceCache cache;
+  return std::max(0, cache.get([&] {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem) != cudaSuccess) return -1;
+    return occ;
+  }));
 }
 
 

@@ -46,6 +46,13 @@ static bool tma_layout_ok(int dtype, const void* A, int64_t lda) {
   return A == nullptr || (reinterpret_cast<uintptr_t>(A) % 16) == 0;
 }
 
+// FP32 and 16-bit rows off 16 bytes, which the same kernel copies row by row.
+static bool rows_layout_ok(int dtype, const void* A, int64_t lda) {
+  if (dtype != BSRHT_F32 && dtype != BSRHT_BF16 && dtype != BSRHT_F16) return false;
+  if (A == kPlainSketchOnly || tma_layout_ok(dtype, A, lda)) return false;
+  return reinterpret_cast<uintptr_t>(A) % dtype_size(dtype) == 0;
+}
+
 // 16-bit panels are 64-byte rows: pair the panels (TileSched) when there are
 // at least two CTAs and two panels; sizes the partial-sum scratch.
 static void set_pairing(SketchPlan& pl) {
@@ -63,7 +70,7 @@ static int make_plan_tma(SketchPlan& pl, bool query_device) {
   pl.W = 32;
   pl.NT = 512;
   pl.R2 = 512;
-  pl.JM = pl.l <= 512 ? 32 : pl.l <= 768 ? 48 : 64;
+  pl.JM = pl.l <= 512 ? 32 : pl.l <= 768 && !pl.rows ? 48 : 64;
   pl.NRL = pl.NT / pl.W;
   pl.jgroup = std::min<int64_t>(pl.l, (int64_t)pl.JM * pl.NRL);
   pl.nch = (pl.rb + pl.R2 - 1) / pl.R2;
@@ -248,11 +255,17 @@ static int make_plan_choice(SketchPlan& pl, int dtype, int64_t n, int64_t m, int
   // unless a chunked instance was chosen; the plain kernel stays the
   // fallback, so a plan made without A reserves scratch for both.
   // (The TMA kernels count a panel's chunks in 32 bits.)
-  const bool tma_ok = pl.r >= 512 && tma_layout_ok(dtype, A, lda) && (int64_t)p * ((pl.rb + 511) / 512) < INT32_MAX;
+  // FP32 and 16-bit rows off 16 bytes take the same kernel with row copies.
+  // FP64 ones stay with the chunked kernel, whose FP64 adds are more exact than
+  // fixed point.
+  const bool big = pl.r >= 512 && (int64_t)p * ((pl.rb + 511) / 512) < INT32_MAX;
+  const bool rows = big && rows_layout_ok(dtype, A, lda);
+  const bool tma_ok = (big && tma_layout_ok(dtype, A, lda)) || rows;
   if (choice == -1 && !(tma_ok || (A == nullptr && pl.r >= 512 && tma_layout_ok(dtype, nullptr, lda))))
     return BSRHT_EINVAL;
   if (tma_ok && choice < 0) {
     SketchPlan t = pl;
+    t.rows = rows ? 1 : 0;
     if (f64)
       make_plan_f64x(t, query_device);
     else
@@ -427,7 +440,6 @@ int sketch_run(const SketchPlan& pl, const void* A, uint64_t seed, void* out, in
       int* err = reinterpret_cast<int*>(w + pl.part_bytes);
       uint64_t* dtab = reinterpret_cast<uint64_t*>(w + pl.part_bytes + 256);
       uint64_t* dttab = reinterpret_cast<uint64_t*>(w + pl.part_bytes + 256 + pl.dtab_bytes);
-      if (j0 == 0) BSRHT_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), stream));
       st = pl.path == 5 ? sketch_launch_f64x(pl, a, out, ldo, err, dtab, dttab, stream)
                         : sketch_launch_tma(pl, a, out, ldo, err, dtab, dttab, stream);
     } else {
@@ -451,7 +463,7 @@ int sketch_make_plan_grouped(SketchPlan& pl, int dtype, int64_t n, int64_t m, in
     // Same sizes through the plain kernel: plan with an address the TMA
     // rules reject (odd), which only steers the path choice.
     st = sketch_make_plan(pl, dtype, BSRHT_VARIANT_CUDACORE, n, m, lda, p, l, true,
-                          reinterpret_cast<const void*>(uintptr_t(1)));
+                          kPlainSketchOnly);
     if (st != BSRHT_OK) return st;
   }
   if (pl.path != 0 || pl.jgroup < pl.l) return BSRHT_EUNSUP;

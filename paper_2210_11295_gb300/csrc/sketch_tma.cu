@@ -17,10 +17,21 @@
 // guarded by mbarriers, so HBM reads of later chunks overlap the butterflies
 // and the gather of the current one.  FP32 inputs are transformed in place
 // in the staged chunk; 16-bit inputs are widened into a separate FP32 tile.
+//
+// Rows off 16 bytes (ROWS), which tensor maps refuse: all threads copy the
+// chunk with 16-byte cp.async of the aligned windows that hold its rows (144
+// bytes of FP32, 80 of a 16-bit type; nine or five copies a thread), and a
+// thread adds its rows' common offset in the window to its addresses (its
+// rows are 16 apart, so the offset is the same for all).  A chunk with a
+// window that would leave the matrix (its first or last rows) is loaded
+// element by element.  (One untiled cp.async.bulk per row took 2.55 ms where
+// this takes 0.55 at 300007 x 1250 FP32, l = 300, and the chunked kernel,
+// whose loads do not overlap its butterflies, 1.00.)
 #include <algorithm>
 #include <mutex>
 
 #include "common.cuh"
+#include "launch.cuh"
 #include "sketch.cuh"
 #include "trace.cuh"
 #include "sketch_kernels.cuh"
@@ -41,7 +52,7 @@ constexpr int stages_for() {
   return sizeof(Tin) == 4 ? 3 : 4;
 }
 
-template <typename Tin, int W, int NT, int R2, int JM, int STAGES>
+template <typename Tin, int W, int NT, int R2, int JM, int STAGES, bool ROWS>
 struct TmaShape {
   static constexpr int NRL = NT / W;
   static constexpr int E = R2 / NRL;
@@ -49,7 +60,10 @@ struct TmaShape {
   static constexpr int JG = JM * NRL;
   static constexpr bool kInPlace = sizeof(Tin) == 4;
   static constexpr int BOXR = R2 < 256 ? R2 : 256;
-  static constexpr size_t stage_bytes = sizeof(Tin) * (size_t)R2 * W;
+  static constexpr int SP = ROWS ? W + 16 / (int)sizeof(Tin) : W;  // row pitch of a stage
+  static constexpr int TP = kInPlace ? SP : W;                     // and of the FP32 tile
+  static constexpr uint32_t ROW_BYTES = SP * sizeof(Tin);
+  static constexpr size_t stage_bytes = sizeof(Tin) * (size_t)R2 * SP;
   static constexpr size_t tile_bytes = kInPlace ? 0 : sizeof(float) * (size_t)R2 * W;
   static constexpr size_t meta_bytes = 2 * sizeof(uint32_t) * JG + sizeof(uint64_t) * STAGES + 16;
   static constexpr size_t smem_bytes() { return STAGES * stage_bytes + tile_bytes + meta_bytes + 128; }
@@ -88,8 +102,10 @@ __device__ __forceinline__ float widen(Tin v) {
 // the D^(i) sign of row rl + 16e of chunk a of block i (the 32 rows a thread
 // of row lane rl owns); dttab holds the Dt^(i) words of the launch's sketch
 // rows.
+// Clears *err first when `clear`.
 __global__ void k_sign_tables(uint64_t seed, int p, int64_t nch, int64_t j0, int64_t tw, uint32_t* __restrict__ dmtab,
-                              uint64_t* __restrict__ dttab) {
+                              uint64_t* __restrict__ dttab, int* __restrict__ err, int clear) {
+  if (clear && blockIdx.x == 0 && threadIdx.x == 0) *err = 0;
   const int64_t nm = (int64_t)p * nch * 16;
   const int64_t total = nm + (int64_t)p * tw;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -111,18 +127,18 @@ __global__ void k_sign_tables(uint64_t seed, int p, int64_t nch, int64_t j0, int
   }
 }
 
-template <typename Tin, int W, int NT, int R2, int JM, int STAGES>
+template <typename Tin, int W, int NT, int R2, int JM, int STAGES, bool ROWS>
 __global__ void __launch_bounds__(NT, 1)
     k_sketch_tma(const __grid_constant__ CUtensorMap tmap, SketchArgs g, const uint32_t* __restrict__ dmtab,
                  const uint64_t* __restrict__ dttab, int64_t tw, int* __restrict__ err) {
-  using S = TmaShape<Tin, W, NT, R2, JM, STAGES>;
-  constexpr int NRL = S::NRL, E = S::E, JG = S::JG, BOXR = S::BOXR;
+  using S = TmaShape<Tin, W, NT, R2, JM, STAGES, ROWS>;
+  constexpr int NRL = S::NRL, E = S::E, JG = S::JG, BOXR = S::BOXR, SP = S::SP, TP = S::TP;
   static_assert(W == 32 && NRL == 16 && E == 32 && R2 == 512, "sign masks assume 16 row lanes x 32 rows");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char* base = smem_raw + ((128 - (reinterpret_cast<uintptr_t>(smem_raw) & 127)) & 127);
-  Tin* stage = reinterpret_cast<Tin*>(base);                                   // [STAGES][R2][W]
+  Tin* stage = reinterpret_cast<Tin*>(base);                                   // [STAGES][R2][SP]
   float* tile_sep = reinterpret_cast<float*>(base + STAGES * S::stage_bytes);  // [R2][W] (16-bit inputs)
-  uint32_t* s_off = reinterpret_cast<uint32_t*>(base + STAGES * S::stage_bytes + S::tile_bytes);  // s_lo * W
+  uint32_t* s_off = reinterpret_cast<uint32_t*>(base + STAGES * S::stage_bytes + S::tile_bytes);  // s_lo * TP
   uint32_t* s_hi = s_off + JG;
   uint64_t* bar = reinterpret_cast<uint64_t*>(s_hi + JG);
   uint32_t* tm_slot = reinterpret_cast<uint32_t*>(bar + STAGES);  // TMEM base address (JM = 64)
@@ -161,11 +177,48 @@ __global__ void __launch_bounds__(NT, 1)
     it.step = sched.step;
     return it;
   };
-  TileIt iss = tile_at(t_begin);  // next tile to issue (thread 0 only)
+  TileIt iss = tile_at(t_begin);  // next tile to issue (thread 0; every thread with ROWS)
   int64_t issued = 0;
-  auto issue_next = [&]() {  // TMA for the CTA's next tile into stage issued % STAGES
+  const uint32_t abase = (uint32_t)(reinterpret_cast<uintptr_t>(g.A) / sizeof(Tin));
+  constexpr uint32_t kUnit = 16 / sizeof(Tin);  // elements per 16 bytes
+  constexpr int kIssuers = ROWS ? NT : 1;
+  auto issue_next = [&]() {  // the CTA's next tile into stage issued % STAGES
     const int s = (int)(issued % STAGES);
-    Tin* dst = stage + (size_t)s * R2 * W;
+    Tin* dst = stage + (size_t)s * R2 * SP;
+    if constexpr (ROWS) {
+      // Warp w copies rows 32 w .. 32 w + 31, NP pieces of 16 bytes each.
+      constexpr int NP = (int)S::ROW_BYTES / 16;
+      const Tin* A = static_cast<const Tin*>(g.A);
+      const int64_t row0 = iss.i * g.rb + iss.a * R2, col0 = iss.pc * W;
+      const int64_t rows_i = min(g.rb, g.n - iss.i * g.rb);
+      const int cnt = (int)max((int64_t)0, min((int64_t)R2, rows_i - iss.a * R2));
+      const uintptr_t a0 = reinterpret_cast<uintptr_t>(A + row0 * g.lda + col0);
+      const uint64_t ldb = (uint64_t)g.lda * sizeof(Tin);
+      const uintptr_t end = reinterpret_cast<uintptr_t>(A + (g.n - 1) * g.lda + g.m);
+      // Windows are ascending: the first and the last tell for all.
+      const bool inside = (a0 & ~(uintptr_t)15) >= reinterpret_cast<uintptr_t>(A) &&
+                          (cnt == 0 || ((a0 + (uint64_t)(cnt - 1) * ldb) & ~(uintptr_t)15) + S::ROW_BYTES <= end);
+      const int r0 = 32 * (tid >> 5), ln = tid & 31;
+      if (inside) {
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+          const int u = ln + 32 * q, r = r0 + u / NP, piece = u % NP;
+          if (r < cnt)
+            copy16_async(reinterpret_cast<unsigned char*>(dst) + r * S::ROW_BYTES + 16 * piece,
+                         ((a0 + (uint64_t)r * ldb) & ~(uintptr_t)15) + 16 * piece);
+        }
+        mbar_arrive_on_copies(&bar[s]);
+      } else {
+        for (int r = r0; r < r0 + 32 && r < cnt; ++r) {
+          const int off = (int)((abase + (uint32_t)(row0 + r) * (uint32_t)g.lda) & (kUnit - 1));
+          if (col0 + ln < g.m) dst[r * SP + off + ln] = A[(row0 + r) * g.lda + col0 + ln];
+        }
+        mbar_arrive_one(&bar[s]);
+      }
+      iss.next(g.nch, g.p);
+      ++issued;
+      return;
+    }
     mbar_arrive_expect_tx(&bar[s], (uint32_t)S::stage_bytes);
     const int32_t x = (int32_t)(iss.pc * W);
     const int64_t y0 = iss.i * g.rb + iss.a * R2;
@@ -177,14 +230,14 @@ __global__ void __launch_bounds__(NT, 1)
   };
 
   if (tid == 0) {
-    for (int s = 0; s < STAGES; ++s) mbar_init(&bar[s], 1);
+    for (int s = 0; s < STAGES; ++s) mbar_init(&bar[s], kIssuers);
     fence_mbar_init();
   }
   for (int jl = tid; jl < JG; jl += NT) {
     uint32_t off = 0, hi = 0;
     if (jl < jn) {
       const uint64_t sv = sample_word(g.seed, (uint64_t)(g.j0 + jl)) & (uint64_t)(g.r - 1);
-      off = (uint32_t)(sv & (R2 - 1)) * W;
+      off = (uint32_t)(sv & (R2 - 1)) * TP;
       hi = (uint32_t)(sv >> S::LOG_R2);
     }
     s_off[(jl % 32) * (JM / 2) + jl / 32] = off;  // [row lane rg][u]: jl = rg + 32 u
@@ -211,7 +264,7 @@ __global__ void __launch_bounds__(NT, 1)
     tc::tc_fence_after();
     tm_addr = *tm_slot + ((uint32_t)(32 * ((tid >> 5) & 3)) << 16) + 64u * (uint32_t)(tid >> 7);
   }
-  if (tid == 0)
+  if (tid < kIssuers)
     for (int64_t k = 0; k < STAGES && k < ntiles; ++k) issue_next();
 
   // Exchange phase and gather: thread = (row lane rg = tid / 16, column
@@ -232,12 +285,26 @@ __global__ void __launch_bounds__(NT, 1)
   int hcur = 0;  // (JM = 64) the half of the sketch rows whose accumulators are in registers
   int64_t cur_pc = -1;
   float* part = static_cast<float*>(g.part);
+  // With ROWS the sums go to the slot every kFlush chunks and start anew there:
+  // the chunked kernel in whose place it stands sums over three times as many
+  // CTAs, and one FP32 sum over all of a CTA's chunks would round more.
+  constexpr int kFlush = 32;
+  bool written = false;  // the panel's slot holds a sum already
+  int since = 0;
   auto flush_rows = [&](int64_t pc, int ubase) {  // sketch rows rg + 32 (ubase + u)
     float* dst = part + sched.slot(pc) * (int64_t)jn * W + 2 * cp;
 #pragma unroll
     for (int u = 0; u < JR; ++u) {
       const int jl = rg + 32 * (ubase + u);
-      if (jl < jn) *reinterpret_cast<float2*>(dst + (int64_t)jl * W) = make_float2(acc[u][0], acc[u][1]);
+      if (jl < jn) {
+        float2* d = reinterpret_cast<float2*>(dst + (int64_t)jl * W);
+        float2 v = make_float2(acc[u][0], acc[u][1]);
+        if (ROWS && written) {
+          const float2 o = *d;
+          v = make_float2(o.x + v.x, o.y + v.y);
+        }
+        *d = v;
+      }
     }
   };
   auto flush = [&](int64_t pc) {
@@ -272,8 +339,12 @@ __global__ void __launch_bounds__(NT, 1)
   int s = 0;
   uint32_t parity = 0;
   for (int64_t k = 0; k < ntiles; ++k) {
-    if (new_panel) {
-      if (cur_pc >= 0) flush(cur_pc);
+    if (new_panel || (ROWS && since == kFlush)) {
+      if (cur_pc >= 0) {
+        flush(cur_pc);
+        written = !new_panel;
+        since = 0;
+      }
 #pragma unroll
       for (int u = 0; u < JR; ++u) acc[u][0] = acc[u][1] = 0.f;
       if constexpr (kTm) tc::tmem_st32(tm_addr + 32u * (uint32_t)(1 - hcur), accv);
@@ -316,27 +387,32 @@ __global__ void __launch_bounds__(NT, 1)
     }
     const bool ok = mbar_wait_bounded(&bar[s], parity, kWaitLimit);
 
-    Tin* st = stage + (size_t)s * R2 * W;
+    Tin* st = stage + (size_t)s * R2 * SP;
     float* tile = S::kInPlace ? reinterpret_cast<float*>(st) : tile_sep;
     // Register phase: rows rl + NRL*e, D^(i) signs, high log2(E) bits.
     float v[E];
+    int sh = 0;  // ROWS: this thread's rows start here in their windows
+    if constexpr (ROWS)
+      sh = (int)((abase + ((uint32_t)i * (uint32_t)g.rb + (uint32_t)a * R2 + (uint32_t)rl) * (uint32_t)g.lda) &
+                 (kUnit - 1));
     if (nvalid == R2) {
 #pragma unroll
       for (int e = 0; e < E; ++e) {
-        const float x = widen<Tin>(st[(rl + NRL * e) * W + cg]);
+        const float x = widen<Tin>(st[(rl + NRL * e) * SP + cg + sh]);
         v[e] = __int_as_float(__float_as_int(x) ^ (int)((dmask << (31 - e)) & 0x80000000u));
       }
     } else {
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const int rr = rl + NRL * e;
-        const float x = rr < nvalid ? widen<Tin>(st[rr * W + cg]) : 0.f;
+        const float x = rr < nvalid ? widen<Tin>(st[rr * SP + cg + sh]) : 0.f;
         v[e] = __int_as_float(__float_as_int(x) ^ (int)((dmask << (31 - e)) & 0x80000000u));
       }
     }
     fwht_regs<float, E>(v);
+    if constexpr (ROWS && S::kInPlace) __syncwarp();  // a row is read, shifted, by the warp that rewrites it
 #pragma unroll
-    for (int e = 0; e < E; ++e) tile[(rl + NRL * e) * W + cg] = v[e];
+    for (int e = 0; e < E; ++e) tile[(rl + NRL * e) * TP + cg] = v[e];
     // One barrier both publishes the register phase and makes a failed
     // (bounded) wait CTA-uniform: data read after a failed wait is garbage
     // but nothing reaches global memory before this check.
@@ -359,8 +435,8 @@ __global__ void __launch_bounds__(NT, 1)
     // In place (FP32): every thread has finished the previous chunk, so its
     // stage is free; refill it (the 16-bit path refills at the chunk end).
     if constexpr (S::kInPlace) {
-      if (tid == 0 && k >= 1 && issued < ntiles) {
-        fence_proxy_async_smem();
+      if (tid < kIssuers && k >= 1 && issued < ntiles) {
+        if constexpr (!ROWS) fence_proxy_async_smem();
         issue_next();
       }
     }
@@ -369,15 +445,15 @@ __global__ void __launch_bounds__(NT, 1)
     // pairs load and store without re-pairing registers).
     {
       f2 w[NRL];
-      float* tp = tile + (NRL * rg) * W + 2 * cp;
+      float* tp = tile + (NRL * rg) * TP + 2 * cp;
 #pragma unroll
-      for (int b = 0; b < NRL; ++b) w[b] = *reinterpret_cast<const f2*>(tp + b * W);
+      for (int b = 0; b < NRL; ++b) w[b] = *reinterpret_cast<const f2*>(tp + b * TP);
       fwht_regs2<NRL>(w);
 #pragma unroll
-      for (int b = 0; b < NRL; ++b) *reinterpret_cast<f2*>(tp + b * W) = w[b];
+      for (int b = 0; b < NRL; ++b) *reinterpret_cast<f2*>(tp + b * TP) = w[b];
     }
     __syncthreads();
-    // Sampled rows (offsets s_lo * W) with the signs of gmask, two columns per load.
+    // Sampled rows (offsets s_lo * TP) with the signs of gmask, two columns per load.
     const float* tq = tile + 2 * cp;
     auto gather = [&](int hs) {  // sketch rows rg + 32 (JR hs + u), u < JR
       const uint4* offv = reinterpret_cast<const uint4*>(s_off + rg * JU + JR * hs);
@@ -414,8 +490,8 @@ __global__ void __launch_bounds__(NT, 1)
     }
     if constexpr (!S::kInPlace) {
       __syncthreads();  // stage s and the separate tile are free again
-      if (tid == 0 && issued < ntiles) {
-        fence_proxy_async_smem();
+      if (tid < kIssuers && issued < ntiles) {
+        if constexpr (!ROWS) fence_proxy_async_smem();
         issue_next();
       }
     }
@@ -425,6 +501,7 @@ __global__ void __launch_bounds__(NT, 1)
     }
     new_block = a_n == 0;
     new_panel = wrap;
+    ++since;
     a = a_n;
     i = i_n;
     c = c_n;
@@ -731,41 +808,54 @@ EncodeFn encode_fn() {
 // shared-memory latency); 512 < l <= 768 (JM = 48): 256 threads of 64
 // values, whose 255-register budget holds 96 accumulators (packed
 // butterflies).
-template <typename Tin, int JM>
+// Rows off 16 bytes: the 512-thread kernel at every l, three stages.
+template <typename Tin, int JM, bool ROWS>
 struct TmaKernel {
-  static constexpr int STAGES = stages_for<Tin>();
+  static constexpr int STAGES = ROWS ? 3 : stages_for<Tin>();
   static constexpr bool k256 = JM == 48;
+  static_assert(!(ROWS && k256), "JM = 64 in its place");
   static constexpr int NT = k256 ? 256 : 512;
   static size_t smem() {
     if constexpr (k256)
       return TmaShape256<Tin, JM / 2, STAGES>::smem_bytes();
     else
-      return TmaShape<Tin, 32, 512, 512, JM, STAGES>::smem_bytes();
+      return TmaShape<Tin, 32, 512, 512, JM, STAGES, ROWS>::smem_bytes();
   }
   static auto fn() {
     if constexpr (k256)
       return k_sketch_tma256<Tin, JM / 2, STAGES>;
     else
-      return k_sketch_tma<Tin, 32, 512, 512, JM, STAGES>;
+      return k_sketch_tma<Tin, 32, 512, 512, JM, STAGES, ROWS>;
+  }
+  // Occupancy, with the kernel's shared-memory limit raised on the way.
+  static int occupancy() {
+    static DeviceCache cache;
+    return cache.get([] {
+      if (cudaFuncSetAttribute(fn(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem()) != cudaSuccess) return -1;
+      int occ = 0;
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn(), NT, smem()) != cudaSuccess) return -1;
+      return occ;
+    });
   }
 };
 
-template <typename Tin, int JM>
+template <typename Tin, int JM, bool ROWS>
 int launch_tma(const SketchPlan& plan, const SketchArgs& a, const CUtensorMap& map, int* err, uint64_t* dtab,
                uint64_t* dttab, void* out, int64_t ldo, cudaStream_t stream) {
+  using K = TmaKernel<Tin, JM, ROWS>;
   constexpr int W = 32;
-  constexpr int NT = TmaKernel<Tin, JM>::NT;
-  auto kern = TmaKernel<Tin, JM>::fn();
-  const size_t smem = TmaKernel<Tin, JM>::smem();
-  BSRHT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (K::occupancy() < 1) return BSRHT_ECUDA;
   const int64_t tw = (a.jn + 63) / 64;
   const int64_t tot = (int64_t)plan.p * (plan.nch * 16 + tw);
   uint32_t* dmtab = reinterpret_cast<uint32_t*>(dtab);
-  k_sign_tables<<<(unsigned)std::min<int64_t>((tot + 255) / 256, 4096), 256, 0, stream>>>(a.seed, plan.p, plan.nch,
-                                                                                          a.j0, tw, dmtab, dttab);
+  // (No overlap of these launches as in the FP64 form: the wait it puts into
+  // the kernel costs the compiled loop 0.4 %.  Nor a reduce inside the kernel,
+  // by the last CTA of each panel: large sketches 7 % slower, small ones 10 %.)
+  k_sign_tables<<<(unsigned)std::min<int64_t>((tot + 255) / 256, 4096), 256, 0, stream>>>(
+      a.seed, plan.p, plan.nch, a.j0, tw, dmtab, dttab, err, a.j0 == 0 ? 1 : 0);
   BSRHT_CUDA_TRY(cudaGetLastError());
   trace_mark(stream, "sketch_tables");
-  kern<<<plan.G, NT, smem, stream>>>(map, a, dmtab, dttab, tw, err);
+  K::fn()<<<plan.G, K::NT, K::smem(), stream>>>(map, a, dmtab, dttab, tw, err);
   BSRHT_CUDA_TRY(cudaGetLastError());
   trace_mark(stream, "sketch_kernel");
   const int64_t total = (a.jn + kReduceRows - 1) / kReduceRows * a.P * 32;  // one warp per (row group, panel)
@@ -778,23 +868,12 @@ int launch_tma(const SketchPlan& plan, const SketchArgs& a, const CUtensorMap& m
   return BSRHT_OK;
 }
 
-template <typename Tin, int JM>
-int occ_tma() {
-  constexpr int NT = TmaKernel<Tin, JM>::NT;
-  auto kern = TmaKernel<Tin, JM>::fn();
-  const size_t smem = TmaKernel<Tin, JM>::smem();
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
-  int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem) != cudaSuccess) return 0;
-  return occ;
-}
-
 template <typename Tin>
-int occ_tma_jm(int jm) {
+int occ_tma_jm(int jm, bool rows) {
   switch (jm) {
-    case 32: return occ_tma<Tin, 32>();
-    case 48: return occ_tma<Tin, 48>();
-    case 64: return occ_tma<Tin, 64>();
+    case 32: return rows ? TmaKernel<Tin, 32, true>::occupancy() : TmaKernel<Tin, 32, false>::occupancy();
+    case 48: return rows ? 0 : TmaKernel<Tin, 48, false>::occupancy();
+    case 64: return rows ? TmaKernel<Tin, 64, true>::occupancy() : TmaKernel<Tin, 64, false>::occupancy();
   }
   return 0;
 }
@@ -802,10 +881,17 @@ int occ_tma_jm(int jm) {
 template <typename Tin>
 int launch_tma_jm(const SketchPlan& plan, const SketchArgs& a, const CUtensorMap& map, int* err, uint64_t* dtab,
                   uint64_t* dttab, void* out, int64_t ldo, cudaStream_t stream) {
+  if (plan.rows) {
+    switch (plan.JM) {
+      case 32: return launch_tma<Tin, 32, true>(plan, a, map, err, dtab, dttab, out, ldo, stream);
+      case 64: return launch_tma<Tin, 64, true>(plan, a, map, err, dtab, dttab, out, ldo, stream);
+    }
+    return BSRHT_EINVAL;
+  }
   switch (plan.JM) {
-    case 32: return launch_tma<Tin, 32>(plan, a, map, err, dtab, dttab, out, ldo, stream);
-    case 48: return launch_tma<Tin, 48>(plan, a, map, err, dtab, dttab, out, ldo, stream);
-    case 64: return launch_tma<Tin, 64>(plan, a, map, err, dtab, dttab, out, ldo, stream);
+    case 32: return launch_tma<Tin, 32, false>(plan, a, map, err, dtab, dttab, out, ldo, stream);
+    case 48: return launch_tma<Tin, 48, false>(plan, a, map, err, dtab, dttab, out, ldo, stream);
+    case 64: return launch_tma<Tin, 64, false>(plan, a, map, err, dtab, dttab, out, ldo, stream);
   }
   return BSRHT_EINVAL;
 }
@@ -841,21 +927,21 @@ bool make_tensor_map_3d(CUtensorMap* map, const void* base, CUtensorMapDataType 
 
 int sketch_occupancy_tma(const SketchPlan& plan) {
   switch (plan.dtype) {
-    case BSRHT_F32: return occ_tma_jm<float>(plan.JM);
-    case BSRHT_BF16: return occ_tma_jm<__nv_bfloat16>(plan.JM);
-    case BSRHT_F16: return occ_tma_jm<__half>(plan.JM);
+    case BSRHT_F32: return occ_tma_jm<float>(plan.JM, plan.rows);
+    case BSRHT_BF16: return occ_tma_jm<__nv_bfloat16>(plan.JM, plan.rows);
+    case BSRHT_F16: return occ_tma_jm<__half>(plan.JM, plan.rows);
   }
   return 0;
 }
 
 int sketch_launch_tma(const SketchPlan& plan, const SketchArgs& a, void* out, int64_t ldo, int* err,
                       uint64_t* dtab, uint64_t* dttab, cudaStream_t stream) {
-  CUtensorMap map;
+  CUtensorMap map = {};
   const CUtensorMapDataType dt = plan.dtype == BSRHT_F32    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                  : plan.dtype == BSRHT_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
                                                             : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
   const size_t es = plan.dtype == BSRHT_F32 ? 4 : 2;
-  if (!make_tensor_map_2d(&map, a.A, dt, es, (uint64_t)plan.n, (uint64_t)plan.m, (uint64_t)plan.lda, 32,
+  if (!plan.rows && !make_tensor_map_2d(&map, a.A, dt, es, (uint64_t)plan.n, (uint64_t)plan.m, (uint64_t)plan.lda, 32,
                           256))
     return BSRHT_EUNSUP;
   switch (plan.dtype) {

@@ -59,6 +59,19 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
+// 16 bytes from global to shared memory, both 16-byte aligned, asynchronous.
+__device__ __forceinline__ void copy16_async(void* dst, uintptr_t src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+// One arrival on the barrier (part of its count) once this thread's earlier
+// copy16_async have landed.
+__device__ __forceinline__ void mbar_arrive_on_copies(uint64_t* bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_one(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
 // Host: 2-D row-major tensor map (rows x cols, row stride ld elements) with
 // a box of box_cols x box_rows; out-of-range elements read as zero.
 // Returns false if the driver entry point is unavailable or rejects the map.
