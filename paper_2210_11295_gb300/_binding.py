@@ -182,18 +182,18 @@ def make_opts(a: torch.Tensor, variant: int = VARIANT_AUTO, workspace: torch.Ten
         raise ValueError("A must be a 2-D tensor with unit column stride (row-major)")
     if a.dtype not in _DTYPES:
         raise ValueError(f"unsupported dtype {a.dtype}")
-    o = Opts()
-    lib.bsrht_opts_init(ctypes.byref(o))
-    o.dtype = _DTYPES[a.dtype]
-    o.variant = int(variant)
-    o.precision = int(precision)
-    o.lda = int(a.stride(0)) if a.shape[0] > 1 else int(a.shape[1])
-    s = stream if stream is not None else torch.cuda.current_stream(a.device)
-    o.stream = ctypes.c_void_p(s.cuda_stream)
-    if workspace is not None:
-        o.workspace = ctypes.c_void_p(workspace.data_ptr())
-        o.workspace_bytes = workspace.numel() * workspace.element_size()
-    return o
+    # Every field of bsrht_opts in one construction, and the raw handle of the
+    # current stream: a small sketch costs less than the objects around it.
+    if stream is not None:
+        s = stream.cuda_stream
+    elif a.is_cuda:
+        s = torch._C._cuda_getCurrentRawStream(a.get_device())
+    else:
+        s = torch.cuda.current_stream(a.device).cuda_stream
+    ws, ws_bytes = (None, 0) if workspace is None else (workspace.data_ptr(),
+                                                        workspace.numel() * workspace.element_size())
+    lda = a.stride(0) if a.shape[0] > 1 else a.shape[1]
+    return Opts(_DTYPES[a.dtype], int(variant), lda, s, ws, ws_bytes, int(precision))
 
 
 def sketch_out_dtype(dtype: torch.dtype, precision: int = 0) -> torch.dtype:
@@ -220,12 +220,13 @@ def bsrht_sketch(a: torch.Tensor, p: int, l: int, seed: int, out: torch.Tensor |
     n, m = a.shape
     odt = sketch_out_dtype(a.dtype, precision)
     if out is None:
-        out = torch.empty(l, m, device=a.device, dtype=odt)
-    if out.shape != (l, m) or not out.is_contiguous() or out.dtype != odt:
+        out = a.new_empty((l, m), dtype=odt)
+    elif out.shape != (l, m) or not out.is_contiguous() or out.dtype != odt:
         raise ValueError("out must be a contiguous l x m tensor of the sketch dtype")
     o = make_opts(a, variant, workspace, stream, precision)
-    _check(lib.bsrht_sketch(_dptr(a), n, m, p, l, seed & (2**64 - 1), _dptr(out), ctypes.byref(o)),
-           "bsrht_sketch")
+    st = lib.bsrht_sketch(a.data_ptr(), n, m, p, l, seed & (2**64 - 1), out.data_ptr(), ctypes.byref(o))
+    if st != BSRHT_OK:
+        raise BsrhtError(st, "bsrht_sketch")
     return out
 
 
