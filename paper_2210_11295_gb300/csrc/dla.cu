@@ -337,20 +337,25 @@ int tri_inverse(const Dla& d, const double* L, double* LT, double* Rinv, int64_t
 
 // ------------------------------------------- fused Cholesky and inverse
 // One cooperative kernel: right-looking blocked Cholesky G = L L^T with
-// 32 x 32 blocks, and the same block eliminations applied to an identity
+// 16 x 16 blocks, and the same block eliminations applied to an identity
 // matrix T, which turns T into L^-1.  Step kb:
 //   (a) L_kk = chol(A_kk) and X_kk = L_kk^-1 (one CTA, shared memory);
-//   (b) panel L_ik = A_ik X_kk^T (one warp per row i > kb) and the final
+//   (b) panel L_ik = A_ik X_kk^T (half a warp per row i > kb) and the final
 //       block row X_kb,c = X_kk T_kb,c of L^-1 (c < kb);
 //   (c) trailing update A_ij -= L_ik L_jk^T (kb < j <= i) and
-//       T_ic -= L_ik X_kb,c (c <= kb < i), one 32 x 32 tile per CTA; the CTA
-//       holding tile (kb+1, kb+1) then factors it, which is (a) of the next
-//       step.
-// Two grid barriers per block step.  Outputs: L in the lower triangle of g
-// (upper zeroed), LT = L^T and Rinv = L^-T (row-major, upper triangular).
-// T and X are l x l scratch.  A pivot <= 0 sets kStatusNotPD (and is
-// replaced by 1 so the kernel runs to the end).
-constexpr int kCB = 32;
+//       T_ic -= L_ik X_kb,c (c <= kb < i), one 16 x 16 tile per warp; CTA 0
+//       updates tile (kb+1, kb+1) alone and factors it in place, which is
+//       (a) of the next step.
+// Two grid barriers per block step.  What bounds it: FP64 operations take
+// about 62 cycles and an SM finishes two a cycle, so the time is the chain of
+// (a) (16 pivots of one reciprocal each) and the barriers.  16-wide blocks
+// keep the tile update and the factorisation of (a), which no other SM can
+// share, to a quarter and an eighth of those of 32-wide ones; the other tiles
+// then fit beside that chain (CHOL_MS).
+// Outputs: L in the lower triangle of g (upper zeroed), LT = L^T and Rinv =
+// L^-T (row-major, upper triangular).  T and X are l x l scratch.  A pivot
+// <= 0 sets kStatusNotPD (and is replaced by 1 so the kernel runs to the end).
+constexpr int kCB = 16;
 
 struct CholInvArgs {
   double* g;
@@ -363,201 +368,192 @@ struct CholInvArgs {
   int* status;
 };
 
-// 1/d for a pivot d > 0: FP32 seed on d scaled by a power of two into
-// [1, 2), then two Newton steps y <- y + y (1 - d y) (relative error 2^-23 ->
-// 2^-46 -> rounding).  A dependent FP64 operation costs about 60 cycles on
-// this GPU (measured), so this chain of six is what one column of the
-// diagonal factorisation waits for.
+// 1/d for a pivot d > 0: FP32 seed y (relative error 2^-22), then
+// y (1 + e + e^2) with e = 1 - d y, whose error e^3 is below FP64's rounding:
+// three dependent FP64 operations on the chain from pivot to pivot.
 __device__ __forceinline__ double ci_rcp(double d) {
-  if (d > 0x1.0p-1000 && d < 0x1.0p1000) {
-    const long long bits = __double_as_longlong(d);
-    const int e = (int)((bits >> 52) & 0x7FF) - 1023;                       // d = f 2^e, f in [1, 2)
-    const double f = __longlong_as_double(bits - ((long long)e << 52));     // f in [1, 2)
-    double y = (double)__frcp_rn((float)f);
-    y = fma(y, fma(-f, y, 1.0), y);
-    y = fma(y, fma(-f, y, 1.0), y);
-    return y * __longlong_as_double((long long)(1023 - e) << 52);          // times 2^-e
+  if (d > 1e-30 && d < 1e30) {
+    const double y = (double)__fdividef(1.0f, (float)d);
+    const double e = fma(-d, y, 1.0);
+    return fma(y, fma(e, e, e), y);
   }
   return 1.0 / d;
 }
 
-// (a): factor the diagonal block kb (already updated), G_kk = L D L^T with
-// unit lower L, and form its inverse alongside: the eliminations of column j
-// (row i -= l_ij row j, l_ij = s_ij / d_j) are applied to the trailing part
-// of s and to an identity block t, which ends as L^-1.  Thread 0 applies
-// column j's elimination to the next pivot first and forms its reciprocal
-// while threads 1..255 apply the rest, so one barrier per column; the
-// square roots come at the end, all at once: L_kk = L D^1/2 and
-// X_kk = L_kk^-1 = D^-1/2 L^-1.
+// (a): the diagonal block in s (already updated, lower triangle), G_kk =
+// L D L^T with unit lower L, and its inverse alongside: the eliminations of
+// column j (row i -= l_ij row j, l_ij = s_ij / d_j) are applied to the
+// trailing part of s and to an identity block t, which ends as L^-1.  Thread
+// (i, c) owns entry (i, c) of both; thread (j+1, j+1) forms the next pivot's
+// reciprocal meanwhile, so there is one barrier per column.  The square roots
+// come at the end, all at once: L_kk = L D^1/2, X_kk = D^-1/2 L^-1.
 __device__ void ci_factor_diag(const CholInvArgs& a, int kb, double (*s)[kCB + 1], double (*t)[kCB + 1],
                                double* dinv, double* dd) {
-  const int tid = threadIdx.x, l = a.l, k0 = kb * kCB;
+  const int tid = threadIdx.x, i = tid >> 4, c = tid & 15, l = a.l, k0 = kb * kCB;
   const int nb = min(kCB, l - k0);
-  for (int e = tid; e < kCB * kCB; e += blockDim.x) {
-    const int i = e / kCB, j = e % kCB;
-    double v = (i == j) ? 1.0 : 0.0;
-    if (i < nb && j < nb && j <= i) v = a.g[(int64_t)(k0 + i) * l + k0 + j];
-    s[i][j] = v;
-    t[i][j] = (i == j) ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    double p = s[0][0];
+  auto pivot = [&](int j, double p) {
     if (!(p > 0.0)) {
       atomicOr(a.status, kStatusNotPD);
       p = 1.0;
     }
-    dd[0] = p;
-    dinv[0] = ci_rcp(p);
-  }
+    dd[j] = p;
+    dinv[j] = ci_rcp(p);
+  };
+  t[i][c] = (i == c) ? 1.0 : 0.0;
+  if (tid == 0) pivot(0, s[0][0]);
   __syncthreads();
   for (int j = 0; j < kCB; ++j) {
-    const double ij = dinv[j];
-    if (tid == 0) {
-      if (j + 1 < kCB) {
-        const double x = s[j + 1][j];
-        double p = fma(-x * ij, x, s[j + 1][j + 1]);
-        if (!(p > 0.0)) {
-          atomicOr(a.status, kStatusNotPD);
-          p = 1.0;
-        }
-        dd[j + 1] = p;
-        dinv[j + 1] = ci_rcp(p);
-      }
-    } else {
-      // Trailing entries (i, c), j < c <= i, except the next pivot; item e ->
-      // row offset u with u (u + 1) / 2 <= e < (u + 1) (u + 2) / 2.  Then the
-      // entries (i, c), i > j, c <= j of t.
-      const int rem = kCB - 1 - j;
-      const int n_tr = rem * (rem + 1) / 2;
-      const int n_items = n_tr + rem * (j + 1);
-      for (int e = tid - 1; e < n_items; e += blockDim.x - 1) {
-        if (e < n_tr) {
-          if (e == 0) continue;  // (j+1, j+1): thread 0
-          int u = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-          while ((u + 1) * (u + 2) / 2 <= e) ++u;
-          while (u * (u + 1) / 2 > e) --u;
-          const int i = j + 1 + u, c = j + 1 + (e - u * (u + 1) / 2);
-          s[i][c] = fma(-s[i][j] * ij, s[c][j], s[i][c]);
-        } else {
-          const int q = e - n_tr, i = j + 1 + q / (j + 1), c = q % (j + 1);
-          t[i][c] = fma(-s[i][j] * ij, t[j][c], t[i][c]);
-        }
+    if (i > j && c <= i) {
+      const double ij = dinv[j], x = s[i][j];
+      if (c > j) {
+        if (i == j + 1)
+          pivot(i, fma(-(x * x), ij, s[i][i]));
+        else
+          s[i][c] = fma(-x * ij, s[c][j], s[i][c]);
+      } else {
+        t[i][c] = fma(-x * ij, t[j][c], t[i][c]);
       }
     }
     __syncthreads();
   }
-  // D^1/2: sqrt(d_j) and 1/sqrt(d_j), all columns at once.
   if (tid < kCB) {
     const double r = sqrt(dd[tid]);
     dd[tid] = r;
     dinv[tid] = 1.0 / r;
   }
   __syncthreads();
-  for (int e = tid; e < nb * nb; e += blockDim.x) {
-    const int i = e / nb, j = e % nb;
-    // L_kk[i][j] = (s_ij / d_j) sqrt(d_j) = s_ij / sqrt(d_j);  X_kk[i][j] = t_ij / sqrt(d_i).
-    a.g[(int64_t)(k0 + i) * l + k0 + j] = (j < i) ? s[i][j] * dinv[j] : (i == j ? dd[j] : 0.0);
-    a.X[(int64_t)(k0 + i) * l + k0 + j] = (j <= i) ? t[i][j] * dinv[i] : 0.0;
+  if (i < nb && c < nb) {
+    // L_kk[i][c] = (s_ic / d_c) sqrt(d_c) = s_ic / sqrt(d_c);  X_kk[i][c] = t_ic / sqrt(d_i).
+    a.g[(int64_t)(k0 + i) * l + k0 + c] = (c < i) ? s[i][c] * dinv[c] : (i == c ? dd[i] : 0.0);
+    a.X[(int64_t)(k0 + i) * l + k0 + c] = (c <= i) ? t[i][c] * dinv[i] : 0.0;
   }
 }
 
 __global__ void __launch_bounds__(256) k_chol_inv(CholInvArgs a) {
   cg::grid_group grid = cg::this_grid();
-  __shared__ double s0[kCB][kCB + 1];
-  __shared__ double s1[kCB][kCB + 1];
+  __shared__ double sw[8][2][kCB][kCB + 1];  // two blocks per warp
+  __shared__ double xk[kCB][kCB + 1];
   __shared__ double dinv[kCB];
   __shared__ double dd[kCB];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int l = a.l, nblk = a.nblk;
   const int64_t ll = (int64_t)l * l;
+  const int ti = tid >> 4, tc = tid & 15;
+  double(*s0)[kCB + 1] = sw[0][0];
+  double(*s1)[kCB + 1] = sw[0][1];
   // T = I (only its lower block triangle is ever read).
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + tid; e < ll; e += (int64_t)gridDim.x * blockDim.x)
     a.T[e] = (e / l == e % l) ? 1.0 : 0.0;
-  if (blockIdx.x == 0) ci_factor_diag(a, 0, s0, s1, dinv, dd);
+  if (blockIdx.x == 0) {
+    s0[ti][tc] = (ti < l && tc <= ti) ? a.g[(int64_t)ti * l + tc] : (ti == tc ? 1.0 : 0.0);
+    __syncthreads();
+    ci_factor_diag(a, 0, s0, s1, dinv, dd);
+  }
   grid.sync();
-  const int gw = blockIdx.x * (blockDim.x >> 5) + w, nwg = gridDim.x * (blockDim.x >> 5);
+  const int gw = blockIdx.x * 8 + w, nwg = gridDim.x * 8;
   for (int kb = 0; kb < nblk; ++kb) {
     const int k0 = kb * kCB, nb = min(kCB, l - k0);
     const int rows_below = l - k0 - nb;
-    // (b) X_kk into shared memory (every CTA), then panel rows and X row block.
-    for (int e = tid; e < kCB * kCB; e += blockDim.x) {
-      const int i = e / kCB, j = e % kCB;
-      s1[i][j] = (i < nb && j < nb) ? a.X[(int64_t)(k0 + i) * l + k0 + j] : 0.0;
-    }
+    // (b) X_kk into shared memory (every CTA), then panel rows, two per warp,
+    // and 32 columns of a row of the X row block.
+    xk[ti][tc] = (ti < nb && tc < nb) ? a.X[(int64_t)(k0 + ti) * l + k0 + tc] : 0.0;
     __syncthreads();
-    const int xrow_items = kb * kCB;  // rows r < 32 of block kb times column blocks c < kb
-    for (int it = gw; it < rows_below + xrow_items; it += nwg) {
-      if (it < rows_below) {
-        const int64_t i = k0 + nb + it;
-        const double v = lane < nb ? a.g[i * l + k0 + lane] : 0.0;
-        double out = 0.0;
-        for (int e = 0; e < kCB; ++e) out = fma(__shfl_sync(0xffffffffu, v, e), s1[lane][e], out);
-        if (lane < nb) a.g[i * l + k0 + lane] = out;
+    const int np = (rows_below + 1) / 2, nch = (k0 + 31) / 32, nx = nb * nch;
+    for (int it = gw; it < np + nx; it += nwg) {
+      if (it < np) {
+        const int64_t row = k0 + nb + 2 * it + (lane >> 4);
+        const int c = lane & 15;
+        const bool in = row < l && c < nb;
+        const double v = in ? a.g[row * l + k0 + c] : 0.0;
+        double o0 = 0.0, o1 = 0.0;
+#pragma unroll
+        for (int e = 0; e < kCB; e += 2) {
+          o0 = fma(__shfl_sync(0xffffffffu, v, e, 16), xk[c][e], o0);
+          o1 = fma(__shfl_sync(0xffffffffu, v, e + 1, 16), xk[c][e + 1], o1);
+        }
+        if (in) a.g[row * l + k0 + c] = o0 + o1;
       } else {
-        const int q = it - rows_below, r = q / kb, c = q % kb;
-        if (r < nb) {
-          // X[k0+r][c*32+lane] = sum_{e<=r} X_kk[r][e] T[k0+e][c*32+lane]
-          double out = 0.0;
-          for (int e = 0; e <= r; ++e) out = fma(s1[r][e], a.T[(int64_t)(k0 + e) * l + c * kCB + lane], out);
-          a.X[(int64_t)(k0 + r) * l + c * kCB + lane] = out;
+        const int q = it - np, r = q / nch, col = (q - r * nch) * 32 + lane;
+        if (col < k0) {
+          double o0 = 0.0, o1 = 0.0;
+#pragma unroll
+          for (int e = 0; e < kCB; e += 2) {  // X_kk[r][e] = 0 for e > r
+            if (e < nb) o0 = fma(xk[r][e], a.T[(int64_t)(k0 + e) * l + col], o0);
+            if (e + 1 < nb) o1 = fma(xk[r][e + 1], a.T[(int64_t)(k0 + e + 1) * l + col], o1);
+          }
+          a.X[(int64_t)(k0 + r) * l + col] = o0 + o1;
         }
       }
     }
     grid.sync();
     if (kb + 1 == nblk) break;
-    // (c) trailing tiles (bi >= bj > kb) and T tiles (bi > kb >= c).
+    // (c) trailing tiles (bi >= bj > kb) and T tiles (bi > kb >= c); item 0
+    // is the diagonal tile (kb+1, kb+1).  (nb = 16: only the last block is short.)
     const int rem = nblk - kb - 1;
     const int n_trail = rem * (rem + 1) / 2, n_t = rem * (kb + 1);
-    const int tx = tid & 31, ty = tid >> 5;
-    for (int item = blockIdx.x; item < n_trail + n_t; item += gridDim.x) {
-      int bi, bj;
-      bool trail = item < n_trail;
-      if (trail) {
-        // item 0 is the diagonal tile (kb+1, kb+1); then the rest row by row.
-        int q = item, row = 0;
-        while (q > row) {
-          q -= row + 1;
-          ++row;
-        }
-        bi = kb + 1 + row;
-        bj = kb + 1 + q;
-      } else {
-        const int q = item - n_trail;
-        bi = kb + 1 + q / (kb + 1);
-        bj = q % (kb + 1);
-      }
+    if (blockIdx.x == 0) {
+      const int64_t r0 = k0 + kCB;
+      s1[ti][tc] = r0 + ti < l ? a.g[(r0 + ti) * l + k0 + tc] : 0.0;
       __syncthreads();
-      // s0 = L rows of block bi (panel of block kb); s1 = L rows of block bj or X row block kb.
-      for (int r = ty; r < kCB; r += 8) {
-        const int64_t ri = (int64_t)bi * kCB + r;
-        s0[r][tx] = (ri < l && tx < nb) ? a.g[ri * l + k0 + tx] : 0.0;
-        if (trail) {
-          const int64_t rj = (int64_t)bj * kCB + r;
-          s1[r][tx] = (rj < l && tx < nb) ? a.g[rj * l + k0 + tx] : 0.0;
-        } else {
-          s1[r][tx] = (r < nb) ? a.X[(int64_t)(k0 + r) * l + bj * kCB + tx] : 0.0;
+      double o0 = 0.0, o1 = 0.0;
+      if (tc <= ti) {
+#pragma unroll
+        for (int e = 0; e < kCB; e += 2) {
+          o0 = fma(s1[ti][e], s1[tc][e], o0);
+          o1 = fma(s1[ti][e + 1], s1[tc][e + 1], o1);
         }
       }
+      s0[ti][tc] = (r0 + ti < l && tc <= ti) ? a.g[(r0 + ti) * l + r0 + tc] - (o0 + o1) : (ti == tc ? 1.0 : 0.0);
       __syncthreads();
-      const int64_t col = (int64_t)bj * kCB + tx;
-      for (int r = ty; r < kCB; r += 8) {
-        const int64_t row = (int64_t)bi * kCB + r;
-        if (row >= l || col >= l) continue;
-        double acc = 0.0;
+      ci_factor_diag(a, kb + 1, s0, s1, dinv, dd);
+    } else {
+      double(*sa)[kCB + 1] = sw[w][0];
+      double(*sb)[kCB + 1] = sw[w][1];
+      for (int item = 1 + (blockIdx.x - 1) * 8 + w; item < n_trail + n_t; item += (gridDim.x - 1) * 8) {
+        const bool trail = item < n_trail;
+        int bi, bj;
         if (trail) {
-#pragma unroll 8
-          for (int e = 0; e < kCB; ++e) acc = fma(s0[r][e], s1[tx][e], acc);
-          a.g[row * l + col] -= acc;
+          int row = (int)((sqrtf(8.0f * (float)item + 1.0f) - 1.0f) * 0.5f);
+          while ((row + 1) * (row + 2) / 2 <= item) ++row;
+          while (row * (row + 1) / 2 > item) --row;
+          bi = kb + 1 + row;
+          bj = kb + 1 + item - row * (row + 1) / 2;
         } else {
-#pragma unroll 8
-          for (int e = 0; e < kCB; ++e) acc = fma(s0[r][e], s1[e][tx], acc);
-          a.T[row * l + col] -= acc;
+          const int q = item - n_trail;
+          bi = kb + 1 + q / (kb + 1);
+          bj = q % (kb + 1);
         }
-      }
-      if (item == 0) {
-        __syncthreads();
-        ci_factor_diag(a, kb + 1, s0, s1, dinv, dd);
+        __syncwarp();
+        const int lc = lane & 15;
+#pragma unroll
+        for (int r = lane >> 4; r < kCB; r += 2) {
+          const int64_t ri = (int64_t)bi * kCB + r, rj = (int64_t)bj * kCB + r;
+          sa[r][lc] = ri < l ? a.g[ri * l + k0 + lc] : 0.0;
+          // Transposed for T tiles, so that both kinds read sb[column][e].
+          if (trail)
+            sb[r][lc] = rj < l ? a.g[rj * l + k0 + lc] : 0.0;
+          else
+            sb[lc][r] = a.X[(int64_t)(k0 + r) * l + bj * kCB + lc];
+        }
+        __syncwarp();
+        // Lane: row lane / 2 of the tile, columns 8 (lane & 1) .. + 7.
+        const int i = lane >> 1, c0 = 8 * (lane & 1);
+        double acc[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc[q] = 0.0;
+#pragma unroll
+        for (int e = 0; e < kCB; ++e) {
+          const double x = sa[i][e];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) acc[q] = fma(x, sb[c0 + q][e], acc[q]);
+        }
+        const int64_t row = (int64_t)bi * kCB + i, col = (int64_t)bj * kCB + c0;
+        double* dst = (trail ? a.g : a.T) + row * l + col;
+        if (row < l) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            if (col + q < l) dst[q] -= acc[q];
+        }
       }
     }
     grid.sync();
@@ -575,9 +571,11 @@ __global__ void __launch_bounds__(256) k_chol_inv(CholInvArgs a) {
 int chol_inv(const Dla& d, double* g, double* LT, double* Rinv, double* T, double* X, int64_t l) {
   if (l <= 0) return BSRHT_OK;
   CholInvArgs a{g, LT, Rinv, T, X, (int)l, (int)((l + kCB - 1) / kCB), d.status};
-  int occ = 0;
-  BSRHT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_chol_inv, 256, 0));
-  const int blocks = num_sms() * std::max(1, std::min(occ, 1));
+  // CTA 0 for the diagonal blocks and one CTA per four tiles of the fullest
+  // step (about nblk^2 / 2), as far as the SMs go: barriers over fewer CTAs
+  // are cheaper.
+  const int64_t tiles = (int64_t)a.nblk * (a.nblk + 1) / 2;
+  const int blocks = (int)std::min<int64_t>(num_sms(), 1 + (tiles + 3) / 4);
   void* args[] = {&a};
   const int st = launch_cooperative((const void*)k_chol_inv, dim3(blocks), dim3(256), args, 0, d.s);
   if (st != BSRHT_OK) return st;

@@ -140,6 +140,11 @@ int gemm_int8x7(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const 
 // FP32-accurate products of 16-bit data: C (M x N, FP32, ldc) = A (M x K,
 // BF16 or F16, 16-byte aligned rows) * B (K x N, FP32 or FP64, ldb); Ct as
 // in gemm_tc.
+// FP32 products at FP16's rate: as gemm_tc (b_kmajor and gram false), for
+// FP32 A with 16-byte aligned rows.
+bool gemm_f32x2_eligible(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda);
+int gemm_f32x2(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, DT tb,
+               const void* B, int64_t ldb, DT tc_out, void* C, int64_t ldc, bool b_upper, float* Ct);
 bool gemm_a16_eligible(DT ta, int64_t M, int64_t N, int64_t K, const void* A, int64_t lda);
 int gemm_a16(const Dla& d, Arena& ar, DT ta, int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, DT tb,
              const void* B, int64_t ldb, float* C, int64_t ldc, float* Ct);

@@ -110,11 +110,11 @@ __global__ void k_int8x7_reduce(const double* __restrict__ P, double* __restrict
   C[i * ldc + j] = s;
 }
 
-// Three 16-bit slices of the columns of B (K x N, row-major, read as FP32),
-// K-major: out[s][c][k], row length ldk.  With max |column| < 2^(E - 126)
-// the column is scaled by 2^(139 - E), so its largest entry lies in [2^13, 2^14)
+// NS 16-bit slices of the columns of B (K x N, row-major, read as FP32),
+// K-major: out[s][c][k], row length ldk.  With 2^(E - 127) <= max |column| <
+// 2^(E - 126) the column is scaled by 2^(140 - E), so its largest entry lies in [2^13, 2^14)
 // (FP16's range with 2^-24 as the smallest step); scale[c] undoes that.
-template <typename TB, typename T16>
+template <typename TB, typename T16, int NS>
 __global__ void __launch_bounds__(256) k_slices16_cols(const TB* __restrict__ B, int64_t K, int64_t N, int64_t ldb,
                                                        T16* __restrict__ out, int64_t ldk,
                                                        const int* __restrict__ exps, int64_t tiles_n,
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(256) k_slices16_cols(const TB* __restrict__ B,
     if (c >= N) continue;
     // exps: FP32 biased exponents.  Columns at the ends of the range are
     // scaled as far as one FP32 factor and its inverse reach.
-    const int sh = min(max(139 - exps[c], -100), 100);
+    const int sh = min(max(140 - exps[c], -126), 126);
     const float f = __uint_as_float((uint32_t)(127 + sh) << 23);
     if (tk == 0 && tx == 0) scale[c] = __uint_as_float((uint32_t)(127 - sh) << 23);
 #pragma unroll
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(256) k_slices16_cols(const TB* __restrict__ B,
       if (k >= ldk) continue;
       float x = t[tx + 32 * h][r] * f;
 #pragma unroll
-      for (int s = 0; s < 3; ++s) {
+      for (int s = 0; s < NS; ++s) {
         const T16 d = (T16)x;
         out[(int64_t)s * plane + c * ldk + k] = d;
         x -= (float)d;
@@ -345,6 +345,52 @@ int gemm_int8x7(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const 
   return part ? reduce(M, C) : BSRHT_OK;
 }
 
+namespace {
+
+// Scratch and preparation of the NS slices of B (K x N) shared by the two
+// kernels that split it once: slices (16-bit, K-major), column scales.
+struct SlicedB {
+  void* slices;
+  float* scale;
+  int64_t ldk;
+  int bn;  // column tiles of equal width (a multiple of 16, at most 256)
+};
+
+size_t sliced_b_bytes(int64_t K, int64_t N, int ns) {
+  return 2 * (size_t)ns * (size_t)N * (size_t)round_up(K, 8) + 8 * (size_t)N + 4096;
+}
+
+template <typename T16, int NS>
+int slice_b(const Dla& d, Arena& ar, int64_t K, int64_t N, DT tb, const void* B, int64_t ldb, SlicedB* out) {
+  out->ldk = round_up(K, 8);
+  out->slices = ar.take(2 * (size_t)NS * (size_t)N * out->ldk);
+  int* exps = static_cast<int*>(ar.take(sizeof(int) * (size_t)N));
+  out->scale = static_cast<float*>(ar.take(sizeof(float) * (size_t)N));
+  const int64_t tn = (N + 255) / 256;
+  out->bn = (int)round_up((N + tn - 1) / tn, 16);
+  if (!ar.ok()) return BSRHT_ENOMEM;
+  if (ar.measure) return BSRHT_OK;
+  BSRHT_CUDA_TRY(cudaMemsetAsync(exps, 0, sizeof(int) * (size_t)N, d.s));
+  const unsigned cb = (unsigned)((N + 63) / 64), ry = row_parts(K, cb);
+  const int64_t t64 = (N + 63) / 64, tk = t64 * ((out->ldk + 63) / 64);
+  if (tk > 0x7FFFFFFF) return BSRHT_EUNSUP;
+  auto prep = [&](auto* b) {
+    using TB = std::remove_pointer_t<decltype(b)>;
+    k_col_exps32<TB><<<dim3(cb, ry), 64, 0, d.s>>>(b, K, N, ldb, (K + ry - 1) / ry, exps);
+    k_slices16_cols<TB, T16, NS><<<(unsigned)tk, 256, 0, d.s>>>(b, K, N, ldb, static_cast<T16*>(out->slices), out->ldk,
+                                                                 exps, t64, out->scale);
+  };
+  if (tb == DT::F64)
+    prep(static_cast<const double*>(B));
+  else
+    prep(static_cast<const float*>(B));
+  BSRHT_CUDA_TRY(cudaGetLastError());
+  note_launches(2);
+  return BSRHT_OK;
+}
+
+}  // namespace
+
 bool gemm_a16_eligible(DT ta, int64_t M, int64_t N, int64_t K, const void* A, int64_t lda) {
   return (ta == DT::BF16 || ta == DT::F16) && M >= 256 && N >= 1 && K >= 64 && (lda % 8) == 0 &&
          (reinterpret_cast<uintptr_t>(A) % 16) == 0;
@@ -354,52 +400,61 @@ int gemm_a16(const Dla& d, Arena& ar, DT ta, int64_t M, int64_t N, int64_t K, co
              const void* B, int64_t ldb, float* C, int64_t ldc, float* Ct) {
   using S = sl::A16;
   if (tb != DT::F32 && tb != DT::F64) return BSRHT_EUNSUP;
-  const int64_t ldk = round_up(K, 8);
-  const size_t need = 6 * (size_t)N * ldk + 8 * (size_t)N + 4096;
-  if (!ar.measure && ar.used + need > ar.cap) return BSRHT_EUNSUP;
-  void* bs = ar.take(6 * (size_t)N * ldk);
-  int* exps = static_cast<int*>(ar.take(sizeof(int) * (size_t)N));
-  float* scale = static_cast<float*>(ar.take(sizeof(float) * (size_t)N));
-  if (!ar.ok()) return BSRHT_ENOMEM;
-  if (ar.measure) return BSRHT_OK;
+  if (!ar.measure && ar.used + sliced_b_bytes(K, N, S::NB) > ar.cap) return BSRHT_EUNSUP;
   const bool bf = ta == DT::BF16;
-  BSRHT_CUDA_TRY(cudaMemsetAsync(exps, 0, sizeof(int) * (size_t)N, d.s));
-  const unsigned cb = (unsigned)((N + 63) / 64), ry = row_parts(K, cb);
-  const int64_t t64 = (N + 63) / 64, tk = t64 * ((ldk + 63) / 64);
-  if (tk > 0x7FFFFFFF) return BSRHT_EUNSUP;
-  auto prep = [&](auto* b) {
-    using TB = std::remove_pointer_t<decltype(b)>;
-    k_col_exps32<TB><<<dim3(cb, ry), 64, 0, d.s>>>(b, K, N, ldb, (K + ry - 1) / ry, exps);
-    if (bf)
-      k_slices16_cols<TB, __nv_bfloat16><<<(unsigned)tk, 256, 0, d.s>>>(b, K, N, ldb, static_cast<__nv_bfloat16*>(bs),
-                                                                        ldk, exps, t64, scale);
-    else
-      k_slices16_cols<TB, __half><<<(unsigned)tk, 256, 0, d.s>>>(b, K, N, ldb, static_cast<__half*>(bs), ldk, exps,
-                                                                 t64, scale);
-  };
-  if (tb == DT::F64)
-    prep(static_cast<const double*>(B));
-  else
-    prep(static_cast<const float*>(B));
-  BSRHT_CUDA_TRY(cudaGetLastError());
-  // Column tiles of equal width (a multiple of 16, at most 256).
-  const int64_t tn = (N + S::BNMAX - 1) / S::BNMAX;
-  const int bn = (int)round_up((N + tn - 1) / tn, 16);
-  const int64_t tiles = (M + sl::BM - 1) / sl::BM * ((N + bn - 1) / bn);
+  SlicedB b;
+  TRY_SL(bf ? (slice_b<__nv_bfloat16, S::NB>(d, ar, K, N, tb, B, ldb, &b))
+            : (slice_b<__half, S::NB>(d, ar, K, N, tb, B, ldb, &b)));
+  if (ar.measure) return BSRHT_OK;
+  const int64_t tiles = (M + sl::BM - 1) / sl::BM * ((N + b.bn - 1) / b.bn);
   if (tiles > 0x7FFFFFFF) return BSRHT_EUNSUP;
   const CUtensorMapDataType dt = bf ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
   CUtensorMap ma, mb;
   if (!make_tensor_map_2d(&ma, A, dt, 2, (uint64_t)M, (uint64_t)K, (uint64_t)lda, S::BK, sl::BM,
                           CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !make_slice_map(&mb, bs, dt, K, N, 3, ldk, S::BK, (uint32_t)bn, CU_TENSOR_MAP_SWIZZLE_128B))
+      !make_slice_map(&mb, b.slices, dt, K, N, S::NB, b.ldk, S::BK, (uint32_t)b.bn, CU_TENSOR_MAP_SWIZZLE_128B))
     return BSRHT_EUNSUP;
   BSRHT_CUDA_TRY(
       cudaFuncSetAttribute(sl::k_gemm_a16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_bytes()));
-  sl::A16Args g{M, N, K, C, ldc, scale, Ct, M, bn, bf ? 1 : 0, d.status};
+  sl::A16Args g{M, N, K, C, ldc, b.scale, Ct, M, b.bn, bf ? 1 : 0, d.status};
   sl::k_gemm_a16<<<(unsigned)tiles, sl::kThreads, S::smem_bytes(), d.s>>>(ma, mb, g);
   BSRHT_CUDA_TRY(cudaGetLastError());
-  note_launches(3);
+  note_launches(1);
   return BSRHT_OK;
+}
+
+// Tiles enough for most SMs (the other kernel splits K instead), wide enough
+// to gain on the split of A, and a K chain of at most 256 folds.
+bool gemm_f32x2_eligible(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda) {
+  return M >= 128 * 96 && N >= 48 && K >= 32 && K <= 8192 && (lda % 4) == 0 &&
+         (reinterpret_cast<uintptr_t>(A) % 16) == 0;
+}
+
+int gemm_f32x2(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, DT tb,
+               const void* B, int64_t ldb, DT tc_out, void* C, int64_t ldc, bool b_upper, float* Ct) {
+  using S = sl::F32x2;
+  if ((tb != DT::F32 && tb != DT::F64) || (tc_out != DT::F32 && tc_out != DT::F64)) return BSRHT_EUNSUP;
+  if (!ar.measure && ar.used + sliced_b_bytes(K, N, S::NB) > ar.cap) return BSRHT_EUNSUP;
+  SlicedB b;
+  TRY_SL((slice_b<__half, S::NB>(d, ar, K, N, tb, B, ldb, &b)));
+  if (ar.measure) return BSRHT_OK;
+  const int64_t tiles = (M + sl::BM - 1) / sl::BM * ((N + b.bn - 1) / b.bn);
+  if (tiles > 0x7FFFFFFF) return BSRHT_EUNSUP;
+  CUtensorMap ma, mb;
+  if (!make_tensor_map_2d(&ma, A, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, (uint64_t)M, (uint64_t)K, (uint64_t)lda, S::BK,
+                          sl::BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !make_slice_map(&mb, b.slices, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, K, N, S::NB, b.ldk, S::BK, (uint32_t)b.bn,
+                      CU_TENSOR_MAP_SWIZZLE_64B))
+    return BSRHT_EUNSUP;
+  sl::F32x2Args g{M, N, K, C, ldc, b.scale, Ct, M, b.bn, b_upper ? 1 : 0, d.status};
+  auto launch = [&](auto kern) -> int {
+    BSRHT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_bytes()));
+    kern<<<(unsigned)tiles, sl::kThreads, S::smem_bytes(), d.s>>>(ma, mb, g);
+    BSRHT_CUDA_TRY(cudaGetLastError());
+    note_launches(1);
+    return BSRHT_OK;
+  };
+  return tc_out == DT::F32 ? launch(sl::k_gemm_f32x2<float>) : launch(sl::k_gemm_f32x2<double>);
 }
 
 }  // namespace bsrht

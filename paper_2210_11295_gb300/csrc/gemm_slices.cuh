@@ -1,6 +1,6 @@
 // Tensor-core products on operands held as 16-bit slices (tcgen05 kind::f16).
 //
-// Two kernels share the layout: K-major slices [slice][row][k] in global
+// Three kernels share the layout: K-major slices [slice][row][k] in global
 // memory, TMA into swizzled shared memory, one thread issuing the MMAs, FP32
 // accumulators in tensor memory, eight warps folding them.
 //
@@ -24,6 +24,17 @@
 // per product; each K block of 64 starts a fresh accumulator, smallest slice
 // first, which the fold adds to FP32 registers, rounding to nearest (the
 // tensor core's own accumulation truncates).
+//
+// k_gemm_f32x2: FP32 products of FP32 data at twice the TF32 rate.  An FP16
+// pair holds as much of an FP32 value as a TF32 pair (11 + 11 bits) once it is
+// scaled into FP16's range, and the 16-bit MMA is twice as fast and reads
+// half the shared memory.  B is split once in global memory (two slices,
+// scaled per column); the fold warps split each staged tile of A, one
+// power-of-two scale per row and K block of 32, and undo that scale when they
+// add the block to their FP32 sums: hi lo + lo hi + hi hi, smallest first;
+// what is dropped lies below 2^-23 of each product, or 2^-38 of the row's
+// largest entry in the block.  Bound by shared memory (copies in, split,
+// operand reads: 152 KB a K block against 768 cycles of MMA).
 #pragma once
 
 #include <cuda.h>
@@ -496,6 +507,229 @@ __global__ void __launch_bounds__(kThreads, 1)
           // Column q is row c0 + q of C^T; lane = row of C: 128 contiguous
           // bytes per warp store.
           if (ct) ct[(int64_t)q * g.ldct] = x;
+        }
+      }
+    }
+  }
+  if (failed) atomicOr(g.err, kErrSl);
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  if (warp == 0) tc::tmem_dealloc(tmem, S::TMEM_COLS);
+}
+
+// ------------------------------------------------ FP32 A, two slices each
+struct F32x2 {
+  static constexpr int BNMAX = 256, BK = 32, STAGES = 3, NB = 2;
+  static constexpr uint32_t RAW_BYTES = BM * BK * 4;              // A as FP32, 128-byte swizzle
+  static constexpr uint32_t A_SLICE = BM * BK * 2;                // its hi and lo slices, 64-byte swizzle
+  static constexpr uint32_t B_SLICE_MAX = BNMAX * BK * 2;
+  static constexpr uint32_t STAGE_BYTES = RAW_BYTES + 2 * A_SLICE + NB * B_SLICE_MAX;
+  static constexpr int SCALES = 4;  // K blocks of row scales kept
+  static constexpr size_t smem_bytes() { return 1024 + (size_t)STAGES * STAGE_BYTES + SCALES * BM * 4 + 256; }
+  static constexpr uint32_t TMEM_COLS = 2 * BNMAX;
+  static_assert(STAGES * STAGE_BYTES + SCALES * BM * 4 + 1280 <= 227 * 1024, "shared memory");
+};
+
+struct F32x2Args {
+  int64_t M, N, K;
+  void* C;
+  int64_t ldc;
+  const float* bscale;  // undoes the column scale of B's slices
+  float* Ct;            // optional FP32 copy of C transposed (N x M)
+  int64_t ldct;
+  int bn;               // tile width: a multiple of 16, at most 256
+  int b_upper;          // B[k][n] = 0 for k > n
+  int* err;
+};
+
+template <typename TC>
+__global__ void __launch_bounds__(kThreads, 1)
+    k_gemm_f32x2(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, F32x2Args g) {
+  using S = F32x2;
+  constexpr int BK = S::BK, STAGES = S::STAGES;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* base = smem_raw + ((1024 - (reinterpret_cast<uintptr_t>(smem_raw) & 1023)) & 1023);
+  float* rscale = reinterpret_cast<float*>(base + STAGES * S::STAGE_BYTES);  // [SCALES][BM]
+  uint64_t* full = reinterpret_cast<uint64_t*>(rscale + S::SCALES * BM);
+  uint64_t* ready = full + STAGES;  // A split
+  uint64_t* empty = ready + STAGES;
+  uint64_t* accf = empty + STAGES;  // [2]
+  uint64_t* accfree = accf + 2;     // [2]
+  uint64_t* drain = accfree + 2;    // every MMA issued has finished
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int bnw = g.bn;
+  const int64_t tn = (g.N + bnw - 1) / bnw;
+  const int64_t bm = (int64_t)blockIdx.x / tn, bn = (int64_t)blockIdx.x - bm * tn;
+  const int64_t m0 = bm * BM, n0 = bn * bnw;
+  const int64_t kmax = g.b_upper ? (g.K < n0 + bnw ? g.K : n0 + bnw) : g.K;
+  const int nkb = (int)((kmax + BK - 1) / BK);
+  const uint32_t bslice = (uint32_t)bnw * BK * 2;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&ready[s], 256);
+      mbar_init(&empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&accf[b], 1);
+      mbar_init(&accfree[b], 8);
+    }
+    mbar_init(drain, 1);
+    fence_mbar_init();
+  }
+  if (warp == 0) tc::tmem_alloc(tmem_slot, S::TMEM_COLS);
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  bool failed = false;
+
+  if (warp == 0) {
+    if (lane == 0) {  // TMA producer
+      int issued = 0;
+      for (int kb = 0; kb < nkb; ++kb) {
+        const int s = kb % STAGES, u = kb / STAGES;
+        if (u > 0 && !mbar_wait_bounded(&empty[s], (uint32_t)((u - 1) & 1), kWaitSl)) {
+          failed = true;
+          break;
+        }
+        unsigned char* p = base + (size_t)s * S::STAGE_BYTES;
+        mbar_arrive_expect_tx(&full[s], S::RAW_BYTES + S::NB * bslice);
+        tma_load_2d(p, &mapA, &full[s], kb * BK, (int32_t)m0);
+        tma_load_3d(p + S::RAW_BYTES + 2 * S::A_SLICE, &mapB, &full[s], kb * BK, (int32_t)n0, 0);
+        issued = kb + 1;
+      }
+      if (failed)
+        for (int kb = (issued > STAGES ? issued - STAGES : 0); kb < issued; ++kb)
+          if (!mbar_wait_bounded(&full[kb % STAGES], (uint32_t)((kb / STAGES) & 1), kWaitSl)) atomicOr(g.err, kErrSl);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {  // MMA issuer
+      const uint32_t idesc = idesc_f16(false, bnw);
+      for (int kb = 0; kb < nkb; ++kb) {
+        const int s = kb % STAGES, u = kb / STAGES, b = kb & 1;
+        if (!mbar_wait_bounded(&ready[s], (uint32_t)(u & 1), kWaitSl) ||
+            (kb >= 2 && !mbar_wait_bounded(&accfree[b], (uint32_t)(((kb >> 1) - 1) & 1), kWaitSl))) {
+          failed = true;
+          break;
+        }
+        tc::tc_fence_after();
+        const uint32_t a_hi = smem_u32(base + (size_t)s * S::STAGE_BYTES) + S::RAW_BYTES, a_lo = a_hi + S::A_SLICE;
+        const uint32_t b_hi = a_lo + S::A_SLICE, b_lo = b_hi + bslice;
+        const uint32_t d = tmem + (uint32_t)(b * S::BNMAX);
+        // The small terms first: the truncating additions then happen while
+        // the accumulator is small.
+#pragma unroll
+        for (int kk = 0; kk < BK / 16; ++kk)
+          mma_f16(d, desc_k<64>(a_hi + 32 * kk), desc_k<64>(b_lo + 32 * kk), idesc, kk > 0 ? 1u : 0u);
+#pragma unroll
+        for (int kk = 0; kk < BK / 16; ++kk)
+          mma_f16(d, desc_k<64>(a_lo + 32 * kk), desc_k<64>(b_hi + 32 * kk), idesc, 1u);
+#pragma unroll
+        for (int kk = 0; kk < BK / 16; ++kk)
+          mma_f16(d, desc_k<64>(a_hi + 32 * kk), desc_k<64>(b_hi + 32 * kk), idesc, 1u);
+        mma_commit(&empty[s]);
+        mma_commit(&accf[b]);
+      }
+      // Never free TMEM under MMAs that may still run.
+      mma_commit(drain);
+      if (!mbar_wait_bounded(drain, 0, kWaitSl)) atomicOr(g.err, kErrSl);
+    }
+  } else {
+    const int wq = warp & 3;
+    const int ch = (warp - 2) >> 2;  // column half: 128 columns of the tile
+    const uint32_t lane_base = tmem + ((uint32_t)(32 * wq) << 16) + (uint32_t)(128 * ch);
+    const int nc = min(128, max(0, bnw - 128 * ch));  // columns of this warp (uniform)
+    const int t = threadIdx.x - 64;
+    const int sr = t >> 1, sh2 = t & 1;  // split: row, half of its 32 values
+    float run[128];
+#pragma unroll
+    for (int i = 0; i < 128; ++i) run[i] = 0.f;
+    auto fold = [&](int kb) -> bool {
+      const bool ok = mbar_wait_bounded(&accf[kb & 1], (uint32_t)((kb >> 1) & 1), kWaitSl);
+      if (!__all_sync(0xffffffffu, ok)) return false;
+      tc::tc_fence_after();
+      const float rs = rscale[(kb % S::SCALES) * BM + 32 * wq + lane];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        if (16 * c < nc) {
+          float v[16];
+          tc::tmem_ld16(lane_base + (uint32_t)((kb & 1) * S::BNMAX + 16 * c), v);
+#pragma unroll
+          for (int q = 0; q < 16; ++q) run[16 * c + q] = fmaf(v[q], rs, run[16 * c + q]);
+        }
+      }
+      tc::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&accfree[kb & 1]);
+      return true;
+    };
+    for (int kb = 0; kb < nkb && !failed; ++kb) {
+      const int s = kb % STAGES, u = kb / STAGES;
+      const bool ok = mbar_wait_bounded(&full[s], (uint32_t)(u & 1), kWaitSl);
+      if (!__all_sync(0xffffffffu, ok)) {
+        failed = true;
+        break;
+      }
+      unsigned char* st = base + (size_t)s * S::STAGE_BYTES;
+      // Row sr: 128 bytes, 16-byte chunk q at q ^ (row & 7).
+      uint32_t x[16];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint4 v = *reinterpret_cast<const uint4*>(st + 128 * sr + 16 * ((4 * sh2 + q) ^ (sr & 7)));
+        x[4 * q] = v.x;
+        x[4 * q + 1] = v.y;
+        x[4 * q + 2] = v.z;
+        x[4 * q + 3] = v.w;
+      }
+      uint32_t mx = 0;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) mx = max(mx, x[q] & 0x7F800000u);
+      mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+      // Largest entry into [2^13, 2^14).
+      const int sh = min(max(140 - (int)(mx >> 23), -126), 126);
+      const float sc = __uint_as_float((uint32_t)(127 + sh) << 23);
+      if (sh2 == 0) rscale[(kb % S::SCALES) * BM + sr] = __uint_as_float((uint32_t)(127 - sh) << 23);
+      uint32_t hi[8], lo[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float a0 = __uint_as_float(x[2 * q]) * sc, a1 = __uint_as_float(x[2 * q + 1]) * sc;
+        const __half2 h = __floats2half2_rn(a0, a1);
+        const float2 f = __half22float2(h);
+        const __half2 r = __floats2half2_rn(a0 - f.x, a1 - f.y);
+        hi[q] = *reinterpret_cast<const uint32_t*>(&h);
+        lo[q] = *reinterpret_cast<const uint32_t*>(&r);
+      }
+      // FP16 row: 64 bytes, chunk q at q ^ ((row >> 1) & 3).
+      unsigned char* hp = st + S::RAW_BYTES + 64 * sr;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int o = 16 * ((2 * sh2 + q) ^ ((sr >> 1) & 3));
+        *reinterpret_cast<uint4*>(hp + o) = make_uint4(hi[4 * q], hi[4 * q + 1], hi[4 * q + 2], hi[4 * q + 3]);
+        *reinterpret_cast<uint4*>(hp + S::A_SLICE + o) = make_uint4(lo[4 * q], lo[4 * q + 1], lo[4 * q + 2], lo[4 * q + 3]);
+      }
+      fence_proxy_async_smem();
+      mbar_arrive(&ready[s]);
+      if (kb > 0 && !fold(kb - 1)) failed = true;
+    }
+    if (!failed && nkb > 0 && !fold(nkb - 1)) failed = true;
+    const int64_t row = m0 + 32 * wq + lane;
+    const int64_t c0 = n0 + 128 * ch;
+    const int64_t left = g.N - c0;
+    const int ncol = (int)(left < nc ? left : nc);
+    if (row < g.M && ncol > 0) {
+      TC* dst = static_cast<TC*>(g.C) + row * g.ldc + c0;
+      float* ct = g.Ct ? g.Ct + c0 * g.ldct + row : nullptr;
+#pragma unroll
+      for (int q = 0; q < 128; ++q) {
+        if (q < ncol) {
+          const float v = failed ? __int_as_float(0x7fc00000) : run[q] * __ldg(g.bscale + c0 + q);
+          dst[q] = (TC)v;
+          if (ct) ct[(int64_t)q * g.ldct] = v;
         }
       }
     }

@@ -82,6 +82,11 @@ int tall_gemm(const Dla& d, Arena& ar, DT ta, DT tc, DT tout, int64_t M, int64_t
         if (st != BSRHT_OK && st != BSRHT_EUNSUP) return st;
       }
     }
+    if (!ar.lean && ta == DT::F32 && tc == DT::F32 && gemm_f32x2_eligible(M, N, K, nullptr, lda)) {
+      const int st = gemm_f32x2(d, ar, M, N, K, nullptr, lda, DT::F64, nullptr, ldb, tout, nullptr, ldc, tri_b, nullptr);
+      ar.release(mk);
+      if (st != BSRHT_OK) return st;
+    }
     if (!ar.lean && tc == DT::F32 && tout == DT::F32 && gemm_a16_eligible(ta, M, N, K, nullptr, lda)) {
       const int st = gemm_a16(d, ar, ta, M, N, K, nullptr, lda, DT::F64, nullptr, ldb, nullptr, ldc, Ct);
       ar.release(mk);
@@ -97,6 +102,15 @@ int tall_gemm(const Dla& d, Arena& ar, DT ta, DT tc, DT tout, int64_t M, int64_t
     const int st = gemm_a16(d, ar, ta, M, N, K, A, lda, DT::F64, B64, ldb, static_cast<float*>(C), ldc, Ct);
     ar.release(mk);
     if (st == BSRHT_OK && ct_done) *ct_done = Ct != nullptr;
+    if (st != BSRHT_EUNSUP) return st;
+  }
+  if (ta == DT::F32 && tc == DT::F32 && B64 != nullptr && gemm_f32x2_eligible(M, N, K, A, lda)) {
+    const size_t mk = ar.mark();
+    float* ct = tout == DT::F32 ? Ct : nullptr;
+    const int st = gemm_f32x2(d, ar, M, N, K, static_cast<const float*>(A), lda, DT::F64, B64, ldb, tout, C, ldc, tri_b,
+                              ct);
+    ar.release(mk);
+    if (st == BSRHT_OK && ct_done) *ct_done = ct != nullptr;
     if (st != BSRHT_EUNSUP) return st;
   }
   if (ta == DT::F32 && use_tc(tc, M, N, K, A, lda) && B64 != nullptr) {
