@@ -105,6 +105,7 @@ int gemm_launch(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const 
   if (tiles < target && K > kMinK) {
     splits = (int)std::min<int64_t>((target + tiles - 1) / tiles, K / kMinRange);
     splits = std::max(1, std::min(splits, 64));
+    splits = (int)ar.parts_that_fit(splits, sizeof(Tacc) * (size_t)M * N);
   }
   // Row and column tiles on one grid dimension (the y dimension's 65535
   // would cap M at about 4 million rows).

@@ -34,6 +34,16 @@ struct Arena {
   size_t mark() const { return used; }
   void release(size_t m) { used = m; }
   bool ok() const { return measure || used <= cap; }
+  // Parts (wanted, at least `least`) of `bytes` each that a product split over
+  // K may use.  Scratch is measured at a call's full widths; a narrower
+  // product met on the way (repeated rows dropped, leading columns only) has
+  // fewer tiles and would split further than what was measured for it.
+  int64_t parts_that_fit(int64_t wanted, size_t bytes, int64_t least = 1) const {
+    if (measure) return wanted;
+    const size_t from = (used + 255) / 256 * 256, room = cap > from ? cap - from : 0;
+    const int64_t fit = (int64_t)(room / (bytes ? bytes : 1));
+    return wanted <= fit ? wanted : (fit > least ? fit : least);
+  }
 };
 
 struct Dla {

@@ -163,12 +163,15 @@ int gemm_tc(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const floa
   splits = std::max<int64_t>(splits, (nkb + 255) / 256);
   if (gram && splits == 1) splits = 2;  // the mirror is applied by the reduce
   splits = std::min<int64_t>(splits, 65535);
+  int* err = static_cast<int*>(ar.take(256));
+  if (splits > 1)
+    splits = ar.parts_that_fit(splits, sizeof(float) * (size_t)M * N,
+                               std::max<int64_t>(gram ? 2 : 1, (nkb + 255) / 256));
   float* P = nullptr;
   if (splits > 1) {
     P = static_cast<float*>(ar.take(sizeof(float) * (size_t)splits * M * N));
     if (!ar.ok()) return BSRHT_ENOMEM;
   }
-  int* err = static_cast<int*>(ar.take(256));
   if (!ar.ok()) return BSRHT_ENOMEM;
   if (ar.measure) return BSRHT_OK;
   CUtensorMap ma, mb, mblo;
