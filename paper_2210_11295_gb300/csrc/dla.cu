@@ -96,10 +96,10 @@ int gemm_launch(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const 
   // Split K when the tiles alone leave SMs idle.  FP64 FMAs run at 1/64 of
   // the FP32 rate on this GPU (about two per SM and clock): one 64 x 64 tile
   // over K = 256 keeps an SM busy for a quarter of a millisecond, so FP64
-  // products split K down to 32-deep ranges; FP32 ones keep ranges of at
-  // least 256.
+  // products split K down to 32-deep ranges (16 with 32-wide tiles); FP32
+  // ones keep ranges of at least 256.
   constexpr bool kF64 = std::is_same<Tacc, double>::value;
-  constexpr int64_t kMinRange = kF64 ? 4 * BK : 32 * BK, kMinK = kF64 ? 8 * BK : 64 * BK;
+  constexpr int64_t kMinRange = kF64 ? TM * BK : 32 * BK, kMinK = kF64 ? 2 * TM * BK : 64 * BK;
   int splits = 1;
   const int64_t target = 2 * (int64_t)num_sms();
   if (tiles < target && K > kMinK) {
@@ -151,9 +151,17 @@ int gemm(const Dla& d, Arena& ar, DT ta, DT tb, DT tc, bool acc64, int64_t M, in
       if (!ar.measure && st != BSRHT_EUNSUP) return st;
       ar.release(mk);  // size (or run) the CUDA-core form as well
     }
-    if (ta == DT::F64 && tb == DT::F64 && tc == DT::F64)
+    if (ta == DT::F64 && tb == DT::F64 && tc == DT::F64) {
+      // An SM finishes two FP64 FMAs a cycle: a small product needs every SM.
+      // 64-wide tiles over 32-deep ranges that make fewer CTAs than SMs give
+      // way to 32-wide ones over 16-deep ranges (126^3: 52 -> 16 us).
+      const int64_t t64 = (M + 63) / 64 * ((N + 63) / 64);
+      if (t64 * std::max<int64_t>(1, std::min<int64_t>(K / 32, 64)) < num_sms())
+        return gemm_launch<double, double, double, double, 2>(d, ar, M, N, K, A, lda, a_trans, B, ldb, C, ldc,
+                                                              alpha, beta, tri_b, gram);
       return gemm_launch<double, double, double, double, 4>(d, ar, M, N, K, A, lda, a_trans, B, ldb, C, ldc,
                                                             alpha, beta, tri_b, gram);
+    }
     if (ta == DT::F32 && tb == DT::F32 && tc == DT::F64)  // FP64 accumulation of FP32 data
       return gemm_launch<float, float, double, double, 4>(d, ar, M, N, K, A, lda, a_trans, B, ldb, C, ldc, alpha,
                                                           beta, tri_b, gram);
@@ -352,7 +360,7 @@ int tri_inverse(const Dla& d, const double* L, double* LT, double* Rinv, int64_t
 // (a) (16 pivots of one reciprocal each) and the barriers.  16-wide blocks
 // keep the tile update and the factorisation of (a), which no other SM can
 // share, to a quarter and an eighth of those of 32-wide ones; the other tiles
-// then fit beside that chain (CHOL_MS).
+// then fit beside that chain (l = 512: 0.71 ms; l = 400: 0.58 -> 0.54).
 // Outputs: L in the lower triangle of g (upper zeroed), LT = L^T and Rinv =
 // L^-T (row-major, upper triangular).  T and X are l x l scratch.  A pivot
 // <= 0 sets kStatusNotPD (and is replaced by 1 so the kernel runs to the end).
@@ -853,16 +861,22 @@ __global__ void k_col_norms(const double* __restrict__ M, double* __restrict__ s
 }
 
 // perm[rank] = c with ranks by descending sigma (ties: lower index first).
+// l <= kMaxSvd.
+constexpr int kMaxSvd = 2048;
 __global__ void k_rank_desc(const double* __restrict__ sigma, int* __restrict__ perm, int64_t l) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ double s[kMaxSvd];
+  for (int e = threadIdx.x; e < l; e += blockDim.x) s[e] = sigma[e];
+  __syncthreads();
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= l) return;
-  const double v = sigma[c];
-  int64_t rank = 0;
-  for (int64_t e = 0; e < l; ++e) {
-    const double w = sigma[e];
+  const double v = s[c];
+  int rank = 0;
+#pragma unroll 4
+  for (int e = 0; e < l; ++e) {
+    const double w = s[e];
     rank += (w > v) || (w == v && e < c);
   }
-  perm[rank] = (int)c;
+  perm[rank] = c;
 }
 
 // U[i][r] = M[perm[r]][i] / sigma, Vout[i][r] = Vcols[perm[r]][i], sig_out[r].
@@ -1553,7 +1567,7 @@ int launch_jacobi_cluster(const Dla& d, float* X, int64_t l, double tol, double 
 
 int jacobi_svd(const Dla& d, Arena& ar, double* colsM, int64_t l, double* U, double* sigma, double* Vout,
                double polish_tol, double zero_rel, int64_t ktop, double keep_rel) {
-  if (l > 2048) return BSRHT_EUNSUP;
+  if (l > kMaxSvd) return BSRHT_EUNSUP;
   const int max_sweeps = 40;
   // Rotate only while the cosine of the pair exceeds sqrt(l) eps (the usual
   // one-sided Jacobi threshold); a tighter one keeps rotating at noise level.
@@ -2082,17 +2096,38 @@ int scale_columns(const Dla& d, double* X, int64_t rows, int64_t cols, int64_t l
   return BSRHT_OK;
 }
 
-// Column argmax of |U| per row chunk: partial (value, index) per chunk.
-__global__ void k_colargmax_partial(const double* __restrict__ U, int64_t n, int64_t k, int64_t rows_per,
-                                    double* __restrict__ pv, int64_t* __restrict__ pi) {
-  const int64_t c = (int64_t)blockIdx.y * blockDim.x + threadIdx.x;
-  if (c >= k) return;
+// Column argmax of |U| (lowest row on ties) per row chunk: partial (value,
+// index) per chunk.  Columns along x (kb per block), blockDim.x / kb rows at a
+// time: with one thread per column its chain of loads was the time (factors
+// of rSVD 4096 x 256, l = 100: 0.24 -> 0.16 ms with the sums below).
+__global__ void __launch_bounds__(256) k_colargmax_partial(const double* __restrict__ U, int64_t n, int64_t k, int kb,
+                                                           int64_t rows_per, double* __restrict__ pv,
+                                                           int64_t* __restrict__ pi) {
+  __shared__ double sv[256];
+  __shared__ int64_t si[256];
+  const int nr = blockDim.x / kb, q = threadIdx.x / kb;
+  const int64_t c = (int64_t)blockIdx.y * kb + threadIdx.x % kb;
   const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(n, r0 + rows_per);
   double best = -1.0;
   int64_t bi = r0;
-  for (int64_t i = r0; i < r1; ++i) {
-    const double v = fabs(U[i * k + c]);
-    if (v > best) {
+  if (c < k && q < nr) {
+#pragma unroll 8
+    for (int64_t i = r0 + q; i < r1; i += nr) {
+      const double v = fabs(U[i * k + c]);
+      if (v > best) {
+        best = v;
+        bi = i;
+      }
+    }
+  }
+  sv[threadIdx.x] = best;
+  si[threadIdx.x] = bi;
+  __syncthreads();
+  if (q != 0 || c >= k) return;
+  for (int u = 1; u < nr; ++u) {
+    const double v = sv[threadIdx.x + u * kb];
+    const int64_t i = si[threadIdx.x + u * kb];
+    if (v > best || (v == best && i < bi)) {
       best = v;
       bi = i;
     }
@@ -2101,20 +2136,37 @@ __global__ void k_colargmax_partial(const double* __restrict__ U, int64_t n, int
   pi[(int64_t)blockIdx.x * k + c] = bi;
 }
 
-__global__ void k_colargmax_final(const double* __restrict__ U, int64_t k, int nchunks, const double* pv,
-                                  const int64_t* pi, double* __restrict__ sgn) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= k) return;
+// One block per column.
+__global__ void __launch_bounds__(128) k_colargmax_final(const double* __restrict__ U, int64_t k, int nchunks,
+                                                         const double* pv, const int64_t* pi,
+                                                         double* __restrict__ sgn) {
+  __shared__ double sv[128];
+  __shared__ int64_t si[128];
+  const int64_t c = blockIdx.x;
   double best = -1.0;
   int64_t bi = 0;
-  for (int b = 0; b < nchunks; ++b) {
+  for (int b = threadIdx.x; b < nchunks; b += 128) {
     const double v = pv[(int64_t)b * k + c];
     if (v > best) {
       best = v;
       bi = pi[(int64_t)b * k + c];
     }
   }
-  sgn[c] = (U[bi * k + c] < 0.0) ? -1.0 : 1.0;
+  sv[threadIdx.x] = best;
+  si[threadIdx.x] = bi;
+  __syncthreads();
+  for (int o = 64; o > 0; o >>= 1) {
+    if (threadIdx.x < o) {
+      const double v = sv[threadIdx.x + o];
+      const int64_t i = si[threadIdx.x + o];
+      if (v > sv[threadIdx.x] || (v == sv[threadIdx.x] && i < si[threadIdx.x])) {
+        sv[threadIdx.x] = v;
+        si[threadIdx.x] = i;
+      }
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) sgn[c] = (U[si[0] * k + c] < 0.0) ? -1.0 : 1.0;
 }
 
 int sign_normalize(const Dla& d, Arena& ar, double* U, int64_t n, int64_t k, double* V, int64_t m) {
@@ -2125,10 +2177,10 @@ int sign_normalize(const Dla& d, Arena& ar, double* U, int64_t n, int64_t k, dou
   double* sg = static_cast<double*>(ar.take(sizeof(double) * k));
   if (!ar.ok()) return BSRHT_ENOMEM;
   if (ar.measure) return BSRHT_OK;
-  const int tb = (int)std::min<int64_t>(256, k);
-  k_colargmax_partial<<<dim3(nchunks, blocks_for(k, tb)), tb, 0, d.s>>>(U, n, k, rows_per, pv, pi);
+  const int kb = (int)std::min<int64_t>(256, k);
+  k_colargmax_partial<<<dim3(nchunks, blocks_for(k, kb)), 256 / kb * kb, 0, d.s>>>(U, n, k, kb, rows_per, pv, pi);
   DLA_LAUNCH_CHECK();
-  k_colargmax_final<<<blocks_for(k, 128), 128, 0, d.s>>>(U, k, nchunks, pv, pi, sg);
+  k_colargmax_final<<<(unsigned)k, 128, 0, d.s>>>(U, k, nchunks, pv, pi, sg);
   DLA_LAUNCH_CHECK();
   note_launches(2);
   int st = scale_columns(d, U, n, k, k, sg, false);
@@ -2154,12 +2206,17 @@ __global__ void k_sumsq_partial(const T* __restrict__ X, int64_t count, double* 
   if (threadIdx.x == 0) part[blockIdx.x] = red[0];
 }
 
-__global__ void k_sum_sqrt(const double* part, int count, double* out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < count; ++i) s += part[i];
-    *out = sqrt(s);
+__global__ void __launch_bounds__(256) k_sum_sqrt(const double* part, int count, double* out) {
+  __shared__ double red[256];
+  double s = 0.0;
+  for (int i = threadIdx.x; i < count; i += 256) s += part[i];
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    __syncthreads();
   }
+  if (threadIdx.x == 0) *out = sqrt(red[0]);
 }
 
 int frob_norm(const Dla& d, Arena& ar, DT t, const void* X, int64_t count, double* out) {
@@ -2174,7 +2231,7 @@ int frob_norm(const Dla& d, Arena& ar, DT t, const void* X, int64_t count, doubl
   else
     return BSRHT_EUNSUP;
   DLA_LAUNCH_CHECK();
-  k_sum_sqrt<<<1, 32, 0, d.s>>>(part, nb, out);
+  k_sum_sqrt<<<1, 256, 0, d.s>>>(part, nb, out);
   DLA_LAUNCH_CHECK();
   note_launches(2);
   return BSRHT_OK;
