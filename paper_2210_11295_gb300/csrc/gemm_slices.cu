@@ -181,9 +181,10 @@ bool make_slice_map(CUtensorMap* map, const void* base, CUtensorMapDataType dt, 
 int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
 unsigned row_parts(int64_t K, int64_t col_blocks) {
-  // Enough CTAs to fill the GPU, at least 64 rows each.
+  // Enough CTAs to fill the GPU, at least 16 rows each (a thread's loads
+  // follow one another).
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>((4 * (int64_t)num_sms() + col_blocks - 1) / col_blocks,
-                                                          (K + 63) / 64));
+                                                          (K + 15) / 16));
 }
 
 int digits_rows(const Dla& d, const double* A, int64_t rows, int64_t K, int64_t lda, uint32_t* out, int64_t ldk,
@@ -424,9 +425,10 @@ int gemm_a16(const Dla& d, Arena& ar, DT ta, int64_t M, int64_t N, int64_t K, co
 }
 
 // Tiles enough for most SMs (the other kernel splits K instead), wide enough
-// to gain on the split of A, and a K chain of at most 256 folds.
+// to gain on the split of A, K long against the epilogue and short enough for
+// a chain of at most 256 folds.
 bool gemm_f32x2_eligible(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda) {
-  return M >= 128 * 96 && N >= 48 && K >= 32 && K <= 8192 && (lda % 4) == 0 &&
+  return M >= 128 * 96 && N >= 128 && K >= 1024 && K <= 8192 && (lda % 4) == 0 &&
          (reinterpret_cast<uintptr_t>(A) % 16) == 0;
 }
 

@@ -90,3 +90,23 @@ def test_rsvd_16bit_matches_oracle(lib, dtype, n, m, ld, l):
     ref = (ur * sr) @ vr.T
     assert np.max(np.abs(s.cpu().numpy() - sr)) <= 1e-5 * sr[0]
     assert np.linalg.norm(_rank_k(u, s, v) - ref) <= 1e-5 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n,m,ld,l", [
+    (12300, 1028, 1028, 130),  # ragged rows, two column tiles, ragged last K block
+    (12288, 1024, 1024, 128),  # exact tiles, at the edge of the rule
+    (12290, 2000, 2048, 257),  # column slice, one column past two tiles
+    (12290, 1026, 1026, 130),  # rows off 16 bytes: the TF32 product
+])
+def test_rsvd_f32_matches_oracle(lib, n, m, ld, l):
+    a, _ = synth.haar_spectrum(n, m, seed=n + m, decay=20.0)
+    rng = np.random.default_rng(l)
+    buf = torch.zeros(n, ld)
+    # Rows 2^-40 .. 1 apart: each is split under its own scale.
+    buf[:, :m] = torch.from_numpy(a * np.exp2(rng.integers(-40, 1, size=(n, 1))))
+    x = buf.cuda()[:, :m]
+    u, s, v = lib.bsrht_rsvd(x, 10, l, 4, 5)
+    ur, sr, vr = orc.rsvd(x.double().cpu().numpy(), 10, l, 4, 5)
+    ref = (ur * sr) @ vr.T
+    assert np.max(np.abs(s.cpu().numpy() - sr)) <= 1e-5 * sr[0]
+    assert np.linalg.norm(_rank_k(u, s, v) - ref) <= 1e-5 * np.linalg.norm(ref)
