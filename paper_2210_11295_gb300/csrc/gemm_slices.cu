@@ -173,9 +173,9 @@ __global__ void k_col_exps32(const TB* __restrict__ B, int64_t K, int64_t N, int
 
 // 3-D map [planes][rows][k] of 16-bit K-major slices, rows of ldk elements.
 bool make_slice_map(CUtensorMap* map, const void* base, CUtensorMapDataType dt, int64_t k, int64_t rows, int planes,
-                    int64_t ldk, uint32_t box_k, uint32_t box_rows, CUtensorMapSwizzle swz) {
+                    int64_t ldk, uint32_t box_k, uint32_t box_rows, CUtensorMapSwizzle swz, int box_planes) {
   return make_tensor_map_3d(map, base, dt, 2, (uint64_t)k, (uint64_t)rows, (uint64_t)planes, (uint64_t)ldk,
-                            (uint64_t)(ldk * rows), box_k, box_rows, (uint32_t)planes, swz);
+                            (uint64_t)(ldk * rows), box_k, box_rows, (uint32_t)box_planes, swz);
 }
 
 int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
@@ -310,8 +310,8 @@ int gemm_int8x7(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const 
   const CUtensorMapSwizzle swz = CU_TENSOR_MAP_SWIZZLE_64B;
   auto launch = [&](int64_t m, int64_t k, double* out, int64_t ldo, int z) -> int {
     CUtensorMap ma, mb;
-    if (!make_slice_map(&ma, ad, f16, k, m, kDig, ldk, S::BK, sl::BM, swz) ||
-        !make_slice_map(&mb, bd, f16, k, N, kDig, ldk, S::BK, S::BN, swz))
+    if (!make_slice_map(&ma, ad, f16, k, m, kDig, ldk, S::BK, sl::BM, swz, kDig) ||
+        !make_slice_map(&mb, bd, f16, k, N, kDig, ldk, S::BK, S::BN, swz, kDig))
       return BSRHT_EUNSUP;
     const int64_t tiles = (m + sl::BM - 1) / sl::BM * tn;
     if (tiles > 0x7FFFFFFF) return BSRHT_EUNSUP;
@@ -413,7 +413,8 @@ int gemm_a16(const Dla& d, Arena& ar, DT ta, int64_t M, int64_t N, int64_t K, co
   CUtensorMap ma, mb;
   if (!make_tensor_map_2d(&ma, A, dt, 2, (uint64_t)M, (uint64_t)K, (uint64_t)lda, S::BK, sl::BM,
                           CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !make_slice_map(&mb, b.slices, dt, K, N, S::NB, b.ldk, S::BK, (uint32_t)b.bn, CU_TENSOR_MAP_SWIZZLE_128B))
+      !make_slice_map(&mb, b.slices, dt, K, N, S::NB, b.ldk, S::BK, (uint32_t)b.bn, CU_TENSOR_MAP_SWIZZLE_128B,
+                      S::NB))
     return BSRHT_EUNSUP;
   BSRHT_CUDA_TRY(
       cudaFuncSetAttribute(sl::k_gemm_a16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_bytes()));
@@ -425,10 +426,12 @@ int gemm_a16(const Dla& d, Arena& ar, DT ta, int64_t M, int64_t N, int64_t K, co
 }
 
 // Tiles enough for most SMs (the other kernel splits K instead), wide enough
-// to gain on the split of A, K long against the epilogue and short enough for
-// a chain of at most 256 folds.
+// to gain on the split of A, K short enough for a chain of at most 256 folds,
+// and long against the start and the stores of a tile, which nothing overlaps:
+// 65536 x 2000 x 400 0.45 ms against 0.70 in TF32, but 2^20 x 512 x 512 (upper
+// triangular) 2.8 ms in both and 2^20 x 512 x 100 1.4 against 1.2.
 bool gemm_f32x2_eligible(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda) {
-  return M >= 128 * 96 && N >= 128 && K >= 1024 && K <= 8192 && (lda % 4) == 0 &&
+  return M >= 128 * 96 && N >= 128 && K >= 1024 && K <= 256 * 64 && (lda % 4) == 0 &&
          (reinterpret_cast<uintptr_t>(A) % 16) == 0;
 }
 
@@ -440,18 +443,19 @@ int gemm_f32x2(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const f
   SlicedB b;
   TRY_SL((slice_b<__half, S::NB>(d, ar, K, N, tb, B, ldb, &b)));
   if (ar.measure) return BSRHT_OK;
-  const int64_t tiles = (M + sl::BM - 1) / sl::BM * ((N + b.bn - 1) / b.bn);
+  // Pairs of row tiles.
+  const int64_t tiles = 2 * ((M + 2 * sl::BM - 1) / (2 * sl::BM)) * ((N + b.bn - 1) / b.bn);
   if (tiles > 0x7FFFFFFF) return BSRHT_EUNSUP;
   CUtensorMap ma, mb;
   if (!make_tensor_map_2d(&ma, A, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, (uint64_t)M, (uint64_t)K, (uint64_t)lda, S::BK,
                           sl::BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !make_slice_map(&mb, b.slices, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, K, N, S::NB, b.ldk, S::BK, (uint32_t)b.bn,
-                      CU_TENSOR_MAP_SWIZZLE_64B))
+      !make_slice_map(&mb, b.slices, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, K, N, S::NB, b.ldk, S::BK,
+                      (uint32_t)b.bn / 2, CU_TENSOR_MAP_SWIZZLE_64B, 1))
     return BSRHT_EUNSUP;
   sl::F32x2Args g{M, N, K, C, ldc, b.scale, Ct, M, b.bn, b_upper ? 1 : 0, d.status};
   auto launch = [&](auto kern) -> int {
     BSRHT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_bytes()));
-    kern<<<(unsigned)tiles, sl::kThreads, S::smem_bytes(), d.s>>>(ma, mb, g);
+    kern<<<(unsigned)tiles, S::THREADS, S::smem_bytes(), d.s>>>(ma, mb, g);
     BSRHT_CUDA_TRY(cudaGetLastError());
     note_launches(1);
     return BSRHT_OK;

@@ -29,12 +29,16 @@
 // pair holds as much of an FP32 value as a TF32 pair (11 + 11 bits) once it is
 // scaled into FP16's range, and the 16-bit MMA is twice as fast and reads
 // half the shared memory.  B is split once in global memory (two slices,
-// scaled per column); the fold warps split each staged tile of A, one
-// power-of-two scale per row and K block of 32, and undo that scale when they
-// add the block to their FP32 sums: hi lo + lo hi + hi hi, smallest first;
+// scaled per column); four warps split each staged tile of A in place, one
+// power-of-two scale per row and 64 of K, which the 16 fold warps undo when
+// they add the 64 to their FP32 sums: hi lo + lo hi + hi hi, smallest first;
 // what is dropped lies below 2^-23 of each product, or 2^-38 of the row's
-// largest entry in the block.  Bound by shared memory (copies in, split,
-// operand reads: 152 KB a K block against 768 cycles of MMA).
+// largest entry in the 64.  Two CTAs (row tiles of one column tile) load half
+// of B each for both.  2^18 x 4096 x 512: 3.0 ms (TF32 form 4.5).  Without the
+// split and the fold it takes 2.2 ms, without two of the three MMAs as well
+// 1.9 ms (copies from L2, 9 TB/s): no single part bounds it, but their use of
+// shared memory, 152 KB per 32 of K against 768 clocks of MMA.  Measured on the
+// way: the fold warps splitting too, 3.9 ms; folding every 32 of K, 3.3 ms.
 #pragma once
 
 #include <cuda.h>
@@ -64,6 +68,26 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
+// The same into both CTAs of a pair: the copy and its byte count arrive at the
+// same offsets of each one's shared memory.
+__device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* map, uint64_t* bar, int32_t x,
+                                                 int32_t y, int32_t z) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster [%0], "
+      "[%1, {%3, %4, %5}], [%2], %6;" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z), "h"((uint16_t)3)
+      : "memory");
+}
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // K-major operand descriptors: rows of 128 bytes (128-byte swizzle, 8-row
 // atoms 1024 bytes apart) or 64 bytes (64-byte swizzle, 512 bytes apart).
 template <int ROW_BYTES>
@@ -90,6 +114,14 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
           d_tmem),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
+      : "memory");
+}
+// Commit that arrives at the same barrier of both CTAs of a pair.
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          smem_u32(bar)),
+      "h"((uint16_t)3)
       : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
@@ -357,6 +389,45 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0) tc::tmem_dealloc(tmem, S::TMEM_COLS);
 }
 
+// Stores a warp's 32 x NC piece of C (row0 + lane in v, columns scaled by
+// bscale; NaN if failed): through shared memory
+// (buf, 32 rows of NC + 4 words), so that every store covers whole sectors
+// whatever ldc and C's alignment are; straight from the registers each
+// instruction would touch 32 rows.  ct: the transposed copy, 128 bytes a store
+// as it stands.
+template <int NC>
+constexpr uint32_t store_buf_bytes() {
+  return 32 * (NC + 4) * 4;
+}
+template <typename TC, int NC>
+__device__ __forceinline__ void store_warp_tile(const float (&v)[NC], float* buf, TC* C, int64_t ldc, float* Ct,
+                                                int64_t ldct, int64_t row0, int64_t M, int64_t c0, int ncol,
+                                                const float* bscale, bool failed) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int q = 0; q < NC; q += 4)
+    *reinterpret_cast<float4*>(buf + lane * (NC + 4) + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+  __syncwarp();
+  const int rows = (int)(M - row0 < 32 ? M - row0 : 32);
+  const float nan = __int_as_float(0x7fc00000);
+  float sc[NC / 32];
+#pragma unroll
+  for (int c = 0; c < NC / 32; ++c) sc[c] = failed ? nan : 32 * c + lane < ncol ? __ldg(bscale + c0 + 32 * c + lane) : 0.f;
+  TC* dst = C + row0 * ldc + c0;
+#pragma unroll 4
+  for (int r = 0; r < rows; ++r) {
+#pragma unroll
+    for (int c = 0; c < NC / 32; ++c)
+      if (32 * c + lane < ncol) dst[r * ldc + 32 * c + lane] = (TC)(buf[r * (NC + 4) + 32 * c + lane] * sc[c]);
+  }
+  if (Ct && lane < rows) {
+    float* ct = Ct + c0 * ldct + row0 + lane;
+#pragma unroll
+    for (int q = 0; q < NC; ++q)
+      if (q < ncol) ct[(int64_t)q * ldct] = failed ? nan : v[q] * __ldg(bscale + c0 + q);
+  }
+}
+
 // --------------------------------------------- 16-bit A, B in three slices
 struct A16 {
   static constexpr int BNMAX = 256, BK = 64, STAGES = 2, NB = 3;
@@ -524,15 +595,17 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // ------------------------------------------------ FP32 A, two slices each
 struct F32x2 {
-  static constexpr int BNMAX = 256, BK = 32, STAGES = 3, NB = 2;
-  static constexpr uint32_t RAW_BYTES = BM * BK * 4;              // A as FP32, 128-byte swizzle
-  static constexpr uint32_t A_SLICE = BM * BK * 2;                // its hi and lo slices, 64-byte swizzle
+  static constexpr int BNMAX = 256, BK = 32, STAGES = 4, NB = 2;
+  static constexpr uint32_t A_BYTES = BM * BK * 4;  // rows of 128 bytes: FP32, then hi | lo
   static constexpr uint32_t B_SLICE_MAX = BNMAX * BK * 2;
-  static constexpr uint32_t STAGE_BYTES = RAW_BYTES + 2 * A_SLICE + NB * B_SLICE_MAX;
-  static constexpr int SCALES = 4;  // K blocks of row scales kept
-  static constexpr size_t smem_bytes() { return 1024 + (size_t)STAGES * STAGE_BYTES + SCALES * BM * 4 + 256; }
+  static constexpr uint32_t STAGE_BYTES = A_BYTES + NB * B_SLICE_MAX;
+  static constexpr int RING = 8;  // K blocks whose split is remembered; half as many row scales
+  static constexpr int SPLIT_WARPS = 4, FOLD_WARPS = 16, NC = 64;
+  static constexpr int THREADS = 32 * (2 + SPLIT_WARPS + FOLD_WARPS);
+  static constexpr size_t smem_bytes() { return 1024 + (size_t)STAGES * STAGE_BYTES + RING / 2 * BM * 4 + 256; }
   static constexpr uint32_t TMEM_COLS = 2 * BNMAX;
-  static_assert(STAGES * STAGE_BYTES + SCALES * BM * 4 + 1280 <= 227 * 1024, "shared memory");
+  static_assert(STAGES * STAGE_BYTES + RING / 2 * BM * 4 + 1280 <= 227 * 1024, "shared memory");
+  static_assert(FOLD_WARPS * store_buf_bytes<NC>() <= STAGES * STAGE_BYTES, "the stages hold the stored tile");
 };
 
 struct F32x2Args {
@@ -548,25 +621,27 @@ struct F32x2Args {
 };
 
 template <typename TC>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32x2::THREADS, 1)
     k_gemm_f32x2(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, F32x2Args g) {
   using S = F32x2;
-  constexpr int BK = S::BK, STAGES = S::STAGES;
+  constexpr int BK = S::BK, STAGES = S::STAGES, RING = S::RING;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = smem_raw + ((1024 - (reinterpret_cast<uintptr_t>(smem_raw) & 1023)) & 1023);
-  float* rscale = reinterpret_cast<float*>(base + STAGES * S::STAGE_BYTES);  // [SCALES][BM]
-  uint64_t* full = reinterpret_cast<uint64_t*>(rscale + S::SCALES * BM);
-  uint64_t* ready = full + STAGES;  // A split
-  uint64_t* empty = ready + STAGES;
+  float* rscale = reinterpret_cast<float*>(base + STAGES * S::STAGE_BYTES);  // [RING / 2][BM]
+  uint64_t* full = reinterpret_cast<uint64_t*>(rscale + RING / 2 * BM);
+  uint64_t* ready = full + STAGES;  // [RING]: A split, row scales written
+  uint64_t* empty = ready + RING;
   uint64_t* accf = empty + STAGES;  // [2]
   uint64_t* accfree = accf + 2;     // [2]
   uint64_t* drain = accfree + 2;    // every MMA issued has finished
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_rank();
   const int bnw = g.bn;
   const int64_t tn = (g.N + bnw - 1) / bnw;
-  const int64_t bm = (int64_t)blockIdx.x / tn, bn = (int64_t)blockIdx.x - bm * tn;
+  // The pair's two row tiles share one column tile.
+  const int64_t pair = (int64_t)blockIdx.x >> 1, bm = 2 * (pair / tn) + rank, bn = pair % tn;
   const int64_t m0 = bm * BM, n0 = bn * bnw;
   const int64_t kmax = g.b_upper ? (g.K < n0 + bnw ? g.K : n0 + bnw) : g.K;
   const int nkb = (int)((kmax + BK - 1) / BK);
@@ -575,12 +650,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&ready[s], 256);
-      mbar_init(&empty[s], 1);
+      mbar_init(&empty[s], 2);
     }
+    for (int s = 0; s < RING; ++s) mbar_init(&ready[s], S::SPLIT_WARPS);
     for (int b = 0; b < 2; ++b) {
       mbar_init(&accf[b], 1);
-      mbar_init(&accfree[b], 8);
+      mbar_init(&accfree[b], S::FOLD_WARPS);
     }
     mbar_init(drain, 1);
     fence_mbar_init();
@@ -588,12 +663,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0) tc::tmem_alloc(tmem_slot, S::TMEM_COLS);
   tc::tc_fence_before();
   __syncthreads();
+  cluster_sync_all();  // the peer's barriers exist before anything arrives at them
   tc::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   bool failed = false;
 
   if (warp == 0) {
-    if (lane == 0) {  // TMA producer
+    if (lane == 0) {  // TMA producer: own rows of A, half of B for both CTAs
       int issued = 0;
       for (int kb = 0; kb < nkb; ++kb) {
         const int s = kb % STAGES, u = kb / STAGES;
@@ -602,9 +678,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           break;
         }
         unsigned char* p = base + (size_t)s * S::STAGE_BYTES;
-        mbar_arrive_expect_tx(&full[s], S::RAW_BYTES + S::NB * bslice);
+        mbar_arrive_expect_tx(&full[s], S::A_BYTES + S::NB * bslice);
         tma_load_2d(p, &mapA, &full[s], kb * BK, (int32_t)m0);
-        tma_load_3d(p + S::RAW_BYTES + 2 * S::A_SLICE, &mapB, &full[s], kb * BK, (int32_t)n0, 0);
+#pragma unroll
+        for (int q = 0; q < S::NB; ++q)
+          tma_load_3d_pair(p + S::A_BYTES + q * bslice + rank * (bslice / 2), &mapB, &full[s], kb * BK,
+                           (int32_t)n0 + (int32_t)rank * (bnw / 2), q);
         issued = kb + 1;
       }
       if (failed)
@@ -615,134 +694,147 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {  // MMA issuer
       const uint32_t idesc = idesc_f16(false, bnw);
       for (int kb = 0; kb < nkb; ++kb) {
-        const int s = kb % STAGES, u = kb / STAGES, b = kb & 1;
-        if (!mbar_wait_bounded(&ready[s], (uint32_t)(u & 1), kWaitSl) ||
-            (kb >= 2 && !mbar_wait_bounded(&accfree[b], (uint32_t)(((kb >> 1) - 1) & 1), kWaitSl))) {
+        const int s = kb % STAGES, u = kb / STAGES, p = kb >> 1, b = p & 1;
+        const bool first = (kb & 1) == 0;
+        if (!mbar_wait_bounded(&ready[kb % RING], (uint32_t)((kb / RING) & 1), kWaitSl) ||
+            !mbar_wait_bounded(&full[s], (uint32_t)(u & 1), kWaitSl) ||
+            (first && p >= 2 && !mbar_wait_bounded(&accfree[b], (uint32_t)(((p >> 1) - 1) & 1), kWaitSl))) {
           failed = true;
           break;
         }
         tc::tc_fence_after();
-        const uint32_t a_hi = smem_u32(base + (size_t)s * S::STAGE_BYTES) + S::RAW_BYTES, a_lo = a_hi + S::A_SLICE;
-        const uint32_t b_hi = a_lo + S::A_SLICE, b_lo = b_hi + bslice;
+        const uint32_t a0 = smem_u32(base + (size_t)s * S::STAGE_BYTES);
+        const uint64_t a_hi = desc_k<128>(a0), a_lo = a_hi + (2 * BK >> 4);
+        const uint64_t b_hi = desc_k<64>(a0 + S::A_BYTES), b_lo = b_hi + (bslice >> 4);
         const uint32_t d = tmem + (uint32_t)(b * S::BNMAX);
         // The small terms first: the truncating additions then happen while
         // the accumulator is small.
 #pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk)
-          mma_f16(d, desc_k<64>(a_hi + 32 * kk), desc_k<64>(b_lo + 32 * kk), idesc, kk > 0 ? 1u : 0u);
+        for (int kk = 0; kk < BK / 16; ++kk) mma_f16(d, a_hi + 2 * kk, b_lo + 2 * kk, idesc, (first && kk == 0) ? 0u : 1u);
 #pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk)
-          mma_f16(d, desc_k<64>(a_lo + 32 * kk), desc_k<64>(b_hi + 32 * kk), idesc, 1u);
+        for (int kk = 0; kk < BK / 16; ++kk) mma_f16(d, a_lo + 2 * kk, b_hi + 2 * kk, idesc, 1u);
 #pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk)
-          mma_f16(d, desc_k<64>(a_hi + 32 * kk), desc_k<64>(b_hi + 32 * kk), idesc, 1u);
-        mma_commit(&empty[s]);
-        mma_commit(&accf[b]);
+        for (int kk = 0; kk < BK / 16; ++kk) mma_f16(d, a_hi + 2 * kk, b_hi + 2 * kk, idesc, 1u);
+        mma_commit_pair(&empty[s]);
+        if (!first || kb == nkb - 1) mma_commit(&accf[b]);
       }
       // Never free TMEM under MMAs that may still run.
       mma_commit(drain);
       if (!mbar_wait_bounded(drain, 0, kWaitSl)) atomicOr(g.err, kErrSl);
     }
-  } else {
-    const int wq = warp & 3;
-    const int ch = (warp - 2) >> 2;  // column half: 128 columns of the tile
-    const uint32_t lane_base = tmem + ((uint32_t)(32 * wq) << 16) + (uint32_t)(128 * ch);
-    const int nc = min(128, max(0, bnw - 128 * ch));  // columns of this warp (uniform)
-    const int t = threadIdx.x - 64;
-    const int sr = t >> 1, sh2 = t & 1;  // split: row, half of its 32 values
-    float run[128];
+  } else if (warp < 2 + S::SPLIT_WARPS) {
+    // Split: one thread per row, in place.  A row's 32 values (128 bytes,
+    // 16-byte chunk q at q ^ (row & 7)) become 32 hi and 32 lo halves, the
+    // same row of a K-major FP16 tile; 8 lanes cover the 8 chunk positions, so
+    // neither loads nor stores meet bank conflicts.  Two K blocks share an
+    // accumulator and therefore the row's scale.
+    const int r = threadIdx.x - 64;
+    auto row_of = [&](int kb) { return base + (size_t)(kb % STAGES) * S::STAGE_BYTES + 128 * r; };
+    auto load = [&](int kb, uint4 (&x)[8], uint32_t mx) {
 #pragma unroll
-    for (int i = 0; i < 128; ++i) run[i] = 0.f;
-    auto fold = [&](int kb) -> bool {
-      const bool ok = mbar_wait_bounded(&accf[kb & 1], (uint32_t)((kb >> 1) & 1), kWaitSl);
-      if (!__all_sync(0xffffffffu, ok)) return false;
-      tc::tc_fence_after();
-      const float rs = rscale[(kb % S::SCALES) * BM + 32 * wq + lane];
+      for (int q = 0; q < 8; ++q) x[q] = *reinterpret_cast<const uint4*>(row_of(kb) + 16 * (q ^ (r & 7)));
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        if (16 * c < nc) {
-          float v[16];
-          tc::tmem_ld16(lane_base + (uint32_t)((kb & 1) * S::BNMAX + 16 * c), v);
-#pragma unroll
-          for (int q = 0; q < 16; ++q) run[16 * c + q] = fmaf(v[q], rs, run[16 * c + q]);
-        }
-      }
-      tc::tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&accfree[kb & 1]);
-      return true;
+      for (int q = 0; q < 8; ++q)
+        mx = max(max(mx, max(x[q].x & 0x7FFFFFFFu, x[q].y & 0x7FFFFFFFu)),
+                 max(x[q].z & 0x7FFFFFFFu, x[q].w & 0x7FFFFFFFu));
+      return mx;
     };
-    for (int kb = 0; kb < nkb && !failed; ++kb) {
-      const int s = kb % STAGES, u = kb / STAGES;
-      const bool ok = mbar_wait_bounded(&full[s], (uint32_t)(u & 1), kWaitSl);
+    auto split = [&](int kb, const uint4 (&x)[8], float sc) {
+      unsigned char* row = row_of(kb);
+      auto two = [&](uint32_t v0, uint32_t v1, uint32_t& hi, uint32_t& lo) {
+        const float a0 = __uint_as_float(v0) * sc, a1 = __uint_as_float(v1) * sc;
+        const __half2 hh = __floats2half2_rn(a0, a1);
+        const float2 f = __half22float2(hh);
+        const __half2 ll = __floats2half2_rn(a0 - f.x, a1 - f.y);
+        hi = *reinterpret_cast<const uint32_t*>(&hh);
+        lo = *reinterpret_cast<const uint32_t*>(&ll);
+      };
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        uint4 hi, lo;
+        two(x[2 * q].x, x[2 * q].y, hi.x, lo.x);
+        two(x[2 * q].z, x[2 * q].w, hi.y, lo.y);
+        two(x[2 * q + 1].x, x[2 * q + 1].y, hi.z, lo.z);
+        two(x[2 * q + 1].z, x[2 * q + 1].w, hi.w, lo.w);
+        *reinterpret_cast<uint4*>(row + 16 * (q ^ (r & 7))) = hi;
+        *reinterpret_cast<uint4*>(row + 16 * ((4 + q) ^ (r & 7))) = lo;
+      }
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&ready[kb % RING]);
+    };
+    for (int kb = 0; kb < nkb; kb += 2) {
+      const bool two = kb + 1 < nkb;
+      const bool ok = mbar_wait_bounded(&full[kb % STAGES], (uint32_t)((kb / STAGES) & 1), kWaitSl) &&
+                      (!two || mbar_wait_bounded(&full[(kb + 1) % STAGES], (uint32_t)(((kb + 1) / STAGES) & 1), kWaitSl));
       if (!__all_sync(0xffffffffu, ok)) {
         failed = true;
         break;
       }
-      unsigned char* st = base + (size_t)s * S::STAGE_BYTES;
-      // Row sr: 128 bytes, 16-byte chunk q at q ^ (row & 7).
-      uint32_t x[16];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint4 v = *reinterpret_cast<const uint4*>(st + 128 * sr + 16 * ((4 * sh2 + q) ^ (sr & 7)));
-        x[4 * q] = v.x;
-        x[4 * q + 1] = v.y;
-        x[4 * q + 2] = v.z;
-        x[4 * q + 3] = v.w;
-      }
-      uint32_t mx = 0;
-#pragma unroll
-      for (int q = 0; q < 16; ++q) mx = max(mx, x[q] & 0x7F800000u);
-      mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+      uint4 x[8];
+      uint32_t mx = two ? load(kb + 1, x, 0u) : 0u;  // its size only, loaded again below
+      mx = load(kb, x, mx);
       // Largest entry into [2^13, 2^14).
       const int sh = min(max(140 - (int)(mx >> 23), -126), 126);
       const float sc = __uint_as_float((uint32_t)(127 + sh) << 23);
-      if (sh2 == 0) rscale[(kb % S::SCALES) * BM + sr] = __uint_as_float((uint32_t)(127 - sh) << 23);
-      uint32_t hi[8], lo[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const float a0 = __uint_as_float(x[2 * q]) * sc, a1 = __uint_as_float(x[2 * q + 1]) * sc;
-        const __half2 h = __floats2half2_rn(a0, a1);
-        const float2 f = __half22float2(h);
-        const __half2 r = __floats2half2_rn(a0 - f.x, a1 - f.y);
-        hi[q] = *reinterpret_cast<const uint32_t*>(&h);
-        lo[q] = *reinterpret_cast<const uint32_t*>(&r);
+      rscale[(kb / 2) % (RING / 2) * BM + r] = __uint_as_float((uint32_t)(127 - sh) << 23);
+      split(kb, x, sc);
+      if (two) {
+        load(kb + 1, x, 0u);
+        split(kb + 1, x, sc);
       }
-      // FP16 row: 64 bytes, chunk q at q ^ ((row >> 1) & 3).
-      unsigned char* hp = st + S::RAW_BYTES + 64 * sr;
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int o = 16 * ((2 * sh2 + q) ^ ((sr >> 1) & 3));
-        *reinterpret_cast<uint4*>(hp + o) = make_uint4(hi[4 * q], hi[4 * q + 1], hi[4 * q + 2], hi[4 * q + 3]);
-        *reinterpret_cast<uint4*>(hp + S::A_SLICE + o) = make_uint4(lo[4 * q], lo[4 * q + 1], lo[4 * q + 2], lo[4 * q + 3]);
-      }
-      fence_proxy_async_smem();
-      mbar_arrive(&ready[s]);
-      if (kb > 0 && !fold(kb - 1)) failed = true;
     }
-    if (!failed && nkb > 0 && !fold(nkb - 1)) failed = true;
-    const int64_t row = m0 + 32 * wq + lane;
-    const int64_t c0 = n0 + 128 * ch;
-    const int64_t left = g.N - c0;
-    const int ncol = (int)(left < nc ? left : nc);
-    if (row < g.M && ncol > 0) {
-      TC* dst = static_cast<TC*>(g.C) + row * g.ldc + c0;
-      float* ct = g.Ct ? g.Ct + c0 * g.ldct + row : nullptr;
+  } else {
+    const int wq = warp & 3, fw = warp - 2 - S::SPLIT_WARPS;
+    const int c = S::NC * (fw >> 2);  // this warp's columns of the tile
+    const int nc = min(S::NC, max(0, bnw - c));
+    const uint32_t lane_base = tmem + ((uint32_t)(32 * wq) << 16) + (uint32_t)c;
+    float run[S::NC];
 #pragma unroll
-      for (int q = 0; q < 128; ++q) {
-        if (q < ncol) {
-          const float v = failed ? __int_as_float(0x7fc00000) : run[q] * __ldg(g.bscale + c0 + q);
-          dst[q] = (TC)v;
-          if (ct) ct[(int64_t)q * g.ldct] = v;
+    for (int i = 0; i < S::NC; ++i) run[i] = 0.f;
+    for (int p = 0; 2 * p < nkb; ++p) {
+      // The ring is long enough for these parities: the split of pair p + 4
+      // needs the MMAs of pair p + 2, which need the fold of pair p.
+      const bool ok = mbar_wait_bounded(&accf[p & 1], (uint32_t)((p >> 1) & 1), kWaitSl) &&
+                      mbar_wait_bounded(&ready[2 * p % RING], (uint32_t)((2 * p / RING) & 1), kWaitSl);
+      if (!__all_sync(0xffffffffu, ok)) {
+        failed = true;
+        break;
+      }
+      tc::tc_fence_after();
+      const float rs = rscale[p % (RING / 2) * BM + 32 * wq + lane];
+#pragma unroll
+      for (int q = 0; q < S::NC / 8; ++q) {
+        if (8 * q < nc) {
+          float v[8];
+          tc::tmem_ld8(lane_base + (uint32_t)((p & 1) * S::BNMAX + 8 * q), v);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) run[8 * q + i] = fmaf(v[i], rs, run[8 * q + i]);
         }
       }
+      tc::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&accfree[p & 1]);
+    }
+    const int64_t c0 = n0 + c, left = g.N - c0;
+    const int ncol = (int)(left < nc ? left : nc);
+    const int64_t row0 = m0 + 32 * wq;
+    // The last accumulator is full: no copy or MMA uses the stages any more
+    // (after a failure they may, so each warp waits for that).
+    if (failed) mbar_wait_bounded(drain, 0, kWaitSl);
+    if (row0 < g.M && ncol > 0) {
+      float* buf = reinterpret_cast<float*>(base + fw * store_buf_bytes<S::NC>());
+      store_warp_tile<TC, S::NC>(run, buf, static_cast<TC*>(g.C), g.ldc, g.Ct, g.ldct, row0, g.M, c0, ncol,
+                                 g.bscale, failed);
     }
   }
   if (failed) atomicOr(g.err, kErrSl);
+  __syncwarp();
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
   if (warp == 0) tc::tmem_dealloc(tmem, S::TMEM_COLS);
+  cluster_sync_all();  // the peer may still copy into this CTA or arrive at its barriers
 }
 
 }  // namespace sl
