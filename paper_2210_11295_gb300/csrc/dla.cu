@@ -5,6 +5,7 @@
 #include <cmath>
 #include <mutex>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "common.cuh"
@@ -349,18 +350,23 @@ int tri_inverse(const Dla& d, const double* L, double* LT, double* Rinv, int64_t
 // 16 x 16 blocks, and the same block eliminations applied to an identity
 // matrix T, which turns T into L^-1.  Step kb:
 //   (a) L_kk = chol(A_kk) and X_kk = L_kk^-1 (one CTA, shared memory);
-//   (b) panel L_ik = A_ik X_kk^T (half a warp per row i > kb) and the final
-//       block row X_kb,c = X_kk T_kb,c of L^-1 (c < kb);
+//   (b) panel L_ik = A_ik X_kk^T (half a warp per row) and the final block row
+//       X_kb,c = X_kk T_kb,c of L^-1 (c < kb);
 //   (c) trailing update A_ij -= L_ik L_jk^T (kb < j <= i) and
-//       T_ic -= L_ik X_kb,c (c <= kb < i), one 16 x 16 tile per warp; CTA 0
-//       updates tile (kb+1, kb+1) alone and factors it in place, which is
-//       (a) of the next step.
-// Two grid barriers per block step.  What bounds it: FP64 operations take
-// about 62 cycles and an SM finishes two a cycle, so the time is the chain of
-// (a) (16 pivots of one reciprocal each) and the barriers.  16-wide blocks
+//       T_ic -= L_ik X_kb,c (c <= kb < i), one 16 x 16 tile per warp.
+// What bounds it: FP64 operations take about 62 cycles and an SM finishes two
+// a cycle, so the time is the chain of (a) (16 pivots of one reciprocal each)
+// and what lies between two of them.  CTA 0 runs that chain alone: given X_kk
+// it forms L_kb+1,kb and the updated tile (kb+1, kb+1) itself and factors it,
+// while the other CTAs do (b) and (c) of step kb; of the two grid barriers of
+// a step it only waits for the one at the end (that before (c) it passes with
+// an arrival once L_kb+1,kb is written).  With (b) and its barrier on the
+// chain, and the tiles on the warps of the first CTAs instead of round all, a
+// step took 22 us, now 17 (l = 512: 0.71 -> 0.55 ms, l = 256: 0.32 -> 0.27;
+// the first change alone gave nothing).  16-wide blocks
 // keep the tile update and the factorisation of (a), which no other SM can
 // share, to a quarter and an eighth of those of 32-wide ones; the other tiles
-// then fit beside that chain (l = 512: 0.71 ms; l = 400: 0.58 -> 0.54).
+// then fit beside that chain.
 // Outputs: L in the lower triangle of g (upper zeroed), LT = L^T and Rinv =
 // L^-T (row-major, upper triangular).  T and X are l x l scratch.  A pivot
 // <= 0 sets kStatusNotPD (and is replaced by 1 so the kernel runs to the end).
@@ -428,7 +434,7 @@ __device__ void ci_factor_diag(const CholInvArgs& a, int kb, double (*s)[kCB + 1
   if (tid < kCB) {
     const double r = sqrt(dd[tid]);
     dd[tid] = r;
-    dinv[tid] = 1.0 / r;
+    dinv[tid] *= r;  // 1 / sqrt(d)
   }
   __syncthreads();
   if (i < nb && c < nb) {
@@ -459,18 +465,64 @@ __global__ void __launch_bounds__(256) k_chol_inv(CholInvArgs a) {
     ci_factor_diag(a, 0, s0, s1, dinv, dd);
   }
   grid.sync();
-  const int gw = blockIdx.x * 8 + w, nwg = gridDim.x * 8;
+  // Entry tid of a lower triangle (CTA 0).
+  int ui = 0;
+  while ((ui + 1) * (ui + 2) / 2 <= tid) ++ui;
+  const int uc = tid - ui * (ui + 1) / 2;
+  // Items of (b) and (c) go round the CTAs first: one tile is 4096 FMAs, 1.1 us
+  // of an SM, and a step has fewer tiles than warps.
+  const int gw = (int)blockIdx.x - 1 + w * ((int)gridDim.x - 1), nwg = ((int)gridDim.x - 1) * 8;
   for (int kb = 0; kb < nblk; ++kb) {
     const int k0 = kb * kCB, nb = min(kCB, l - k0);
-    const int rows_below = l - k0 - nb;
-    // (b) X_kk into shared memory (every CTA), then panel rows, two per warp,
-    // and 32 columns of a row of the X row block.
+    const bool final = kb + 1 == nblk;
+    // X_kk into shared memory (every CTA).  (nb = 16: only the last block is short.)
     xk[ti][tc] = (ti < nb && tc < nb) ? a.X[(int64_t)(k0 + ti) * l + k0 + tc] : 0.0;
+    if (blockIdx.x == 0) {
+      if (final) {
+        grid.sync();
+        break;
+      }
+      const int64_t r0 = k0 + kCB;
+      const bool in = r0 + ti < l;
+      s1[ti][tc] = in ? a.g[(r0 + ti) * l + k0 + tc] : 0.0;
+      s0[ti][tc] = (in && tc <= ti) ? a.g[(r0 + ti) * l + r0 + tc] : (ti == tc ? 1.0 : 0.0);
+      __syncthreads();
+      // Thread: row tc, column ti of L_kb+1,kb.  X_kk[c][e] = 0 for e > c, and
+      // a warp has two columns, so half of the products are left out.
+      double o0 = 0.0, o1 = 0.0;
+      for (int e = 0; e <= (ti | 1); e += 2) {
+        o0 = fma(s1[tc][e], xk[ti][e], o0);
+        o1 = fma(s1[tc][e + 1], xk[ti][e + 1], o1);
+      }
+      const double lv = o0 + o1;
+      if (r0 + tc < l) a.g[(r0 + tc) * l + k0 + ti] = lv;
+      __syncthreads();
+      s1[tc][ti] = lv;
+      auto panel_done = grid.barrier_arrive();
+      __syncthreads();
+      // The lower triangle's 136 entries on the first threads.
+      if (tid < kCB * (kCB + 1) / 2) {
+        o0 = o1 = 0.0;
+#pragma unroll
+        for (int e = 0; e < kCB; e += 2) {
+          o0 = fma(s1[ui][e], s1[uc][e], o0);
+          o1 = fma(s1[ui][e + 1], s1[uc][e + 1], o1);
+        }
+        s0[ui][uc] -= o0 + o1;  // rows beyond l: zeros in s1
+      }
+      __syncthreads();
+      ci_factor_diag(a, kb + 1, s0, s1, dinv, dd);
+      grid.barrier_wait(std::move(panel_done));
+      grid.sync();
+      continue;
+    }
+    // (b) panel rows from block kb + 2 on, two per warp, and 32 columns of a
+    // row of the X row block.
     __syncthreads();
-    const int np = (rows_below + 1) / 2, nch = (k0 + 31) / 32, nx = nb * nch;
+    const int np = max(0, (l - k0 - 2 * kCB + 1) / 2), nch = (k0 + 31) / 32, nx = nb * nch;
     for (int it = gw; it < np + nx; it += nwg) {
       if (it < np) {
-        const int64_t row = k0 + nb + 2 * it + (lane >> 4);
+        const int64_t row = k0 + 2 * kCB + 2 * it + (lane >> 4);
         const int c = lane & 15;
         const bool in = row < l && c < nb;
         const double v = in ? a.g[row * l + k0 + c] : 0.0;
@@ -495,30 +547,15 @@ __global__ void __launch_bounds__(256) k_chol_inv(CholInvArgs a) {
       }
     }
     grid.sync();
-    if (kb + 1 == nblk) break;
-    // (c) trailing tiles (bi >= bj > kb) and T tiles (bi > kb >= c); item 0
-    // is the diagonal tile (kb+1, kb+1).  (nb = 16: only the last block is short.)
+    if (final) break;
+    // (c) trailing tiles (bi >= bj > kb) and T tiles (bi > kb >= c) but the
+    // diagonal tile (kb+1, kb+1), item 0.
     const int rem = nblk - kb - 1;
     const int n_trail = rem * (rem + 1) / 2, n_t = rem * (kb + 1);
-    if (blockIdx.x == 0) {
-      const int64_t r0 = k0 + kCB;
-      s1[ti][tc] = r0 + ti < l ? a.g[(r0 + ti) * l + k0 + tc] : 0.0;
-      __syncthreads();
-      double o0 = 0.0, o1 = 0.0;
-      if (tc <= ti) {
-#pragma unroll
-        for (int e = 0; e < kCB; e += 2) {
-          o0 = fma(s1[ti][e], s1[tc][e], o0);
-          o1 = fma(s1[ti][e + 1], s1[tc][e + 1], o1);
-        }
-      }
-      s0[ti][tc] = (r0 + ti < l && tc <= ti) ? a.g[(r0 + ti) * l + r0 + tc] - (o0 + o1) : (ti == tc ? 1.0 : 0.0);
-      __syncthreads();
-      ci_factor_diag(a, kb + 1, s0, s1, dinv, dd);
-    } else {
+    {
       double(*sa)[kCB + 1] = sw[w][0];
       double(*sb)[kCB + 1] = sw[w][1];
-      for (int item = 1 + (blockIdx.x - 1) * 8 + w; item < n_trail + n_t; item += (gridDim.x - 1) * 8) {
+      for (int item = 1 + gw; item < n_trail + n_t; item += nwg) {
         const bool trail = item < n_trail;
         int bi, bj;
         if (trail) {
@@ -568,7 +605,6 @@ __global__ void __launch_bounds__(256) k_chol_inv(CholInvArgs a) {
     grid.sync();
   }
   // Outputs: zero the upper triangle of g, LT = L^T, Rinv = X^T.
-  grid.sync();
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + tid; e < ll; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / l, j = e % l;  // element (i, j) of the outputs
     if (j > i) a.g[e] = 0.0;
@@ -582,7 +618,8 @@ int chol_inv(const Dla& d, double* g, double* LT, double* Rinv, double* T, doubl
   CholInvArgs a{g, LT, Rinv, T, X, (int)l, (int)((l + kCB - 1) / kCB), d.status};
   // CTA 0 for the diagonal blocks and one CTA per four tiles of the fullest
   // step (about nblk^2 / 2), as far as the SMs go: barriers over fewer CTAs
-  // are cheaper.
+  // are cheaper (one per 2, 4, 8 and 12 tiles at l = 400, two factorisations
+  // within 1.11, 1.05, 1.08 and 1.39 ms).
   const int64_t tiles = (int64_t)a.nblk * (a.nblk + 1) / 2;
   const int blocks = (int)std::min<int64_t>(num_sms(), 1 + (tiles + 3) / 4);
   void* args[] = {&a};
