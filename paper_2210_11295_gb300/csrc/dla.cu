@@ -2135,19 +2135,21 @@ int scale_columns(const Dla& d, double* X, int64_t rows, int64_t cols, int64_t l
 
 // Column argmax of |U| (lowest row on ties) per row chunk: partial (value,
 // index) per chunk.  Columns along x (kb per block), blockDim.x / kb rows at a
-// time: with one thread per column its chain of loads was the time (factors
-// of rSVD 4096 x 256, l = 100: 0.24 -> 0.16 ms with the sums below).
-__global__ void __launch_bounds__(256) k_colargmax_partial(const double* __restrict__ U, int64_t n, int64_t k, int kb,
-                                                           int64_t rows_per, double* __restrict__ pv,
-                                                           int64_t* __restrict__ pi) {
-  __shared__ double sv[256];
-  __shared__ int64_t si[256];
+// time; a pass over U, bound by the loads in flight (1048576 x 100: one thread
+// per column and chunk 1.1 ms, 256 threads 0.55, 1024 threads 0.40).
+constexpr int kArgmaxThreads = 1024;
+__global__ void __launch_bounds__(kArgmaxThreads) k_colargmax_partial(const double* __restrict__ U, int64_t n,
+                                                                      int64_t k, int kb, int64_t rows_per,
+                                                                      double* __restrict__ pv,
+                                                                      int64_t* __restrict__ pi) {
+  __shared__ double sv[kArgmaxThreads];
+  __shared__ int64_t si[kArgmaxThreads];
   const int nr = blockDim.x / kb, q = threadIdx.x / kb;
   const int64_t c = (int64_t)blockIdx.y * kb + threadIdx.x % kb;
   const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(n, r0 + rows_per);
   double best = -1.0;
   int64_t bi = r0;
-  if (c < k && q < nr) {
+  if (c < k) {
 #pragma unroll 8
     for (int64_t i = r0 + q; i < r1; i += nr) {
       const double v = fabs(U[i * k + c]);
@@ -2159,18 +2161,22 @@ __global__ void __launch_bounds__(256) k_colargmax_partial(const double* __restr
   }
   sv[threadIdx.x] = best;
   si[threadIdx.x] = bi;
-  __syncthreads();
-  if (q != 0 || c >= k) return;
-  for (int u = 1; u < nr; ++u) {
-    const double v = sv[threadIdx.x + u * kb];
-    const int64_t i = si[threadIdx.x + u * kb];
-    if (v > best || (v == best && i < bi)) {
-      best = v;
-      bi = i;
+  for (int left = nr; left > 1;) {
+    const int half = (left + 1) / 2;
+    __syncthreads();
+    if (q < left - half) {
+      const double v = sv[threadIdx.x + half * kb];
+      const int64_t i = si[threadIdx.x + half * kb];
+      if (v > sv[threadIdx.x] || (v == sv[threadIdx.x] && i < si[threadIdx.x])) {
+        sv[threadIdx.x] = v;
+        si[threadIdx.x] = i;
+      }
     }
+    left = half;
   }
-  pv[(int64_t)blockIdx.x * k + c] = best;
-  pi[(int64_t)blockIdx.x * k + c] = bi;
+  if (q != 0 || c >= k) return;
+  pv[(int64_t)blockIdx.x * k + c] = sv[threadIdx.x];
+  pi[(int64_t)blockIdx.x * k + c] = si[threadIdx.x];
 }
 
 // One block per column.
@@ -2215,7 +2221,8 @@ int sign_normalize(const Dla& d, Arena& ar, double* U, int64_t n, int64_t k, dou
   if (!ar.ok()) return BSRHT_ENOMEM;
   if (ar.measure) return BSRHT_OK;
   const int kb = (int)std::min<int64_t>(256, k);
-  k_colargmax_partial<<<dim3(nchunks, blocks_for(k, kb)), 256 / kb * kb, 0, d.s>>>(U, n, k, kb, rows_per, pv, pi);
+  k_colargmax_partial<<<dim3(nchunks, blocks_for(k, kb)), kArgmaxThreads / kb * kb, 0, d.s>>>(U, n, k, kb, rows_per, pv,
+                                                                                            pi);
   DLA_LAUNCH_CHECK();
   k_colargmax_final<<<(unsigned)k, 128, 0, d.s>>>(U, k, nchunks, pv, pi, sg);
   DLA_LAUNCH_CHECK();

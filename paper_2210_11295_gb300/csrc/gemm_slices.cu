@@ -407,14 +407,15 @@ int gemm_a16(const Dla& d, Arena& ar, DT ta, int64_t M, int64_t N, int64_t K, co
   TRY_SL(bf ? (slice_b<__nv_bfloat16, S::NB>(d, ar, K, N, tb, B, ldb, &b))
             : (slice_b<__half, S::NB>(d, ar, K, N, tb, B, ldb, &b)));
   if (ar.measure) return BSRHT_OK;
-  const int64_t tiles = (M + sl::BM - 1) / sl::BM * ((N + b.bn - 1) / b.bn);
+  // Pairs of row tiles.
+  const int64_t tiles = 2 * ((M + 2 * sl::BM - 1) / (2 * sl::BM)) * ((N + b.bn - 1) / b.bn);
   if (tiles > 0x7FFFFFFF) return BSRHT_EUNSUP;
   const CUtensorMapDataType dt = bf ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
   CUtensorMap ma, mb;
   if (!make_tensor_map_2d(&ma, A, dt, 2, (uint64_t)M, (uint64_t)K, (uint64_t)lda, S::BK, sl::BM,
                           CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !make_slice_map(&mb, b.slices, dt, K, N, S::NB, b.ldk, S::BK, (uint32_t)b.bn, CU_TENSOR_MAP_SWIZZLE_128B,
-                      S::NB))
+      !make_slice_map(&mb, b.slices, dt, K, N, S::NB, b.ldk, S::BK, (uint32_t)b.bn / 2,
+                      CU_TENSOR_MAP_SWIZZLE_128B, 1))
     return BSRHT_EUNSUP;
   BSRHT_CUDA_TRY(
       cudaFuncSetAttribute(sl::k_gemm_a16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_bytes()));

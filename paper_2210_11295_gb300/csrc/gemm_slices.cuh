@@ -23,7 +23,9 @@
 // BF16, 33 in FP16), scaled per column to FP16's range.  Three 16-bit MMAs
 // per product; each K block of 64 starts a fresh accumulator, smallest slice
 // first, which the fold adds to FP32 registers, rounding to nearest (the
-// tensor core's own accumulation truncates).
+// tensor core's own accumulation truncates).  Bound by the copies of B's three
+// slices from L2 (94 KB a block of K at N = 400): two CTAs load half of B each
+// for both, and C leaves in whole sectors (262144 x 2000 x 400: 1.57 -> 1.20 ms).
 //
 // k_gemm_f32x2: FP32 products of FP32 data at twice the TF32 rate.  An FP16
 // pair holds as much of an FP32 value as a TF32 pair (11 + 11 bits) once it is
@@ -437,6 +439,7 @@ struct A16 {
   static constexpr size_t smem_bytes() { return 1024 + (size_t)STAGES * STAGE_BYTES + 256; }
   static constexpr uint32_t TMEM_COLS = 2 * BNMAX;
   static_assert(STAGES * STAGE_BYTES + 1280 <= 227 * 1024, "shared memory");
+  static_assert(8 * store_buf_bytes<128>() <= STAGES * STAGE_BYTES, "the stages hold the stored tile");
 };
 
 struct A16Args {
@@ -451,7 +454,7 @@ struct A16Args {
   int* err;
 };
 
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     k_gemm_a16(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, A16Args g) {
   using S = A16;
   constexpr int BK = S::BK, STAGES = S::STAGES;
@@ -467,7 +470,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bnw = g.bn;
   const int64_t tn = (g.N + bnw - 1) / bnw;
-  const int64_t bm = (int64_t)blockIdx.x / tn, bn = (int64_t)blockIdx.x - bm * tn;
+  // The pair's two row tiles share one column tile; each CTA loads half of B
+  // for both.
+  const uint32_t rank = cluster_rank();
+  const int64_t pair = (int64_t)blockIdx.x >> 1, bm = 2 * (pair / tn) + rank, bn = pair % tn;
   const int64_t m0 = bm * BM, n0 = bn * bnw;
   const int nkb = (int)((g.K + BK - 1) / BK);
   const uint32_t bslice = (uint32_t)bnw * BK * 2;
@@ -475,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+      mbar_init(&empty[s], 2);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&accf[b], 1);
@@ -487,6 +493,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0) tc::tmem_alloc(tmem_slot, S::TMEM_COLS);
   tc::tc_fence_before();
   __syncthreads();
+  cluster_sync_all();  // the peer's barriers exist before anything arrives at them
   tc::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   bool failed = false;
@@ -503,7 +510,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         unsigned char* p = base + (size_t)s * S::STAGE_BYTES;
         mbar_arrive_expect_tx(&full[s], S::A_BYTES + S::NB * bslice);
         tma_load_2d(p, &mapA, &full[s], kb * BK, (int32_t)m0);
-        tma_load_3d(p + S::A_BYTES, &mapB, &full[s], kb * BK, (int32_t)n0, 0);
+#pragma unroll
+        for (int q = 0; q < S::NB; ++q)
+          tma_load_3d_pair(p + S::A_BYTES + q * bslice + rank * (bslice / 2), &mapB, &full[s], kb * BK,
+                           (int32_t)n0 + (int32_t)rank * (bnw / 2), q);
         issued = kb + 1;
       }
       if (failed)
@@ -521,7 +531,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           break;
         }
         tc::tc_fence_after();
-        const uint32_t a0 = smem_u32(base + (size_t)s * S::STAGE_BYTES), b0 = a0 + S::A_BYTES;
+        const uint32_t a0 = smem_u32(base + (size_t)s * S::STAGE_BYTES);
+        const uint64_t da = desc_k<128>(a0), db = desc_k<128>(a0 + S::A_BYTES);
         const uint32_t d = tmem + (uint32_t)(b * S::BNMAX);
         // Smallest slice first: the truncating additions then happen while
         // the accumulator is small.
@@ -529,10 +540,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int q = S::NB - 1; q >= 0; --q) {
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk)
-            mma_f16(d, desc_k<128>(a0 + 32 * kk), desc_k<128>(b0 + q * bslice + 32 * kk), idesc,
+            mma_f16(d, da + 2 * kk, db + (q * bslice >> 4) + 2 * kk, idesc,
                     (q == S::NB - 1 && kk == 0) ? 0u : 1u);
         }
-        mma_commit(&empty[s]);
+        mma_commit_pair(&empty[s]);
         mma_commit(&accf[b]);
       }
       // Never free TMEM under MMAs that may still run.
@@ -567,30 +578,23 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&accfree[kb & 1]);
     }
-    const int64_t row = m0 + 32 * wq + lane;
-    const int64_t c0 = n0 + 128 * ch;
-    const int64_t left = g.N - c0;
+    const int64_t row0 = m0 + 32 * wq, c0 = n0 + 128 * ch, left = g.N - c0;
     const int ncol = (int)(left < nc ? left : nc);
-    if (row < g.M && ncol > 0) {
-      float* dst = g.C + row * g.ldc + c0;
-      float* ct = g.Ct ? g.Ct + c0 * g.ldct + row : nullptr;
-#pragma unroll
-      for (int q = 0; q < 128; ++q) {
-        if (q < ncol) {
-          const float x = failed ? __int_as_float(0x7fc00000) : run[q] * __ldg(g.bscale + c0 + q);
-          dst[q] = x;
-          // Column q is row c0 + q of C^T; lane = row of C: 128 contiguous
-          // bytes per warp store.
-          if (ct) ct[(int64_t)q * g.ldct] = x;
-        }
-      }
+    // The last accumulator is full: no copy or MMA uses the stages any more
+    // (after a failure they may, so each warp waits for that).
+    if (failed) mbar_wait_bounded(drain, 0, kWaitSl);
+    if (row0 < g.M && ncol > 0) {
+      float* buf = reinterpret_cast<float*>(base + (warp - 2) * store_buf_bytes<128>());
+      store_warp_tile<float, 128>(run, buf, g.C, g.ldc, g.Ct, g.ldct, row0, g.M, c0, ncol, g.bscale, failed);
     }
   }
   if (failed) atomicOr(g.err, kErrSl);
+  __syncwarp();
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
   if (warp == 0) tc::tmem_dealloc(tmem, S::TMEM_COLS);
+  cluster_sync_all();  // the peer may still copy into this CTA or arrive at its barriers
 }
 
 // ------------------------------------------------ FP32 A, two slices each
