@@ -2136,7 +2136,7 @@ int scale_columns(const Dla& d, double* X, int64_t rows, int64_t cols, int64_t l
 // Column argmax of |U| (lowest row on ties) per row chunk: partial (value,
 // index) per chunk.  Columns along x (kb per block), blockDim.x / kb rows at a
 // time; a pass over U, bound by the loads in flight (1048576 x 100: one thread
-// per column and chunk 1.1 ms, 256 threads 0.55, 1024 threads 0.40).
+// per column and chunk 1.1 ms, 256 threads 0.55, 1024 threads 0.42).
 constexpr int kArgmaxThreads = 1024;
 __global__ void __launch_bounds__(kArgmaxThreads) k_colargmax_partial(const double* __restrict__ U, int64_t n,
                                                                       int64_t k, int kb, int64_t rows_per,
