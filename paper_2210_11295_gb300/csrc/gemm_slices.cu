@@ -213,13 +213,13 @@ size_t digit_bytes_of(int64_t rows, int64_t ldk) { return (size_t)kDig * 2 * (si
 
 }  // namespace
 
-// Scratch the digits of one launch may take: enough rows of A for two waves
-// of 128 x 64 tiles over the SMs at K = 2048, l = 256.
+// Scratch the digits of one launch may take: enough rows of A for a wave of
+// 128 x 64 tiles over the SMs at K = 2048, l = 256 (139 MB).
 constexpr size_t kDigitScratch = (size_t)192 << 20;
 
 // Measured on GB300 (int8x7 against the CUDA-core GEMM, FP64): below about 20
 // million FMAs the preparation's launches cost more than they save (256^3
-// 0.054 / 0.045 ms, 300^3 0.055 / 0.084, 400^3 0.058 / 0.196).
+// 0.048 / 0.049 ms, 300^3 0.049 / 0.085, 400^3 0.052 / 0.195).
 bool gemm_int8x7_wants(int64_t M, int64_t N, int64_t K) {
   return M >= 32 && N >= 16 && K >= 32 && (double)M * (double)N * (double)K >= 2e7;
 }
