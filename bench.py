@@ -286,17 +286,17 @@ TRAFFIC_RECORDS = {
     # FP32: the reads are A itself; the writes are the per-(CTA, panel)
     # partial sums, written once (they do not grow with n).
     ("f32", 1 << 20, 4096, 4, 512): {
-        "kernel": "k_sketch_tma", "read_n2e18": 4295577600, "write_n2e18": 10937344, "write_scales": False,
+        "kernel": "k_sketch_tma", "read_n2e18": 4295609088, "write_n2e18": 10859776, "write_scales": False,
         "sources": ("paper_2210_11295_gb300/csrc/sketch_tma.cu", "paper_2210_11295_gb300/csrc/tma.cuh",
                     "paper_2210_11295_gb300/csrc/f32x2.cuh", "paper_2210_11295_gb300/csrc/tmem.cuh"),
-        "sha256": "ca6860d416ec01d8c929f0487f7bd6c01e8f56c165772ffdb2198846db92a4b4"},
+        "sha256": "636f3905aee97161edcfe253e80ccb875fc396b4b57bdb457c7a9bd76e89b8fb"},
     # FP64: besides A, the read-modify-write of the FP64 partial sums at
     # every flush of the integer sums (one per 32 chunks of a CTA), which
     # grows with n like the reads.
     ("f64", 1 << 20, 4096, 4, 512): {
-        "kernel": "k_sketch_f64x", "read_n2e18": 8838070016, "write_n2e18": 266583552, "write_scales": True,
+        "kernel": "k_sketch_f64x", "read_n2e18": 8838101504, "write_n2e18": 266206208, "write_scales": True,
         "sources": ("paper_2210_11295_gb300/csrc/sketch_f64x.cu", "paper_2210_11295_gb300/csrc/tma.cuh"),
-        "sha256": "13dd167a62728e7de4f5dafe612557852b4d179c5eab3a41148373abf2378615"},
+        "sha256": "bda48dc8aefdc298ae20d25dd2a2d94166275d4ad17a08f6834135e6992e0cc4"},
 }
 
 
