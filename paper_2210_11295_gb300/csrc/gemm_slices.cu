@@ -426,14 +426,18 @@ int gemm_a16(const Dla& d, Arena& ar, DT ta, int64_t M, int64_t N, int64_t K, co
   return BSRHT_OK;
 }
 
-// Tiles enough for most SMs (the other kernel splits K instead), wide enough
-// to gain on the split of A, K short enough for a chain of at most 256 folds,
-// and long against the start and the stores of a tile, which nothing overlaps:
-// 65536 x 2000 x 400 0.45 ms against 0.70 in TF32, but 2^20 x 512 x 512 (upper
-// triangular) 2.8 ms in both and 2^20 x 512 x 100 1.4 against 1.2.
+// Tiles enough for most SMs (the other kernel splits K instead) and not a wave
+// with little more than it (12290 x 1024 x 257, 1.3 waves: 0.091 ms against 0.079
+// in TF32; 16384 x 1024 x 512, 1.7 waves: 0.104 against 0.110), K short enough for
+// a chain of at most 256 folds, and K and the tile long and wide against a
+// tile's start and stores, which nothing overlaps: 65536 x 2000 x 400 0.45 ms
+// against 0.70 in TF32, 262144 x 1024 x 256 0.60 against 0.69, but 2^20 x 512 x 512
+// (upper triangular) 2.8 ms in both and 262144 x 1024 x 128, one 128-wide tile,
+// 0.53 against 0.41.
 bool gemm_f32x2_eligible(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda) {
-  return M >= 128 * 96 && N >= 128 && K >= 1024 && K <= 256 * 64 && (lda % 4) == 0 &&
-         (reinterpret_cast<uintptr_t>(A) % 16) == 0;
+  const int64_t tiles = (M + sl::BM - 1) / sl::BM * ((N + 255) / 256), sms = num_sms();
+  return M >= 128 * 96 && N > 128 && (tiles <= sms || 2 * tiles >= 3 * sms) && K >= 1024 && K <= 256 * 64 &&
+         (lda % 4) == 0 && (reinterpret_cast<uintptr_t>(A) % 16) == 0;
 }
 
 int gemm_f32x2(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, DT tb,

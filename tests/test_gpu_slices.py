@@ -94,8 +94,10 @@ def test_rsvd_16bit_matches_oracle(lib, dtype, n, m, ld, l):
 
 @pytest.mark.parametrize("n,m,ld,l", [
     (12300, 1028, 1028, 130),  # ragged rows, two column tiles, ragged last K block
-    (12288, 1024, 1024, 128),  # exact tiles, at the edge of the rule
-    (12290, 2000, 2048, 257),  # column slice, one column past two tiles
+    (12288, 1024, 1024, 128),  # one narrow tile: the TF32 product
+    (12290, 2000, 2048, 257),  # column slice, little more than a wave: the TF32 product
+    (16384, 1024, 1024, 256),  # exact tiles
+    (16500, 1100, 1104, 257),  # column slice, one column past a tile, odd number of row tiles
     (12290, 1026, 1026, 130),  # rows off 16 bytes: the TF32 product
 ])
 def test_rsvd_f32_matches_oracle(lib, n, m, ld, l):
