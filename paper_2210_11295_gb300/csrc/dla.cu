@@ -1051,8 +1051,6 @@ __global__ void k_gather_directions(const float* __restrict__ X, const double* _
   V[idx] = n > 0.0 ? (double)X[c * l + i] / n : 0.0;
 }
 
-__global__ void k_scale_cols(double* X, int64_t rows, int64_t cols, int64_t ld, const double* sc, int inv);
-
 // Flags of the FP64 refinement.
 constexpr int kRefPair = 1;     // some pair's cosine exceeds the stopping threshold
 constexpr int kRefCluster = 2;  // such a pair is too close for the first-order rotation
@@ -1060,6 +1058,17 @@ constexpr int kRefCoarse = 4;   // such a pair turns by more than kRefFine
 constexpr int kRefOrth = 8;     // V was not yet orthogonal to rounding
 // Below this angle I + X + X^2 / 2 is a rotation to rounding (error X^4 / 4).
 constexpr double kRefFine = 0x1.0p-26;
+// Largest angle of a step that does not make V orthonormal again: at l = 768,
+// every angle at this limit with random signs, X has a norm of 2^-11.2 and V's
+// defect is 2^-47.  (kRefFine for it leaves the columns beyond the wanted ones
+// as they are, and their cosines cost another step: 0.2 ms of the 8.55 of a
+// Nystrom request of l = 400.)
+constexpr double kRefKeepsV = 0x1.0p-17;
+// Largest angle before the sweeps: among close values larger ones are mostly
+// rounding, and undone by the sweeps (CPU model of these steps, half of 256
+// values equal: 2 sweeps after it, 10 after angles up to 0.03; pairs 1e-4 to
+// 1e-15 apart: 3 sweeps either way, 5 without this rotation).
+constexpr double kRefBeforeSweeps = 0x1.0p-10;
 
 // Coefficients of one orthonormalisation step V <- V G of nearly orthonormal
 // columns from their Gram G, in place.  tri: Gram-Schmidt to first order
@@ -1104,7 +1113,11 @@ __global__ void k_scale_norms(const double* __restrict__ C, int64_t n, double* _
 // Z = D X D^-1 (D = diag(s)), c the cosine of the pair and s_i = sig_i |u_i|.
 // Z (for U's columns once normalised) stays as small as the cosines (over the relative gaps) however far apart
 // the norms are, so small columns are made orthogonal to their own accuracy.
-// Pairs with |X_ij| > 0.03 (clustered singular values) are left alone.
+// Pairs with |X_ij| > 0.03 (clustered singular values) are left alone, and so
+// are pairs orthogonal to the threshold that would turn by more than
+// kRefKeepsV: over a small enough gap the rounding of a cosine turns by any
+// angle.  (Leaving alone all of them lets some drift past the threshold:
+// another step, 0.2 ms as above.)
 // Flags: see above; a pair exceeds by the test of a Jacobi sweep (k_jacobi).
 // Only pairs with one of the first `lead` columns (the caller's triplets, of
 // columns by descending norm) set flags: the others need not be orthogonal
@@ -1123,7 +1136,7 @@ __global__ void k_refine_generator(const double* __restrict__ C, const double* _
     const double ni = C[i * n + i], nj = C[j * n + j];
     const double si = sig[i] * sqrt(ni), sj = sig[j] * sqrt(nj);
     if (!(si <= tiny && sj <= tiny) && g != 0.0) {
-      const bool exceeds = (i < lead || j < lead) && !(g * g <= tol * tol * ni * nj);
+      const bool exceeds = !(g * g <= tol * tol * ni * nj);
       // Ratio of the smaller norm to the larger one: no overflow, no
       // difference of squares.
       const bool up = sj >= si;
@@ -1135,7 +1148,8 @@ __global__ void k_refine_generator(const double* __restrict__ C, const double* _
         x = (up ? c : -c) * q / den;
         z = up ? c * (q * q) / den : -c / den;        // s_i^2 over s_j^2 - s_i^2
       }
-      if (exceeds) {
+      if (!exceeds && fabs(x) > kRefKeepsV) x = z = 0.0;
+      if (exceeds && (i < lead || j < lead)) {
         int f = kRefPair;
         if (!ok) f |= kRefCluster;
         if (fabs(x) > kRefFine) f |= kRefCoarse;
@@ -1145,6 +1159,12 @@ __global__ void k_refine_generator(const double* __restrict__ C, const double* _
   }
   X[idx] = x;
   Z[idx] = z;
+}
+
+// Leaves out the rotations by more than `most`.
+__global__ void k_refine_cap(double* __restrict__ X, double* __restrict__ Z, int64_t n, double most) {
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx < n * n && !(fabs(X[idx]) <= most)) X[idx] = Z[idx] = 0.0;
 }
 
 // T = I + X + P / 2 (P = X X, in place in P).
@@ -1738,9 +1758,12 @@ int jacobi_svd(const Dla& d, Arena& ar, double* colsM, int64_t l, double* U, dou
   //     large, V is then made orthonormal again and Y = M V formed anew; a
   //     new Y carries rounding of ||M||, so the last steps, whose angles are
   //     too small to disturb V, update U itself and leave each column
-  //     orthogonal to its own accuracy.  Pairs too close for first order
-  //     (clustered singular values) are left to FP64 Jacobi sweeps, which
-  //     the result passes through only then.
+  //     orthogonal to its own accuracy.  (Larger angles among the columns
+  //     that do not count for the stop are left out of these steps.)  Pairs
+  //     too close for first order (clustered singular values) are left to
+  //     FP64 Jacobi sweeps, which the result passes through only then: from
+  //     V made orthonormal to rounding, since the sweeps keep whatever
+  //     defect V has.
   // *done stays false (and colsM as it was) when the FP32 phase's directions
   // are not near orthonormal (M numerically singular in FP32): the caller
   // goes on with accumulated rotations.
@@ -1801,11 +1824,12 @@ int jacobi_svd(const Dla& d, Arena& ar, double* colsM, int64_t l, double* U, dou
     BSRHT_CUDA_TRY(cudaMemsetAsync(cflag, 0, sizeof(int), d.s));
     TRY_DLA(orth_step(true, 1e-3, kRefCluster));
     TRY_DLA(read_flags());
-    if (flags) {  // not near orthonormal
+    auto give_up = [&]() -> int {
       s = part && ktop > 0 ? s : l;
       BSRHT_CUDA_TRY(cudaMemsetAsync(rot, 0, sizeof(int) * 2 * max_sweeps, d.s));
       return BSRHT_OK;
-    }
+    };
+    if (flags) return give_up();  // not near orthonormal
     constexpr double kLoose = 1e-10;  // one Newton-Schulz step then reaches rounding
     TRY_DLA(orth_step(false, kLoose, kRefOrth));
     TRY_DLA(form_y());
@@ -1833,6 +1857,12 @@ int jacobi_svd(const Dla& d, Arena& ar, double* colsM, int64_t l, double* U, dou
       std::swap(W, Wn);
       return BSRHT_OK;
     };
+    auto cap = [&](double most) -> int {
+      k_refine_cap<<<sb, 256, 0, d.s>>>(Xg, Zg, s, most);
+      DLA_LAUNCH_CHECK();
+      note_launches(1);
+      return BSRHT_OK;
+    };
     TRY_DLA(normalize_y());
     bool converged = false;
     for (int it = 0; it < 8; ++it) {
@@ -1850,25 +1880,36 @@ int jacobi_svd(const Dla& d, Arena& ar, double* colsM, int64_t l, double* U, dou
       }
       if (converged) break;
       BSRHT_CUDA_TRY(cudaMemsetAsync(cflag, 0, sizeof(int), d.s));
+      if (flags & kRefCluster) {
+        TRY_DLA(cap(kRefBeforeSweeps));
+        TRY_DLA(rotate(Xg, V, Vn));
+        break;
+      }
       if (flags & (kRefCoarse | kRefOrth)) {
         if (flags & kRefPair) TRY_DLA(rotate(Xg, V, Vn));
         TRY_DLA(orth_step(false, kLoose, kRefOrth));
         TRY_DLA(form_y());
         TRY_DLA(normalize_y());
       } else {
+        TRY_DLA(cap(kRefKeepsV));
         TRY_DLA(rotate(Xg, V, Vn));
         TRY_DLA(rotate(Zg, U1, U2));
       }
-      if ((flags & kRefCluster) && !(flags & kRefOrth)) break;
     }
     const double *Yf = U1, *Vf = V;
     int64_t si = s, sc = 1;
     if (!converged) {
-      // FP64 Jacobi sweeps on the columns of U diag(sig) (the caller's M is
-      // spent).
-      k_scale_cols<<<lb, 256, 0, d.s>>>(U1, l, s, s, sigS, 0);
-      DLA_LAUNCH_CHECK();
-      TRY_DLA(transpose_cast(d, DT::F64, U1, l, s, s, DT::F64, colsM, l));
+      // V orthonormal to rounding (each step squares its defect), then FP64
+      // Jacobi sweeps on the columns of Y = M V (the caller's M is spent).
+      int left = 8;
+      do {
+        if (left-- == 0) return give_up();
+        BSRHT_CUDA_TRY(cudaMemsetAsync(cflag, 0, sizeof(int), d.s));
+        TRY_DLA(orth_step(false, kLoose, kRefOrth));
+        TRY_DLA(read_flags());
+      } while (flags);
+      TRY_DLA(form_y());
+      TRY_DLA(transpose_cast(d, DT::F64, Y, l, s, s, DT::F64, colsM, l));
       TRY_DLA(transpose_cast(d, DT::F64, V, l, s, s, DT::F64, G, l));
       TRY_DLA(polish(colsM, G, s, l));
       k_col_norms_t<double><<<blocks_for(s, 8), 256, 0, d.s>>>(colsM, sigS, s, l);
