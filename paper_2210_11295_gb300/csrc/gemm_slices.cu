@@ -407,15 +407,14 @@ int gemm_a16(const Dla& d, Arena& ar, DT ta, int64_t M, int64_t N, int64_t K, co
   TRY_SL(bf ? (slice_b<__nv_bfloat16, S::NB>(d, ar, K, N, tb, B, ldb, &b))
             : (slice_b<__half, S::NB>(d, ar, K, N, tb, B, ldb, &b)));
   if (ar.measure) return BSRHT_OK;
-  // Pairs of row tiles.
-  const int64_t tiles = 2 * ((M + 2 * sl::BM - 1) / (2 * sl::BM)) * ((N + b.bn - 1) / b.bn);
+  const int64_t tiles = (M + sl::BM - 1) / sl::BM * ((N + b.bn - 1) / b.bn);
   if (tiles > 0x7FFFFFFF) return BSRHT_EUNSUP;
   const CUtensorMapDataType dt = bf ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
   CUtensorMap ma, mb;
   if (!make_tensor_map_2d(&ma, A, dt, 2, (uint64_t)M, (uint64_t)K, (uint64_t)lda, S::BK, sl::BM,
                           CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !make_slice_map(&mb, b.slices, dt, K, N, S::NB, b.ldk, S::BK, (uint32_t)b.bn / 2,
-                      CU_TENSOR_MAP_SWIZZLE_128B, 1))
+      !make_slice_map(&mb, b.slices, dt, K, N, S::NB, b.ldk, S::BK, (uint32_t)b.bn, CU_TENSOR_MAP_SWIZZLE_128B,
+                      1))
     return BSRHT_EUNSUP;
   BSRHT_CUDA_TRY(
       cudaFuncSetAttribute(sl::k_gemm_a16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_bytes()));
@@ -427,13 +426,13 @@ int gemm_a16(const Dla& d, Arena& ar, DT ta, int64_t M, int64_t N, int64_t K, co
 }
 
 // Tiles enough for most SMs (the other kernel splits K instead) and not a wave
-// with little more than it (12290 x 1024 x 257, 1.3 waves: 0.091 ms against 0.079
-// in TF32; 16384 x 1024 x 512, 1.7 waves: 0.104 against 0.110), K short enough for
+// with little more than it (12290 x 1536 x 257, 1.3 waves: 0.111 ms against 0.102
+// in TF32; 16000 x 1536 x 512, 1.6 waves: 0.126 against 0.151), K short enough for
 // a chain of at most 256 folds, and K and the tile long and wide against a
-// tile's start and stores, which nothing overlaps: 65536 x 2000 x 400 0.45 ms
-// against 0.70 in TF32, 262144 x 1024 x 256 0.60 against 0.69, but 2^20 x 512 x 512
-// (upper triangular) 2.8 ms in both and 262144 x 1024 x 128, one 128-wide tile,
-// 0.53 against 0.41.
+// tile's start and stores, which nothing overlaps: 65536 x 2000 x 400 0.44 ms
+// against 0.70 in TF32, 262144 x 1024 x 256 0.58 against 0.69, but 2^20 x 512 x 512
+// (upper triangular) 2.7 ms against 2.8, 2^20 x 512 x 100 1.32 against 1.24 and
+// 262144 x 2048 x 128, one 128-wide tile, 0.81 against 0.73.
 bool gemm_f32x2_eligible(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda) {
   const int64_t tiles = (M + sl::BM - 1) / sl::BM * ((N + 255) / 256), sms = num_sms();
   return M >= 128 * 96 && N > 128 && (tiles <= sms || 2 * tiles >= 3 * sms) && K >= 1024 && K <= 256 * 64 &&
@@ -448,14 +447,13 @@ int gemm_f32x2(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const f
   SlicedB b;
   TRY_SL((slice_b<__half, S::NB>(d, ar, K, N, tb, B, ldb, &b)));
   if (ar.measure) return BSRHT_OK;
-  // Pairs of row tiles.
-  const int64_t tiles = 2 * ((M + 2 * sl::BM - 1) / (2 * sl::BM)) * ((N + b.bn - 1) / b.bn);
+  const int64_t tiles = (M + sl::BM - 1) / sl::BM * ((N + b.bn - 1) / b.bn);
   if (tiles > 0x7FFFFFFF) return BSRHT_EUNSUP;
   CUtensorMap ma, mb;
   if (!make_tensor_map_2d(&ma, A, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, (uint64_t)M, (uint64_t)K, (uint64_t)lda, S::BK,
                           sl::BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !make_slice_map(&mb, b.slices, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, K, N, S::NB, b.ldk, S::BK,
-                      (uint32_t)b.bn / 2, CU_TENSOR_MAP_SWIZZLE_64B, 1))
+                      (uint32_t)b.bn, CU_TENSOR_MAP_SWIZZLE_64B, 1))
     return BSRHT_EUNSUP;
   sl::F32x2Args g{M, N, K, C, ldc, b.scale, Ct, M, b.bn, b_upper ? 1 : 0, d.status};
   auto launch = [&](auto kern) -> int {

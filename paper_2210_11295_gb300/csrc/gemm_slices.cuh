@@ -27,8 +27,8 @@
 // per product; each K block of 64 starts a fresh accumulator, smallest slice
 // first, which the fold adds to FP32 registers, rounding to nearest (the
 // tensor core's own accumulation truncates).  Bound by the copies of B's three
-// slices from L2 (94 KB a block of K at N = 400): two CTAs load half of B each
-// for both, and C leaves in whole sectors (262144 x 2000 x 400: 1.57 -> 1.20 ms).
+// slices from L2 (94 KB a block of K at N = 400) and the stores of C, which
+// leaves in whole sectors (262144 x 2000 x 400: 1.57 -> 1.20 ms).
 //
 // k_gemm_f32x2: FP32 products of FP32 data at twice the TF32 rate.  An FP16
 // pair holds as much of an FP32 value as a TF32 pair (11 + 11 bits) once it is
@@ -38,12 +38,13 @@
 // power-of-two scale per row and 64 of K, which the 16 fold warps undo when
 // they add the 64 to their FP32 sums: hi lo + lo hi + hi hi, smallest first;
 // what is dropped lies below 2^-23 of each product, or 2^-38 of the row's
-// largest entry in the 64.  Two CTAs (row tiles of one column tile) load half
-// of B each for both.  2^18 x 4096 x 512: 3.0 ms (TF32 form 4.5).  Without the
-// split and the fold it takes 2.2 ms, without two of the three MMAs as well
-// 1.9 ms (copies from L2, 9 TB/s): no single part bounds it, but their use of
+// largest entry in the 64.  2^18 x 4096 x 512: 2.93 ms (TF32 form 4.48).
+// Without the split and the fold it takes 2.2 ms, without two of the three MMAs
+// as well 1.9 ms (copies from L2): no single part bounds it, but their use of
 // shared memory, 152 KB per 32 of K against 768 clocks of MMA.  Measured on the
-// way: the fold warps splitting too, 3.9 ms; folding every 32 of K, 3.3 ms.
+// way: the fold warps splitting too, 3.9 ms; folding every 32 of K, 3.3 ms; two
+// CTAs loading half of B each for both, 2.98 ms (and 1.20 as above for
+// k_gemm_a16): every CTA loads its own.
 #pragma once
 
 #include <cuda.h>
@@ -73,26 +74,6 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
-// The same into both CTAs of a pair: the copy and its byte count arrive at the
-// same offsets of each one's shared memory.
-__device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* map, uint64_t* bar, int32_t x,
-                                                 int32_t y, int32_t z) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster [%0], "
-      "[%1, {%3, %4, %5}], [%2], %6;" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z), "h"((uint16_t)3)
-      : "memory");
-}
-
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
-}
-
 // K-major operand descriptors: rows of 128 bytes (128-byte swizzle, 8-row
 // atoms 1024 bytes apart) or 64 bytes (64-byte swizzle, 512 bytes apart).
 template <int ROW_BYTES>
@@ -119,14 +100,6 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
           d_tmem),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
-      : "memory");
-}
-// Commit that arrives at the same barrier of both CTAs of a pair.
-__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-          smem_u32(bar)),
-      "h"((uint16_t)3)
       : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
@@ -457,7 +430,7 @@ struct A16Args {
   int* err;
 };
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, 1)
     k_gemm_a16(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, A16Args g) {
   using S = A16;
   constexpr int BK = S::BK, STAGES = S::STAGES;
@@ -473,10 +446,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bnw = g.bn;
   const int64_t tn = (g.N + bnw - 1) / bnw;
-  // The pair's two row tiles share one column tile; each CTA loads half of B
-  // for both.
-  const uint32_t rank = cluster_rank();
-  const int64_t pair = (int64_t)blockIdx.x >> 1, bm = 2 * (pair / tn) + rank, bn = pair % tn;
+  const int64_t bm = (int64_t)blockIdx.x / tn, bn = (int64_t)blockIdx.x - bm * tn;
   const int64_t m0 = bm * BM, n0 = bn * bnw;
   const int nkb = (int)((g.K + BK - 1) / BK);
   const uint32_t bslice = (uint32_t)bnw * BK * 2;
@@ -484,7 +454,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 2);
+      mbar_init(&empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&accf[b], 1);
@@ -496,7 +466,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   if (warp == 0) tc::tmem_alloc(tmem_slot, S::TMEM_COLS);
   tc::tc_fence_before();
   __syncthreads();
-  cluster_sync_all();  // the peer's barriers exist before anything arrives at them
   tc::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   bool failed = false;
@@ -515,8 +484,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         tma_load_2d(p, &mapA, &full[s], kb * BK, (int32_t)m0);
 #pragma unroll
         for (int q = 0; q < S::NB; ++q)
-          tma_load_3d_pair(p + S::A_BYTES + q * bslice + rank * (bslice / 2), &mapB, &full[s], kb * BK,
-                           (int32_t)n0 + (int32_t)rank * (bnw / 2), q);
+          tma_load_3d(p + S::A_BYTES + q * bslice, &mapB, &full[s], kb * BK, (int32_t)n0, q);
         issued = kb + 1;
       }
       if (failed)
@@ -546,7 +514,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             mma_f16(d, da + 2 * kk, db + (q * bslice >> 4) + 2 * kk, idesc,
                     (q == S::NB - 1 && kk == 0) ? 0u : 1u);
         }
-        mma_commit_pair(&empty[s]);
+        mma_commit(&empty[s]);
         mma_commit(&accf[b]);
       }
       // Never free TMEM under MMAs that may still run.
@@ -597,7 +565,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc::tc_fence_after();
   if (warp == 0) tc::tmem_dealloc(tmem, S::TMEM_COLS);
-  cluster_sync_all();  // the peer may still copy into this CTA or arrive at its barriers
 }
 
 // ------------------------------------------------ FP32 A, two slices each
@@ -628,7 +595,7 @@ struct F32x2Args {
 };
 
 template <typename TC>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32x2::THREADS, 1)
+__global__ void __launch_bounds__(F32x2::THREADS, 1)
     k_gemm_f32x2(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, F32x2Args g) {
   using S = F32x2;
   constexpr int BK = S::BK, STAGES = S::STAGES, RING = S::RING;
@@ -644,11 +611,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32x2::THREADS, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_rank();
   const int bnw = g.bn;
   const int64_t tn = (g.N + bnw - 1) / bnw;
-  // The pair's two row tiles share one column tile.
-  const int64_t pair = (int64_t)blockIdx.x >> 1, bm = 2 * (pair / tn) + rank, bn = pair % tn;
+  const int64_t bm = (int64_t)blockIdx.x / tn, bn = (int64_t)blockIdx.x - bm * tn;
   const int64_t m0 = bm * BM, n0 = bn * bnw;
   const int64_t kmax = g.b_upper ? (g.K < n0 + bnw ? g.K : n0 + bnw) : g.K;
   const int nkb = (int)((kmax + BK - 1) / BK);
@@ -657,7 +622,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32x2::THREADS, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 2);
+      mbar_init(&empty[s], 1);
     }
     for (int s = 0; s < RING; ++s) mbar_init(&ready[s], S::SPLIT_WARPS);
     for (int b = 0; b < 2; ++b) {
@@ -670,13 +635,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32x2::THREADS, 1)
   if (warp == 0) tc::tmem_alloc(tmem_slot, S::TMEM_COLS);
   tc::tc_fence_before();
   __syncthreads();
-  cluster_sync_all();  // the peer's barriers exist before anything arrives at them
   tc::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   bool failed = false;
 
   if (warp == 0) {
-    if (lane == 0) {  // TMA producer: own rows of A, half of B for both CTAs
+    if (lane == 0) {  // TMA producer
       int issued = 0;
       for (int kb = 0; kb < nkb; ++kb) {
         const int s = kb % STAGES, u = kb / STAGES;
@@ -689,8 +653,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32x2::THREADS, 1)
         tma_load_2d(p, &mapA, &full[s], kb * BK, (int32_t)m0);
 #pragma unroll
         for (int q = 0; q < S::NB; ++q)
-          tma_load_3d_pair(p + S::A_BYTES + q * bslice + rank * (bslice / 2), &mapB, &full[s], kb * BK,
-                           (int32_t)n0 + (int32_t)rank * (bnw / 2), q);
+          tma_load_3d(p + S::A_BYTES + q * bslice, &mapB, &full[s], kb * BK, (int32_t)n0, q);
         issued = kb + 1;
       }
       if (failed)
@@ -722,7 +685,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32x2::THREADS, 1)
         for (int kk = 0; kk < BK / 16; ++kk) mma_f16(d, a_lo + 2 * kk, b_hi + 2 * kk, idesc, 1u);
 #pragma unroll
         for (int kk = 0; kk < BK / 16; ++kk) mma_f16(d, a_hi + 2 * kk, b_hi + 2 * kk, idesc, 1u);
-        mma_commit_pair(&empty[s]);
+        mma_commit(&empty[s]);
         if (!first || kb == nkb - 1) mma_commit(&accf[b]);
       }
       // Never free TMEM under MMAs that may still run.
@@ -841,7 +804,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32x2::THREADS, 1)
   __syncthreads();
   tc::tc_fence_after();
   if (warp == 0) tc::tmem_dealloc(tmem, S::TMEM_COLS);
-  cluster_sync_all();  // the peer may still copy into this CTA or arrive at its barriers
 }
 
 }  // namespace sl
