@@ -897,12 +897,13 @@ __global__ void k_col_norms(const double* __restrict__ M, double* __restrict__ s
   if (lane == 0) sigma[c] = sqrt(s);
 }
 
-// perm[rank] = c with ranks by descending sigma (ties: lower index first).
-// l <= kMaxSvd.
+// perm[rank] = c with ranks by descending sigma (ties: lower index first; NaN
+// as infinity, so that perm is a permutation whatever the data: entries left
+// unwritten would be read as indices).  l <= kMaxSvd.
 constexpr int kMaxSvd = 2048;
 __global__ void k_rank_desc(const double* __restrict__ sigma, int* __restrict__ perm, int64_t l) {
   __shared__ double s[kMaxSvd];
-  for (int e = threadIdx.x; e < l; e += blockDim.x) s[e] = sigma[e];
+  for (int e = threadIdx.x; e < l; e += blockDim.x) s[e] = isnan(sigma[e]) ? (double)INFINITY : sigma[e];
   __syncthreads();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= l) return;
