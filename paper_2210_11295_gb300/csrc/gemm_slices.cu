@@ -219,7 +219,7 @@ constexpr size_t kDigitScratch = (size_t)192 << 20;
 
 // Measured on GB300 (int8x7 against the CUDA-core GEMM, FP64): below about 20
 // million FMAs the preparation's launches cost more than they save (256^3
-// 0.048 / 0.049 ms, 300^3 0.049 / 0.085, 400^3 0.052 / 0.195).
+// 0.051 / 0.050 ms, 300^3 0.050 / 0.083, 400^3 0.053 / 0.197).
 bool gemm_int8x7_wants(int64_t M, int64_t N, int64_t K) {
   return M >= 32 && N >= 16 && K >= 32 && (double)M * (double)N * (double)K >= 2e7;
 }

@@ -12,13 +12,16 @@
 // 128, exact in FP16).  A product of two digits is at most 2^14, so the FP32
 // accumulators add up to 7 x 128 of them (2^23.8) without rounding.  The
 // digit products of equal weight, i + j = c, share one accumulator; classes
-// c = 0 .. 6 are formed (28 of 49 products), the rest lies below 2^-55 of
-// the row's and the column's largest entries.  After every 128 columns of K the
-// seven accumulators are folded into two 64-bit integers per entry, and the
-// sum is rounded to FP64 once, at the end.  Bound by shared memory: an MMA
-// of 128 x 64 x 16 reads 6 KB (48 clocks against 32 of tensor work), 56 of them
-// and the copies of a stage come to 1.8 us, measured 2.7 us a stage of 32 of K.
-// 131072 x 2048 x 256: 6.05 ms with the digits' preparation (FP64 units: 110 ms).
+// c = 0 .. 7 are formed (34 of 49 products).  What is left out lies below 2^-59
+// of the row's and the column's largest entries, under the 2^-54 of the two
+// operands' rounding.  (Without class 7 it reaches 2^-51.4, and rows whose
+// entries spread over 2^40 came out up to seven times as far off as on the FP64
+// units.)  After every 128 columns of K the eight accumulators, all of tensor
+// memory, are folded into two 64-bit integers per entry, and the sum is rounded
+// to FP64 once, at the end.  Bound by shared memory: an MMA of 128 x 64 x 16
+// reads 6 KB (48 clocks against 32 of tensor work), 68 of them and the copies of
+// a stage come to 2.1 us, measured about 3 us a stage of 32 of K.
+// 131072 x 2048 x 256: 6.8 ms with the digits' preparation (FP64 units: 110 ms).
 //
 // k_gemm_a16: FP32-accurate products of 16-bit data.  A (BF16 or FP16) is
 // exact as it is stored and comes in by TMA straight into the MMA operand;
@@ -58,6 +61,7 @@ namespace bsrht {
 namespace sl {
 
 constexpr int kDig = 7;               // digits of an FP64 operand
+constexpr int kCls = 8;               // classes of digit products that are formed
 constexpr int BM = 128;
 constexpr uint32_t kWaitSl = 1u << 24;  // bounded mbarrier waits
 constexpr int kErrSl = 8;             // status bit of a failed wait (kStatusTcWait)
@@ -188,7 +192,7 @@ struct Int8x7 {
   static constexpr uint32_t A_BYTES = kDig * A_SLICE, B_BYTES = kDig * B_SLICE;
   static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr size_t smem_bytes() { return 1024 + (size_t)STAGES * STAGE_BYTES + 256; }
-  static constexpr uint32_t TMEM_COLS = 512;  // 7 x 64 used
+  static constexpr uint32_t TMEM_COLS = kCls * BN;
   // Exact sums: 2^14 per product, at most 7 products a class, KG BK columns.
   static_assert(kDig * KG * BK * (1 << 14) <= (1 << 24), "exact FP32 accumulation");
   static_assert(A_SLICE % 1024 == 0 && B_SLICE % 1024 == 0, "swizzle atoms");
@@ -216,9 +220,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   unsigned char* base = smem_raw + ((1024 - (reinterpret_cast<uintptr_t>(smem_raw) & 1023)) & 1023);
   uint64_t* full = reinterpret_cast<uint64_t*>(base + STAGES * S::STAGE_BYTES);
   uint64_t* empty = full + STAGES;
-  uint64_t* accf = empty + STAGES;     // [7] class finished
-  uint64_t* accfree = accf + kDig;     // [7] class folded
-  uint64_t* drain = accfree + kDig;    // every MMA issued has finished
+  uint64_t* accf = empty + STAGES;     // [kCls] class finished
+  uint64_t* accfree = accf + kCls;     // [kCls] class folded
+  uint64_t* drain = accfree + kCls;    // every MMA issued has finished
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -240,7 +244,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    for (int c = 0; c < kDig; ++c) {
+    for (int c = 0; c < kCls; ++c) {
       mbar_init(&accf[c], 1);
       mbar_init(&accfree[c], 8);
     }
@@ -293,18 +297,19 @@ __global__ void __launch_bounds__(kThreads, 1)
         // and is folded as soon as it is complete.
         const uint64_t da = desc_k<64>(a0), db = desc_k<64>(b0);
 #pragma unroll
-        for (int c = 0; c < kDig; ++c) {
+        for (int c = 0; c < kCls; ++c) {
           if (first && grp > 0 && !failed) {
             failed = !mbar_wait_bounded(&accfree[c], (uint32_t)((grp - 1) & 1), kWaitSl);
             tc::tc_fence_after();
           }
           if (!failed) {
 #pragma unroll
-            for (int i = 0; i <= c; ++i) {
+            for (int i = c < kDig ? 0 : c - kDig + 1; i <= c && i < kDig; ++i) {
 #pragma unroll
               for (int kk = 0; kk < BK / 16; ++kk)
                 mma_f16(tmem + (uint32_t)(c * BN), da + ((i * S::A_SLICE + 32 * kk) >> 4),
-                        db + (((c - i) * S::B_SLICE + 32 * kk) >> 4), idesc, (first && i == 0 && kk == 0) ? 0u : 1u);
+                        db + (((c - i) * S::B_SLICE + 32 * kk) >> 4), idesc,
+                        (first && (i == 0 || c - i == kDig - 1) && kk == 0) ? 0u : 1u);
             }
             if (last) mma_commit(&accf[c]);
           }
@@ -340,9 +345,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       return true;
     };
     for (int grp = 0; grp < ngroups && !failed; ++grp) {
-      failed = !(fold(0, grp, H, 1 << 16) && fold(1, grp, H, 1 << 8) && fold(2, grp, H, 1) &&
-                 fold(3, grp, L, 1 << 24) && fold(4, grp, L, 1 << 16) && fold(5, grp, L, 1 << 8) &&
-                 fold(6, grp, L, 1));
+      failed = !(fold(0, grp, H, 1 << 24) && fold(1, grp, H, 1 << 16) && fold(2, grp, H, 1 << 8) &&
+                 fold(3, grp, H, 1) && fold(4, grp, L, 1 << 24) && fold(5, grp, L, 1 << 16) &&
+                 fold(6, grp, L, 1 << 8) && fold(7, grp, L, 1));
     }
     const int64_t row = m0 + 32 * wq + lane;
     const int64_t c0 = n0 + 32 * ch;
@@ -353,8 +358,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int q = 0; q < 32; ++q) {
         if (c0 + q >= g.N) break;
         const int eb = g.eb[c0 + q];
-        // Entry scales 2^(E - 1022 - 55) each; weights 2^48 and up.
-        double v = scale_int(H[q], L[q], 48 + (ea - 1077) + (eb - 1077));
+        // Entry scales 2^(E - 1022 - 55) each; weights 2^40 and up.
+        double v = scale_int(H[q], L[q], 40 + (ea - 1077) + (eb - 1077));
         if (failed || ea >= kNonFiniteExp || eb >= kNonFiniteExp) v = __longlong_as_double(0x7ff8000000000000ll);
         dst[q] = v;
       }

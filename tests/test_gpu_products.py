@@ -1,0 +1,143 @@
+"""The products on 16-bit slices by themselves (dla.cuh), entry by entry: each
+row of A and column of B has its own scale, so every entry is held against the
+largest entries, or the norms, of its own row and column.
+
+Tolerances: FP64 in seven digits, K 2^-54 (both operands' rounding) + K 2^-59
+(digit products left out) times the row's and the column's largest entries, and
+2^-53 of the entry (rounded once, and once more per part of a split K).  FP32
+arithmetic: two FP16 slices of each operand drop 2^-22 of a product, FP32 sums over
+a chunk of K a few 2^-24 more: 2^-20 of the row's and the column's norms.
+"""
+
+import ctypes
+from fractions import Fraction
+
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+F64, F32, BF16, F16 = 0, 1, 2, 3  # bsrht::DT
+
+
+class _Arena(ctypes.Structure):  # bsrht::Arena
+    _fields_ = [("base", ctypes.c_void_p), ("cap", ctypes.c_size_t), ("used", ctypes.c_size_t),
+                ("high", ctypes.c_size_t), ("measure", ctypes.c_bool), ("lean", ctypes.c_bool)]
+
+
+class _Dla(ctypes.Structure):  # bsrht::Dla
+    _fields_ = [("s", ctypes.c_void_p), ("status", ctypes.c_void_p)]
+
+
+class _Products:
+    """The library's internal products, by their mangled names."""
+
+    def __init__(self, lib):
+        i64, vp, ci, cb = ctypes.c_int64, ctypes.c_void_p, ctypes.c_int, ctypes.c_bool
+        head = [ctypes.POINTER(_Dla), ctypes.POINTER(_Arena)]
+        self.int8x7 = getattr(lib, "_ZN5bsrht11gemm_int8x7ERKNS_3DlaERNS_5ArenaElllPKdlbS6_lPdlbb")
+        self.int8x7.argtypes = head + [i64, i64, i64, vp, i64, cb, vp, i64, vp, i64, cb, cb]
+        self.f32x2 = getattr(lib, "_ZN5bsrht10gemm_f32x2ERKNS_3DlaERNS_5ArenaElllPKflNS_2DTEPKvlS7_PvlbPf")
+        self.f32x2.argtypes = head + [i64, i64, i64, vp, i64, ci, vp, i64, ci, vp, i64, cb, vp]
+        self.a16 = getattr(lib, "_ZN5bsrht8gemm_a16ERKNS_3DlaERNS_5ArenaENS_2DTElllPKvlS5_S7_lPflS8_")
+        self.a16.argtypes = head + [ci, i64, i64, i64, vp, i64, ci, vp, i64, vp, i64, vp]
+        self.scratch = torch.empty(256 << 20, device="cuda", dtype=torch.uint8)
+        self.status = torch.zeros(64, device="cuda", dtype=torch.int32)
+
+    def run(self, fn, *args):
+        torch.cuda.synchronize()
+        d = _Dla(torch.cuda.current_stream().cuda_stream, self.status.data_ptr())
+        ar = _Arena(self.scratch.data_ptr(), self.scratch.numel(), 0, 0, False, False)
+        st = fn(ctypes.byref(d), ctypes.byref(ar), *args)
+        torch.cuda.synchronize()
+        assert st == 0 and int(self.status[0]) == 0
+
+
+@pytest.fixture(scope="module")
+def prod():
+    import paper_2210_11295_gb300._binding as b
+
+    return _Products(b.lib)
+
+
+def _spread(rng, rows, cols, axis, lo, hi):
+    x = rng.standard_normal((rows, cols))
+    return x * np.exp2(rng.integers(lo, hi + 1, size=(rows, 1) if axis == 0 else (1, cols)))
+
+
+@pytest.mark.parametrize("K", [1, 40, 1000])
+def test_digits_of_one_sign(prod, K):
+    """Every digit product that is left out has the same sign."""
+    t = 65 * 2**48 - 128 * ((2**48 - 1) // 255)  # digits 65, -128, -128, ...
+    v = float(t)
+    assert int(v) == t
+    M, N = 130, 70
+    a = torch.full((M, K), v, device="cuda", dtype=torch.float64)
+    b = torch.full((K, N), v, device="cuda", dtype=torch.float64)
+    c = torch.empty(M, N, device="cuda", dtype=torch.float64)
+    prod.run(prod.int8x7, M, N, K, a.data_ptr(), K, False, b.data_ptr(), N, c.data_ptr(), N, False, False)
+    exact = Fraction(t) ** 2 * K
+    got = c.unique().cpu().tolist()
+    assert len(got) == 1
+    assert abs(Fraction(got[0]) - exact) <= exact * (Fraction(1, 2**53) + Fraction(1, 2**59))
+
+
+@pytest.mark.parametrize("M,N,K,trans,gram,upper", [
+    (129, 65, 257, False, False, False),
+    (300, 300, 300, False, False, True),
+    (100, 70, 1000, True, False, False),
+    (130, 130, 4000, True, True, False),
+])
+def test_fp64_per_entry(prod, M, N, K, trans, gram, upper):
+    rng = np.random.default_rng(M + K)
+    a = _spread(rng, M, K, 0, -30, 30)  # op(A)
+    b = a.T.copy() if gram else _spread(rng, K, N, 1, -30, 30)
+    if upper:
+        b = np.triu(b)
+    stored = torch.from_numpy(np.ascontiguousarray(a.T if trans else a)).cuda()
+    bd = stored if gram else torch.from_numpy(b).cuda()
+    c = torch.empty(M, N, device="cuda", dtype=torch.float64)
+    prod.run(prod.int8x7, M, N, K, stored.data_ptr(), M if trans else K, trans, bd.data_ptr(), N, c.data_ptr(), N,
+             upper, gram)
+    exact = np.matmul(a.astype(np.longdouble), b.astype(np.longdouble))
+    largest = np.abs(a).max(1)[:, None] * np.abs(b).max(0)[None, :]
+    off = np.abs(c.cpu().numpy() - exact)
+    parts = 64  # a split K: sums of at most as many rounded parts
+    assert np.all(off <= (K * 2.0**-54 + K * 2.0**-59) * largest + 2.0**-53 * np.abs(exact)
+                  + (0 if K < 512 else parts * 2.0**-53 * K * largest))
+
+
+@pytest.mark.parametrize("M,N,K,f64out", [(300, 130, 257, False), (257, 272, 1000, True), (12290, 40, 96, False)])
+def test_fp32_per_row(prod, M, N, K, f64out):
+    rng = np.random.default_rng(M + K)
+    lda = (K + 3) // 4 * 4
+    a = _spread(rng, M, K, 0, -40, 0).astype(np.float32)
+    b = _spread(rng, K, N, 1, -20, 20)
+    buf = torch.zeros(M, lda)
+    buf[:, :K] = torch.from_numpy(a)
+    ad, bd = buf.cuda(), torch.from_numpy(b).cuda()
+    c = torch.empty(M, N, device="cuda", dtype=torch.float64 if f64out else torch.float32)
+    prod.run(prod.f32x2, M, N, K, ad.data_ptr(), lda, F64, bd.data_ptr(), N, F64 if f64out else F32, c.data_ptr(), N,
+             False, None)
+    exact = a.astype(np.float64) @ b
+    norms = np.linalg.norm(a.astype(np.float64), axis=1)[:, None] * np.linalg.norm(b, axis=0)[None, :]
+    assert np.all(np.abs(c.double().cpu().numpy() - exact) <= 2.0**-20 * norms)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("M,N,K", [(300, 130, 256), (257, 272, 1000)])
+def test_16bit_per_row(prod, dtype, M, N, K):
+    rng = np.random.default_rng(M + K)
+    a = torch.from_numpy(_spread(rng, M, K, 0, -10, 0)).to(dtype)
+    b = _spread(rng, K, N, 1, -20, 20)
+    ad, bd = a.cuda(), torch.from_numpy(b).cuda()
+    c = torch.empty(M, N, device="cuda", dtype=torch.float32)
+    ct = torch.empty(N, M, device="cuda", dtype=torch.float32)
+    prod.run(prod.a16, BF16 if dtype is torch.bfloat16 else F16, M, N, K, ad.data_ptr(), K, F64, bd.data_ptr(), N,
+             c.data_ptr(), N, ct.data_ptr())
+    vals = a.double().numpy()
+    exact = vals @ b
+    norms = np.linalg.norm(vals, axis=1)[:, None] * np.linalg.norm(b, axis=0)[None, :]
+    assert np.all(np.abs(c.double().cpu().numpy() - exact) <= 2.0**-20 * norms)
+    assert torch.equal(ct.T, c)
