@@ -231,14 +231,16 @@ int gemm_int8x7(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const 
   if (gram && !a_trans) return BSRHT_EUNSUP;
   if (gram || a_trans) b_upper = false;
   const int64_t tn = (N + S::BN - 1) / S::BN;
-  const size_t avail = ar.measure ? (size_t)-1 : (ar.cap > ar.used + 4096 ? ar.cap - ar.used - 4096 : 0);
+  // What take() below uses, to the byte: a product that is the peak of a call
+  // runs as it was measured in a workspace of the measured size.
+  auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+  const size_t avail = ar.measure ? (size_t)-1 : (ar.cap > up(ar.used) ? ar.cap - up(ar.used) : 0);
   const int64_t sms = num_sms();
   // Rows of A (A^T: columns of K) whose digits are made and used at a time.
   // Both dimensions of a pass stay small enough that the digits of one pass
   // fit the scratch; the split of K fills the SMs when the tiles do not.
   int64_t mc = M, kc = K;
   const int64_t ldk_full = round_up(K, 8);
-  size_t fixed = sizeof(int) * (size_t)(M + N) + 4096;
   int splits = 1, passes = 1;
   auto tiles_of = [&](int64_t m) {
     int64_t t = 0;
@@ -252,10 +254,16 @@ int gemm_int8x7(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const 
     if (tiles >= sms) return (int64_t)1;
     return std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>((sms + tiles / 2) / tiles, groups), 64));
   };
-  size_t need = 0;
+  auto need = [&]() {
+    const int64_t rows = a_trans ? M : mc, ld = a_trans ? round_up(kc, 8) : ldk_full;
+    const bool part = splits > 1 || gram || (a_trans && passes > 1);
+    return up(digit_bytes_of(N, ld)) + up(sizeof(int) * (size_t)N) +
+           (gram ? 0 : up(digit_bytes_of(rows, ld)) + up(sizeof(int) * (size_t)rows)) +
+           (part ? sizeof(double) * (size_t)(a_trans ? splits * passes : splits) * (size_t)M * (size_t)N : 0);
+  };
   if (!a_trans) {
-    const size_t bb = digit_bytes_of(N, ldk_full);
-    const size_t budget = std::min(kDigitScratch, avail > fixed + bb ? avail - fixed - bb : 0);
+    const size_t of_b = up(digit_bytes_of(N, ldk_full)) + up(sizeof(int) * (size_t)N);
+    const size_t budget = std::min(kDigitScratch, avail > of_b ? avail - of_b : 0);
     const int64_t fit = (int64_t)(budget / digit_bytes_of(1, ldk_full));
     if (fit < std::min<int64_t>(M, sl::BM)) return BSRHT_EUNSUP;
     if (mc > fit) {
@@ -263,14 +271,11 @@ int gemm_int8x7(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const 
       // Whole waves of tiles when a pass holds at least one.
       const int64_t wave = std::max<int64_t>(1, sms / tn) * sl::BM;
       if (mc > wave) mc = mc / wave * wave;
-      passes = (int)((M + mc - 1) / mc);
     }
     splits = (int)splits_of(tiles_of(mc), K);
-    need = fixed + bb + digit_bytes_of(mc, ldk_full) + (splits > 1 ? sizeof(double) * (size_t)splits * M * N : 0);
-    if (need > avail && splits > 1) {
-      splits = 1;
-      need = fixed + bb + digit_bytes_of(mc, ldk_full);
-    }
+    if (need() > avail) splits = 1;
+    while (need() > avail && mc > sl::BM) mc = (mc - 1) / sl::BM * sl::BM;
+    passes = (int)((M + mc - 1) / mc);
   } else {
     const size_t per_k = digit_bytes_of(gram ? N : M + N, 8) / 8;
     const int64_t groups_min = S::KG * S::BK;
@@ -282,16 +287,12 @@ int gemm_int8x7(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const 
       kc = std::min<int64_t>(K, round_up((K + passes - 1) / passes, groups_min));
       passes = (int)((K + kc - 1) / kc);
       splits = (int)splits_of(tiles, kc);
-      need = fixed + digit_bytes_of(gram ? N : M + N, round_up(kc, 8)) +
-             sizeof(double) * (size_t)splits * (size_t)passes * M * N;
       return true;
     };
     if (!plan(kDigitScratch)) return BSRHT_EUNSUP;
-    if (need > avail) {
-      if (avail < fixed || !plan(std::min(kDigitScratch, (avail - fixed) / 2))) return BSRHT_EUNSUP;
-    }
+    if (need() > avail && !plan(std::min(kDigitScratch, avail / 2))) return BSRHT_EUNSUP;
   }
-  if (need > avail) return BSRHT_EUNSUP;
+  if (need() > avail) return BSRHT_EUNSUP;
   const int64_t ldk = round_up(a_trans ? kc : K, 8);
   uint32_t* bd = static_cast<uint32_t*>(ar.take(digit_bytes_of(N, ldk)));
   uint32_t* ad = gram ? bd : static_cast<uint32_t*>(ar.take(digit_bytes_of(a_trans ? M : mc, ldk)));

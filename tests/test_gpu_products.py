@@ -42,13 +42,20 @@ class _Products:
         self.f32x2.argtypes = head + [i64, i64, i64, vp, i64, ci, vp, i64, ci, vp, i64, cb, vp]
         self.a16 = getattr(lib, "_ZN5bsrht8gemm_a16ERKNS_3DlaERNS_5ArenaENS_2DTElllPKvlS5_S7_lPflS8_")
         self.a16.argtypes = head + [ci, i64, i64, i64, vp, i64, ci, vp, i64, vp, i64, vp]
-        self.scratch = torch.empty(256 << 20, device="cuda", dtype=torch.uint8)
+        self.scratch = torch.empty(1 << 30, device="cuda", dtype=torch.uint8)
         self.status = torch.zeros(64, device="cuda", dtype=torch.int32)
 
-    def run(self, fn, *args):
+    def measure(self, fn, *args):
+        """Bytes of scratch that a call of these sizes takes, with the slack that the workspace queries add."""
+        d = _Dla(None, None)
+        ar = _Arena(None, 0, 0, 0, True, False)
+        assert fn(ctypes.byref(d), ctypes.byref(ar), *args) == 0
+        return ar.high + 256
+
+    def run(self, fn, *args, scratch=None):
         torch.cuda.synchronize()
         d = _Dla(torch.cuda.current_stream().cuda_stream, self.status.data_ptr())
-        ar = _Arena(self.scratch.data_ptr(), self.scratch.numel(), 0, 0, False, False)
+        ar = _Arena(self.scratch.data_ptr(), scratch or self.scratch.numel(), 0, 0, False, False)
         st = fn(ctypes.byref(d), ctypes.byref(ar), *args)
         torch.cuda.synchronize()
         assert st == 0 and int(self.status[0]) == 0
@@ -141,3 +148,29 @@ def test_16bit_per_row(prod, dtype, M, N, K):
     norms = np.linalg.norm(vals, axis=1)[:, None] * np.linalg.norm(b, axis=0)[None, :]
     assert np.all(np.abs(c.double().cpu().numpy() - exact) <= 2.0**-20 * norms)
     assert torch.equal(ct.T, c)
+
+
+@pytest.mark.parametrize("M,N,K,trans,gram", [
+    (1000, 130, 257, False, False),   # split K
+    (40000, 100, 700, False, False),  # several passes over the rows
+    (300, 200, 60000, True, False),   # several passes over K
+    (256, 256, 100000, True, True),
+])
+def test_fp64_scratch_as_measured(prod, M, N, K, trans, gram):
+    """The scratch that is measured for a product holds it: the same launches as with ample scratch."""
+    import paper_2210_11295_gb300 as lib
+
+    a = torch.randn((K, M) if trans else (M, K), device="cuda", dtype=torch.float64)
+    b = a if gram else torch.randn(K, N, device="cuda", dtype=torch.float64)
+    c = torch.empty(M, N, device="cuda", dtype=torch.float64)
+    args = (M, N, K, a.data_ptr(), M if trans else K, trans, b.data_ptr(), N, c.data_ptr(), N, False, gram)
+
+    def launches(scratch):
+        before = lib.bsrht_kernel_launches()
+        prod.run(prod.int8x7, *args, scratch=scratch)
+        return lib.bsrht_kernel_launches() - before
+
+    ample = launches(None)
+    full = c.clone()
+    assert launches(prod.measure(prod.int8x7, *args)) == ample
+    assert torch.equal(c, full)
