@@ -1600,7 +1600,7 @@ int launch_jacobi_cluster_jq(const Dla& d, jc::Args a, int nc) {
 }
 
 int launch_jacobi_cluster(const Dla& d, float* X, int64_t l, double tol, double tol_stop, double tiny, int64_t lead,
-                          int max_sweeps, int* rot, float* nrm) {
+                          int64_t need, int max_sweeps, int* rot, float* nrm) {
   if (l < 2 || l > jc::kMaxRows) return BSRHT_EUNSUP;
   const int nc = l <= 64 ? 2 : l <= 128 ? 4 : l <= 256 ? 8 : 16;
   jc::Args a;
@@ -1612,6 +1612,7 @@ int launch_jacobi_cluster(const Dla& d, float* X, int64_t l, double tol, double 
   a.tstop2 = (float)(tol_stop * tol_stop);
   a.tiny2 = (float)(tiny * tiny);
   a.lead = (int)lead;
+  a.need = (int)need;
   a.max_sweeps = max_sweeps;
   a.rot_counts = rot;
   a.nrm = nrm;
@@ -1780,7 +1781,9 @@ int jacobi_svd(const Dla& d, Arena& ar, double* colsM, int64_t l, double* U, dou
     // last sweep then leaves cosines of rounding size.
     const double tstop32 = 16.0 * std::sqrt((double)l) * 0x1.0p-24;
     const int64_t lead = part && ktop > 0 ? s : 0;
-    const int st = launch_jacobi_cluster(d, X, l, 0x1.0p-21, tstop32, (double)l * 0x1.0p-24, lead, 20,
+    // (With keep_rel alone the columns above its threshold are wanted, however few.)
+    const int64_t need = part && ktop <= 0 ? 0 : s;
+    const int st = launch_jacobi_cluster(d, X, l, 0x1.0p-21, tstop32, (double)l * 0x1.0p-24, lead, need, 20,
                                          rot + max_sweeps, nrm);
     if (st == BSRHT_EUNSUP) return BSRHT_OK;
     if (st != BSRHT_OK) return st;

@@ -12,6 +12,7 @@ import pytest
 import torch
 
 import synth
+from oracle import lowrank as orc
 
 pytestmark = pytest.mark.gpu
 
@@ -67,3 +68,23 @@ def test_nystrom_close_values(lib, l, spread):
     assert _orth_error(u) <= 1e-12
     assert np.max(np.abs(got - lam[:k])) <= 1e-7 * lam[0]
     assert np.linalg.norm(a @ u - u * got) <= 1e-7 * np.linalg.norm(a)
+
+
+@pytest.mark.parametrize("l,decay", [(80, 4.0), (128, 8.0), (300, 15.0), (700, 40.0)])
+def test_rsvd_core_singular_in_fp32(lib, l, decay):
+    """exp(-i / decay): the l x l core reaches below FP32's rounding of its
+    largest value (2e-9 to 2.5e-8), so its FP32 phase gives no basis.  (Omega has
+    a repeated row at l = 300 and 700: the rank-k part is the oracle's, off A's
+    by 3e-9 and 3e-8.)"""
+    rng = np.random.default_rng(l)
+    sigma = np.exp(-np.arange(l) / decay)
+    n, m, k = 8192, l + 13, 20
+    uu, vv = synth.haar(n, l, rng), synth.haar(m, l, rng)
+    a = np.ascontiguousarray((uu * sigma) @ vv.T)
+    u, s, v = (x.cpu().numpy() for x in lib.bsrht_rsvd(torch.from_numpy(a).cuda(), k, l, 16, 3))
+    assert _orth_error(v) <= 1e-12
+    assert _orth_error(u) <= 1e-12
+    assert np.max(np.abs(s - sigma[:k])) <= 1e-12
+    ur, sr, vr = orc.rsvd(a, k, l, 16, 3)
+    ref = (ur * sr) @ vr.T
+    assert np.linalg.norm((u * s) @ v.T - ref) <= 1e-12 * np.linalg.norm(ref)
