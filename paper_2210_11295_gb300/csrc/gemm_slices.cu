@@ -111,14 +111,17 @@ __global__ void k_int8x7_reduce(const double* __restrict__ P, double* __restrict
 }
 
 // NS 16-bit slices of the columns of B (K x N, row-major, read as FP32),
-// K-major: out[s][c][k], row length ldk.  With 2^(E - 127) <= max |column| <
-// 2^(E - 126) the column is scaled by 2^(140 - E), so its largest entry lies in [2^13, 2^14)
-// (FP16's range with 2^-24 as the smallest step); scale[c] undoes that.
+// K-major: out[s][c][k], row length ldk; scale[c] undoes the column's power of
+// two.  FP16: with 2^(E - 127) <= max |column| < 2^(E - 126) the column is scaled
+// by 2^(140 - E), so its largest entry lies in [2^13, 2^14) (FP16's range with
+// 2^-24 as the smallest step).  BF16 has FP32's range and A is not scaled: only
+// columns above 1, or so small that the last slice would be subnormal, are, so
+// that no sum overflows that the product itself does not.
 template <typename TB, typename T16, int NS>
 __global__ void __launch_bounds__(256) k_slices16_cols(const TB* __restrict__ B, int64_t K, int64_t N, int64_t ldb,
                                                        T16* __restrict__ out, int64_t ldk,
                                                        const int* __restrict__ exps, int64_t tiles_n,
-                                                       float* __restrict__ scale) {
+                                                       float* __restrict__ scale, float undo) {
   __shared__ float t[64][65];
   const int64_t tk = (int64_t)blockIdx.x / tiles_n, tb = (int64_t)blockIdx.x - tk * tiles_n;
   const int64_t k0 = tk * 64, c0 = tb * 64;
@@ -139,9 +142,11 @@ __global__ void __launch_bounds__(256) k_slices16_cols(const TB* __restrict__ B,
     if (c >= N) continue;
     // exps: FP32 biased exponents.  Columns at the ends of the range are
     // scaled as far as one FP32 factor and its inverse reach.
-    const int sh = min(max(140 - exps[c], -126), 126);
+    const int E = exps[c];
+    const int sh = std::is_same<T16, __half>::value ? min(max(140 - E, -126), 126)
+                                                    : (E > 127 ? 127 - E : E < 63 ? 63 - E : 0);
     const float f = __uint_as_float((uint32_t)(127 + sh) << 23);
-    if (tk == 0 && tx == 0) scale[c] = __uint_as_float((uint32_t)(127 - sh) << 23);
+    if (tk == 0 && tx == 0) scale[c] = __uint_as_float((uint32_t)(127 - sh) << 23) * undo;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int64_t k = k0 + tx + 32 * h;
@@ -363,7 +368,8 @@ size_t sliced_b_bytes(int64_t K, int64_t N, int ns) {
 }
 
 template <typename T16, int NS>
-int slice_b(const Dla& d, Arena& ar, int64_t K, int64_t N, DT tb, const void* B, int64_t ldb, SlicedB* out) {
+int slice_b(const Dla& d, Arena& ar, int64_t K, int64_t N, DT tb, const void* B, int64_t ldb, SlicedB* out,
+            float undo = 1.f) {
   out->ldk = round_up(K, 8);
   out->slices = ar.take(2 * (size_t)NS * (size_t)N * out->ldk);
   int* exps = static_cast<int*>(ar.take(sizeof(int) * (size_t)N));
@@ -380,7 +386,7 @@ int slice_b(const Dla& d, Arena& ar, int64_t K, int64_t N, DT tb, const void* B,
     using TB = std::remove_pointer_t<decltype(b)>;
     k_col_exps32<TB><<<dim3(cb, ry), 64, 0, d.s>>>(b, K, N, ldb, (K + ry - 1) / ry, exps);
     k_slices16_cols<TB, T16, NS><<<(unsigned)tk, 256, 0, d.s>>>(b, K, N, ldb, static_cast<T16*>(out->slices), out->ldk,
-                                                                 exps, t64, out->scale);
+                                                                 exps, t64, out->scale, undo);
   };
   if (tb == DT::F64)
     prep(static_cast<const double*>(B));
@@ -446,7 +452,7 @@ int gemm_f32x2(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const f
   if ((tb != DT::F32 && tb != DT::F64) || (tc_out != DT::F32 && tc_out != DT::F64)) return BSRHT_EUNSUP;
   if (!ar.measure && ar.used + sliced_b_bytes(K, N, S::NB) > ar.cap) return BSRHT_EUNSUP;
   SlicedB b;
-  TRY_SL((slice_b<__half, S::NB>(d, ar, K, N, tb, B, ldb, &b)));
+  TRY_SL((slice_b<__half, S::NB>(d, ar, K, N, tb, B, ldb, &b, 1.f / S::LOWER)));
   if (ar.measure) return BSRHT_OK;
   const int64_t tiles = (M + sl::BM - 1) / sl::BM * ((N + b.bn - 1) / b.bn);
   if (tiles > 0x7FFFFFFF) return BSRHT_EUNSUP;

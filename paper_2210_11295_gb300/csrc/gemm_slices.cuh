@@ -26,7 +26,7 @@
 // k_gemm_a16: FP32-accurate products of 16-bit data.  A (BF16 or FP16) is
 // exact as it is stored and comes in by TMA straight into the MMA operand;
 // B (FP32 values) is split once into three slices of A's type (24 bits in
-// BF16, 33 in FP16), scaled per column to FP16's range.  Three 16-bit MMAs
+// BF16, 33 in FP16), for FP16 scaled per column to its range.  Three 16-bit MMAs
 // per product; each K block of 64 starts a fresh accumulator, smallest slice
 // first, which the fold adds to FP32 registers, rounding to nearest (the
 // tensor core's own accumulation truncates).  Bound by the copies of B's three
@@ -580,6 +580,10 @@ struct F32x2 {
   static constexpr uint32_t STAGE_BYTES = A_BYTES + NB * B_SLICE_MAX;
   static constexpr int RING = 8;  // K blocks whose split is remembered; half as many row scales
   static constexpr int SPLIT_WARPS = 4, FOLD_WARPS = 16, NC = 64;
+  // The sums are kept at LOWER times B's scale over the product: divided by the
+  // column's largest entry, 2^-11 to 1 in an orthonormal one.  (At B's own scale,
+  // 2^13 more, they overflowed where the product was above 2^111.)
+  static constexpr float LOWER = 0x1.0p-13f;
   static constexpr int THREADS = 32 * (2 + SPLIT_WARPS + FOLD_WARPS);
   static constexpr size_t smem_bytes() { return 1024 + (size_t)STAGES * STAGE_BYTES + RING / 2 * BM * 4 + 256; }
   static constexpr uint32_t TMEM_COLS = 2 * BNMAX;
@@ -591,7 +595,7 @@ struct F32x2Args {
   int64_t M, N, K;
   void* C;
   int64_t ldc;
-  const float* bscale;  // undoes the column scale of B's slices
+  const float* bscale;  // undoes the column scale of B's slices and LOWER
   float* Ct;            // optional FP32 copy of C transposed (N x M)
   int64_t ldct;
   int bn;               // tile width: a multiple of 16, at most 256
@@ -752,7 +756,7 @@ __global__ void __launch_bounds__(F32x2::THREADS, 1)
       // Largest entry into [2^13, 2^14).
       const int sh = min(max(140 - (int)(mx >> 23), -126), 126);
       const float sc = __uint_as_float((uint32_t)(127 + sh) << 23);
-      rscale[(kb / 2) % (RING / 2) * BM + r] = __uint_as_float((uint32_t)(127 - sh) << 23);
+      rscale[(kb / 2) % (RING / 2) * BM + r] = __uint_as_float((uint32_t)(127 - sh) << 23) * S::LOWER;
       split(kb, x, sc);
       if (two) {
         load(kb + 1, x, 0u);

@@ -115,21 +115,41 @@ def test_fp64_per_entry(prod, M, N, K, trans, gram, upper):
                   + (0 if K < 512 else parts * 2.0**-53 * K * largest))
 
 
-@pytest.mark.parametrize("M,N,K,f64out", [(300, 130, 257, False), (257, 272, 1000, True), (12290, 40, 96, False)])
-def test_fp32_per_row(prod, M, N, K, f64out):
-    rng = np.random.default_rng(M + K)
+def _check_fp32(c, a, b):
+    exact = a @ b
+    norms = np.linalg.norm(a, axis=1)[:, None] * np.linalg.norm(b, axis=0)[None, :]
+    assert np.all(np.abs(c.double().cpu().numpy() - exact) <= 2.0**-20 * norms)
+
+
+def _f32x2(prod, a, b, f64out=False):
+    (M, K), N = a.shape, b.shape[1]
     lda = (K + 3) // 4 * 4
-    a = _spread(rng, M, K, 0, -40, 0).astype(np.float32)
-    b = _spread(rng, K, N, 1, -20, 20)
     buf = torch.zeros(M, lda)
     buf[:, :K] = torch.from_numpy(a)
     ad, bd = buf.cuda(), torch.from_numpy(b).cuda()
     c = torch.empty(M, N, device="cuda", dtype=torch.float64 if f64out else torch.float32)
     prod.run(prod.f32x2, M, N, K, ad.data_ptr(), lda, F64, bd.data_ptr(), N, F64 if f64out else F32, c.data_ptr(), N,
              False, None)
-    exact = a.astype(np.float64) @ b
-    norms = np.linalg.norm(a.astype(np.float64), axis=1)[:, None] * np.linalg.norm(b, axis=0)[None, :]
-    assert np.all(np.abs(c.double().cpu().numpy() - exact) <= 2.0**-20 * norms)
+    return c
+
+
+def _a16(prod, a, b):
+    (M, K), N = a.shape, b.shape[1]
+    ad, bd = a.cuda(), torch.from_numpy(b).cuda()
+    c = torch.empty(M, N, device="cuda", dtype=torch.float32)
+    ct = torch.empty(N, M, device="cuda", dtype=torch.float32)
+    prod.run(prod.a16, BF16 if a.dtype is torch.bfloat16 else F16, M, N, K, ad.data_ptr(), K, F64, bd.data_ptr(), N,
+             c.data_ptr(), N, ct.data_ptr())
+    assert torch.equal(ct.T, c)
+    return c
+
+
+@pytest.mark.parametrize("M,N,K,f64out", [(300, 130, 257, False), (257, 272, 1000, True), (12290, 40, 96, False)])
+def test_fp32_per_row(prod, M, N, K, f64out):
+    rng = np.random.default_rng(M + K)
+    a = _spread(rng, M, K, 0, -40, 0).astype(np.float32)
+    b = _spread(rng, K, N, 1, -20, 20)
+    _check_fp32(_f32x2(prod, a, b, f64out), a.astype(np.float64), b)
 
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
@@ -138,16 +158,19 @@ def test_16bit_per_row(prod, dtype, M, N, K):
     rng = np.random.default_rng(M + K)
     a = torch.from_numpy(_spread(rng, M, K, 0, -10, 0)).to(dtype)
     b = _spread(rng, K, N, 1, -20, 20)
-    ad, bd = a.cuda(), torch.from_numpy(b).cuda()
-    c = torch.empty(M, N, device="cuda", dtype=torch.float32)
-    ct = torch.empty(N, M, device="cuda", dtype=torch.float32)
-    prod.run(prod.a16, BF16 if dtype is torch.bfloat16 else F16, M, N, K, ad.data_ptr(), K, F64, bd.data_ptr(), N,
-             c.data_ptr(), N, ct.data_ptr())
-    vals = a.double().numpy()
-    exact = vals @ b
-    norms = np.linalg.norm(vals, axis=1)[:, None] * np.linalg.norm(b, axis=0)[None, :]
-    assert np.all(np.abs(c.double().cpu().numpy() - exact) <= 2.0**-20 * norms)
-    assert torch.equal(ct.T, c)
+    _check_fp32(_a16(prod, a, b), a.double().numpy(), b)
+
+
+@pytest.mark.parametrize("ea,eb", [(118, -4), (105, 10), (-110, 4), (60, -100), (-60, 100)])
+def test_ends_of_the_range(prod, ea, eb):
+    """FP32 and BF16 data near the ends of FP32's range, products within it."""
+    rng = np.random.default_rng(7)
+    a = rng.standard_normal((300, 128)) * 2.0**ea
+    b = rng.standard_normal((128, 40)) * 2.0**eb
+    a32, b32 = a.astype(np.float32), b.astype(np.float32).astype(np.float64)
+    _check_fp32(_f32x2(prod, a32, b32), a32.astype(np.float64), b32)
+    a16 = torch.from_numpy(a).to(torch.bfloat16)
+    _check_fp32(_a16(prod, a16, b32), a16.double().numpy(), b32)
 
 
 @pytest.mark.parametrize("M,N,K,trans,gram", [
