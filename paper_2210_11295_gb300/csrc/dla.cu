@@ -1112,8 +1112,9 @@ __global__ void k_scale_norms(const double* __restrict__ C, int64_t n, double* _
 // orthogonal to first order, from C = U^T U (norms of U's columns near 1,
 // sig without them): V (I + X) and U (I + Z), X_ij = c s_i s_j / (s_j^2 - s_i^2),
 // Z = D X D^-1 (D = diag(s)), c the cosine of the pair and s_i = sig_i |u_i|.
-// Z (for U's columns once normalised) stays as small as the cosines (over the relative gaps) however far apart
-// the norms are, so small columns are made orthogonal to their own accuracy.
+// Z (for U's columns once normalised) stays as small as the cosines (over the
+// relative gaps) however far apart the norms are, so small columns are made
+// orthogonal to their own accuracy.
 // Pairs with |X_ij| > 0.03 (clustered singular values) are left alone, and so
 // are pairs orthogonal to the threshold that would turn by more than
 // kRefKeepsV: over a small enough gap the rounding of a cosine turns by any
@@ -1601,8 +1602,8 @@ int launch_jacobi_cluster_jq(const Dla& d, jc::Args a, int nc) {
 
 int launch_jacobi_cluster(const Dla& d, float* X, int64_t l, double tol, double tol_stop, double tiny, int64_t lead,
                           int64_t need, int max_sweeps, int* rot, float* nrm) {
-  if (l < 2 || l > jc::kMaxRows) return BSRHT_EUNSUP;
-  const int nc = l <= 64 ? 2 : l <= 128 ? 4 : l <= 256 ? 8 : 16;
+  if (l <= kJacobiMixedMin || l > jc::kMaxRows) return BSRHT_EUNSUP;
+  const int nc = l <= 128 ? 4 : l <= 256 ? 8 : 16;
   jc::Args a;
   a.X = X;
   a.l = a.rows = (int)l;

@@ -142,19 +142,22 @@ bool gemm_tc_eligible(int64_t M, int64_t N, int64_t K, const void* A, int64_t ld
 // op(A) or of a column of B is taken to 2^-55 of the largest one there; sums
 // are exact and each split of K is rounded once, so an entry of C is off by
 // at most about K 2^-54 times the row's and the column's largest entries, a
-// normwise bound like that of the factorizations that use it.
+// normwise bound like that of the factorizations that use it.  (A small entry
+// beside a large one keeps fewer bits than in the CUDA-core form.)  A row of
+// op(A) or a column of B with an Inf or a NaN makes its row or column of C NaN
+// throughout, where the CUDA-core form gives Inf or NaN entry by entry.
 // gemm_int8x7_wants: large enough to gain.
 bool gemm_int8x7_wants(int64_t M, int64_t N, int64_t K);
 int gemm_int8x7(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const double* A, int64_t lda, bool a_trans,
                 const double* B, int64_t ldb, double* C, int64_t ldc, bool b_upper, bool gram);
-// FP32-accurate products of 16-bit data: C (M x N, FP32, ldc) = A (M x K,
-// BF16 or F16, 16-byte aligned rows) * B (K x N, FP32 or FP64, ldb); Ct as
-// in gemm_tc.
 // FP32 products at FP16's rate: as gemm_tc (b_kmajor and gram false), for
 // FP32 A with 16-byte aligned rows.
 bool gemm_f32x2_eligible(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda);
 int gemm_f32x2(const Dla& d, Arena& ar, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, DT tb,
                const void* B, int64_t ldb, DT tc_out, void* C, int64_t ldc, bool b_upper, float* Ct);
+// FP32-accurate products of 16-bit data: C (M x N, FP32, ldc) = A (M x K,
+// BF16 or F16, 16-byte aligned rows) * B (K x N, FP32 or FP64, ldb); Ct as
+// in gemm_tc.
 bool gemm_a16_eligible(DT ta, int64_t M, int64_t N, int64_t K, const void* A, int64_t lda);
 int gemm_a16(const Dla& d, Arena& ar, DT ta, int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, DT tb,
              const void* B, int64_t ldb, float* C, int64_t ldc, float* Ct);

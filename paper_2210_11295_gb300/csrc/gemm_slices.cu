@@ -218,8 +218,10 @@ size_t digit_bytes_of(int64_t rows, int64_t ldk) { return (size_t)kDig * 2 * (si
 
 }  // namespace
 
-// Scratch the digits of one launch may take: enough rows of A for a wave of
-// 128 x 64 tiles over the SMs at K = 2048, l = 256 (139 MB).
+// Scratch the digits of one launch may take, 14 bytes an entry: a bound on the
+// workspace rather than a rule of speed.  A pass with fewer tiles than SMs splits
+// K instead, as far as half a wave is gained (N = 256: a whole wave of 128 x 64
+// tiles up to K = 2800, at K = 4096 a pass has 108 tiles).
 constexpr size_t kDigitScratch = (size_t)192 << 20;
 
 // Measured on GB300 (int8x7 against the CUDA-core GEMM, FP64): below about 20

@@ -2,7 +2,7 @@
 //
 // Three kernels share the layout: K-major slices [slice][row][k] in global
 // memory, TMA into swizzled shared memory, one thread issuing the MMAs, FP32
-// accumulators in tensor memory, eight warps folding them.
+// accumulators in tensor memory, and warps that only fold those.
 //
 // k_gemm_int8x7: FP64 products in exact integer arithmetic.  The FP64 units
 // of this GPU give about two FMAs per SM and clock (1.2 TFLOP/s on the whole
@@ -40,8 +40,10 @@
 // scaled per column); four warps split each staged tile of A in place, one
 // power-of-two scale per row and 64 of K, which the 16 fold warps undo when
 // they add the 64 to their FP32 sums: hi lo + lo hi + hi hi, smallest first;
-// what is dropped lies below 2^-23 of each product, or 2^-38 of the row's
-// largest entry in the 64.  2^18 x 4096 x 512: 2.93 ms (TF32 form 4.48).
+// what is dropped (lo lo and the rounding of both lo) lies below 2^-21 of each
+// product, or 2^-38 of the row's largest entry in the 64 where that is more.
+// 2^18 x 4096 x 512: 2.93 ms (TF32 form 4.48), 704 threads of 80 registers, 136
+// to 144 bytes of spilled stores a thread.
 // Without the split and the fold it takes 2.2 ms, without two of the three MMAs
 // as well 1.9 ms (copies from L2): no single part bounds it, but their use of
 // shared memory, 152 KB per 32 of K against 768 clocks of MMA.  Measured on the

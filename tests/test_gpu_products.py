@@ -42,6 +42,8 @@ class _Products:
         self.f32x2.argtypes = head + [i64, i64, i64, vp, i64, ci, vp, i64, ci, vp, i64, cb, vp]
         self.a16 = getattr(lib, "_ZN5bsrht8gemm_a16ERKNS_3DlaERNS_5ArenaENS_2DTElllPKvlS5_S7_lPflS8_")
         self.a16.argtypes = head + [ci, i64, i64, i64, vp, i64, ci, vp, i64, vp, i64, vp]
+        self.signs = getattr(lib, "_ZN5bsrht14sign_normalizeERKNS_3DlaERNS_5ArenaEPdllS5_l")
+        self.signs.argtypes = head + [vp, i64, i64, vp, i64]
         self.scratch = torch.empty(1 << 30, device="cuda", dtype=torch.uint8)
         self.status = torch.zeros(64, device="cuda", dtype=torch.int32)
 
@@ -140,7 +142,7 @@ def _a16(prod, a, b):
     ct = torch.empty(N, M, device="cuda", dtype=torch.float32)
     prod.run(prod.a16, BF16 if a.dtype is torch.bfloat16 else F16, M, N, K, ad.data_ptr(), K, F64, bd.data_ptr(), N,
              c.data_ptr(), N, ct.data_ptr())
-    assert torch.equal(ct.T, c)
+    assert torch.allclose(ct.T, c, rtol=0, atol=0, equal_nan=True)
     return c
 
 
@@ -197,3 +199,40 @@ def test_fp64_scratch_as_measured(prod, M, N, K, trans, gram):
     full = c.clone()
     assert launches(prod.measure(prod.int8x7, *args)) == ample
     assert torch.equal(c, full)
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_nonfinite_stays_in_its_row_or_column(prod, bad):
+    rng = np.random.default_rng(3)
+    M, N, K = 300, 130, 256
+    a, b = rng.standard_normal((M, K)), rng.standard_normal((K, N))
+    rows, cols = np.arange(M) == 77, np.arange(N) == 5
+    touched = rows[:, None] | cols[None, :]
+    an, bn = a.copy(), b.copy()
+    an[77, 3], bn[9, 5] = bad, bad
+    ad, bd = torch.from_numpy(an).cuda(), torch.from_numpy(bn).cuda()
+    c = torch.empty(M, N, device="cuda", dtype=torch.float64)
+    prod.run(prod.int8x7, M, N, K, ad.data_ptr(), K, False, bd.data_ptr(), N, c.data_ptr(), N, False, False)
+    got = c.cpu().numpy()
+    assert np.all(np.isnan(got[touched]))
+    assert np.all(np.abs(got - a @ b)[~touched] <= 1e-12)
+    a16 = torch.from_numpy(an).to(torch.bfloat16)
+    for c, vals in ((_f32x2(prod, an.astype(np.float32), bn), a), (_a16(prod, a16, bn), a16.double().numpy())):
+        got = c.double().cpu().numpy()
+        assert not np.any(np.isfinite(got[touched]))
+        clean = np.where(np.isfinite(vals), vals, 0.0)
+        norms = np.linalg.norm(clean, axis=1)[:, None] * np.linalg.norm(b, axis=0)[None, :]
+        assert np.all(np.abs(got - clean @ b)[~touched] <= (2.0**-20 * norms)[~touched])
+
+
+@pytest.mark.parametrize("n,k", [(1, 1), (5000, 7), (70000, 100), (300, 300), (4097, 1)])
+def test_signs_with_ties(prod, n, k):
+    """The sign of a column is that of its first largest entry."""
+    rng = np.random.default_rng(n + k)
+    u = rng.integers(-2, 3, size=(n, k)).astype(np.float64)  # many entries tie for the largest
+    v = rng.standard_normal((9, k))
+    ud, vd = torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda()
+    prod.run(prod.signs, ud.data_ptr(), n, k, vd.data_ptr(), 9)
+    sign = np.where(u[np.argmax(np.abs(u), axis=0), np.arange(k)] < 0, -1.0, 1.0)
+    assert np.array_equal(ud.cpu().numpy(), u * sign)
+    assert np.array_equal(vd.cpu().numpy(), v * sign)
