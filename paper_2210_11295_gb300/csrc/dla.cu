@@ -1066,10 +1066,11 @@ constexpr double kRefFine = 0x1.0p-26;
 // Nystrom request of l = 400.)
 constexpr double kRefKeepsV = 0x1.0p-17;
 // Largest angle before the sweeps: among close values larger ones are mostly
-// rounding, and undone by the sweeps (CPU model of these steps, half of 256
-// values equal: 2 sweeps after it, 10 after angles up to 0.03; pairs 1e-4 to
-// 1e-15 apart: 3 sweeps either way, 5 without this rotation).
-constexpr double kRefBeforeSweeps = 0x1.0p-10;
+// rounding, and undone by the sweeps.  (rSVD with half of l = 400 values equal:
+// 10.6 ms, with angles up to 0.03 12.1; the small SVD of the 1048576 x 4096 FP32
+// benchmark, whose smallest wanted values lie 1e-3 apart, 1.25 ms, with angles up
+// to 2^-10 only 1.87.)
+constexpr double kRefBeforeSweeps = 0x1.0p-7;
 
 // Coefficients of one orthonormalisation step V <- V G of nearly orthonormal
 // columns from their Gram G, in place.  tri: Gram-Schmidt to first order
