@@ -20,7 +20,7 @@
 // memory, are folded into two 64-bit integers per entry, and the sum is rounded
 // to FP64 once, at the end.  Bound by shared memory: an MMA of 128 x 64 x 16
 // reads 6 KB (48 clocks against 32 of tensor work), 68 of them and the copies of
-// a stage come to 2.1 us, measured about 3 us a stage of 32 of K.
+// a stage come to 2.1 us, measured 3.2 us a stage of 32 of K (tensor pipe 35 %).
 // 131072 x 2048 x 256: 6.8 ms with the digits' preparation (FP64 units: 110 ms).
 //
 // k_gemm_a16: FP32-accurate products of 16-bit data.  A (BF16 or FP16) is
@@ -29,9 +29,10 @@
 // BF16, 33 in FP16), for FP16 scaled per column to its range.  Three 16-bit MMAs
 // per product; each K block of 64 starts a fresh accumulator, smallest slice
 // first, which the fold adds to FP32 registers, rounding to nearest (the
-// tensor core's own accumulation truncates).  Bound by the copies of B's three
-// slices from L2 (94 KB a block of K at N = 400) and the stores of C, which
-// leaves in whole sectors (262144 x 2000 x 400: 1.57 -> 1.20 ms).
+// tensor core's own accumulation truncates).  Bound by two stages of 112 KB:
+// the copies of a block of K (94 KB at N = 400) and its MMAs mostly take turns
+// (tensor pipe 47 %, L2 22 %).  C leaves in whole sectors (262144 x 2000 x 400:
+// 1.57 -> 1.20 ms).
 //
 // k_gemm_f32x2: FP32 products of FP32 data at twice the TF32 rate.  An FP16
 // pair holds as much of an FP32 value as a TF32 pair (11 + 11 bits) once it is
@@ -45,8 +46,9 @@
 // 2^18 x 4096 x 512: 2.93 ms (TF32 form 4.48), 704 threads of 80 registers, 136
 // to 144 bytes of spilled stores a thread.
 // Without the split and the fold it takes 2.2 ms, without two of the three MMAs
-// as well 1.9 ms (copies from L2): no single part bounds it, but their use of
-// shared memory, 152 KB per 32 of K against 768 clocks of MMA.  Measured on the
+// as well 1.9 ms: no single part bounds it (tensor pipe 48 %, L1 and shared
+// memory 47 %, L2 35 %), but their use of shared memory, 152 KB per 32 of K against
+// 768 clocks of MMA, and what a CTA alone on its SM does not overlap.  Measured on the
 // way: the fold warps splitting too, 3.9 ms; folding every 32 of K, 3.3 ms; two
 // CTAs loading half of B each for both, 2.98 ms (and 1.20 as above for
 // k_gemm_a16): every CTA loads its own.
