@@ -88,3 +88,22 @@ def test_rsvd_core_singular_in_fp32(lib, l, decay):
     ur, sr, vr = orc.rsvd(a, k, l, 16, 3)
     ref = (ur * sr) @ vr.T
     assert np.linalg.norm((u * s) @ v.T - ref) <= 1e-12 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("l,spread", [(80, 1e-4), (160, 1e-6), (256, 0.0), (300, "steep")])
+def test_rsvd_fp32_data(lib, l, spread):
+    """The same cores from FP32 data, whose FP64 polish stops at 16 sqrt(l) 2^-40
+    and whose tall factors are accurate to FP32: 1e-5, V orthonormal to 1e-12, U to
+    1e-4 as for FP32 data elsewhere."""
+    rng = np.random.default_rng(l)
+    sigma = np.exp(-np.arange(l) / 15.0) if spread == "steep" else _spectrum(l, spread, rng)
+    n, m, k = 8192, l + 13, 20 if spread == "steep" else l // 2
+    uu, vv = synth.haar(n, l, rng), synth.haar(m, l, rng)
+    x = torch.from_numpy((uu * sigma) @ vv.T).float()
+    a = x.double().numpy()
+    u, s, v = (t.cpu().numpy() for t in lib.bsrht_rsvd(x.cuda(), k, l, 16, 3))
+    assert _orth_error(v) <= 1e-12
+    assert _orth_error(u) <= 1e-4
+    assert np.max(np.abs(s - sigma[:k])) <= 1e-5 * sigma[0]
+    assert np.linalg.norm(a @ v - u * s) <= 1e-5 * np.linalg.norm(a)
+    assert np.linalg.norm(a.T @ u - v * s) <= 1e-5 * np.linalg.norm(a)
